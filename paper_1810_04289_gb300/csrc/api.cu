@@ -922,37 +922,28 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
 
     // packed factor streams for the TMA-fed apply
     {
-      std::vector<int64_t> Lcnt(R.gnode.size()), Ucnt(R.gnode.size()), Loff(R.np + 1), Uoff(R.np + 1), Lsrc, Usrc,
-          Upiv;
-      std::vector<int32_t> Lcol, Ucol;
-      int64_t maxblk = 1;
-      for (int32_t sd = 0; sd < R.np; ++sd) {
-        const int64_t a = R.sd_row[sd], b = R.sd_row[sd + 1];
-        Loff[sd] = (int64_t)Lsrc.size();
-        for (int64_t q = a; q < b; ++q) {
-          for (int64_t e = R.row_ptr[q]; e < R.diag[q]; ++e) {
-            Lsrc.push_back(e);
-            Lcol.push_back((int32_t)(R.col[e] - a));
-          }
-          Lcnt[q] = R.diag[q] - R.row_ptr[q];
-          maxblk = std::max(maxblk, Lcnt[q]);
-        }
-        Uoff[sd] = (int64_t)Usrc.size();
-        for (int64_t q = b - 1; q >= a; --q) {
-          Usrc.push_back(R.diag[q]);
-          Ucol.push_back((int32_t)(q - a));
-          Upiv.push_back(-1);
-          for (int64_t e = R.diag[q] + 1; e < R.row_ptr[q + 1]; ++e) {
-            Usrc.push_back(e);
-            Ucol.push_back((int32_t)(R.col[e] - a));
-            Upiv.push_back(R.diag[q]);
-          }
-          Ucnt[q] = R.row_ptr[q + 1] - R.diag[q];
-          maxblk = std::max(maxblk, Ucnt[q]);
-        }
-      }
-      Loff[R.np] = (int64_t)Lsrc.size();
-      Uoff[R.np] = (int64_t)Usrc.size();
+      // stage geometry: NST (2) stages of SB blocks. The target is ceil(np / 152)
+      // CTAs per SM, at most 8 (all subdomains resident at once up to 1,216), and
+      // the ring gets what the shared memory per CTA leaves after the vector; the
+      // stage_blocks and stages options override the choice
+      const int vsz = cp->mixed ? 4 : 8, stride = 56;  // packed block: 7 rows of 8 values
+      int nst = o.stages > 0 ? o.stages : 2;
+      const int64_t W = (int64_t)1 << R.max_depth;  // warps (rings) per CTA
+      const int64_t per_sm = std::min<int64_t>(8, (R.np + 151) / 152);
+      const int64_t fixed = 128 * ((W * 64 + 127) / 128) + 8 * R.max_rows * vsz + 4 * R.max_rows + 16 + 1024;
+      // (the budget never exceeds the 200 KB the streamed apply may use)
+      const int64_t budget = std::min<int64_t>((int64_t)(227 * 1024) / per_sm, (int64_t)(200 * 1024));
+      int64_t SB = (budget - fixed) / (W * nst * stride * vsz);
+      SB = std::max<int64_t>(W > 1 ? 8 : 16, std::min<int64_t>(SB, cp->mixed ? 128 : 64));
+      if (o.stage_blocks > 0) SB = o.stage_blocks;
+      // the chain apply's two stages get what the vector leaves of the same budget. Mixed: it forms a
+      // row's sum in the pieces the ring's stages cut it into, so that both kernels give the same bits;
+      // in FP64 whole rows
+      const int64_t most = cp->mixed ? 16 : 8;
+      int64_t CB = (budget - 2048 - 8 * R.max_rows * vsz) / (2 * stride * vsz);
+      CB = std::max<int64_t>(most, std::min<int64_t>(CB, 64));
+      const StreamPlan S = build_stream(R, cp->mixed ? SB : (int64_t)1 << 40, most, CB);
+      const std::vector<int64_t>&Lcnt = S.L_cnt, &Ucnt = S.U_cnt;
       // per nested-dissection item: its first / end block in the subdomain's L
       // stream (rows ascending) and U stream (rows descending)
       std::vector<int32_t> iblk(4 * R.item_row.size());
@@ -986,45 +977,32 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       rs.sd_row = rd.sd_row;
       rs.gnode = rd.gnode;
       rs.owned = rd.owned;
-      rs.L_cnt = cp->upload(Lcnt);
-      rs.U_cnt = cp->upload(Ucnt);
-      rs.L_off = cp->upload(Loff);
-      rs.U_off = cp->upload(Uoff);
-      rs.nL = (int64_t)Lsrc.size();
-      rs.nU = (int64_t)Usrc.size();
-      rs.Lsrc = cp->upload(Lsrc);
-      rs.Lcol = cp->upload(Lcol);
-      rs.Usrc = cp->upload(Usrc);
-      rs.Ucol = cp->upload(Ucol);
-      rs.Upiv = cp->upload(Upiv);
-      // stage geometry: NST (2) stages of SB blocks. The target is ceil(np / 152)
-      // CTAs per SM, at most 8 (all subdomains resident at once up to 1,216), and
-      // the ring gets what the shared memory per CTA leaves after the vector; the
-      // stage_blocks and stages options override the choice
-      const int vsz = cp->mixed ? 4 : 8, stride = 56;  // packed block: 7 rows of 8 values
-      int nst = o.stages > 0 ? o.stages : 2;
-      const int64_t W = (int64_t)1 << R.max_depth;  // warps (rings) per CTA
-      const int64_t per_sm = std::min<int64_t>(8, (R.np + 151) / 152);
-      const int64_t fixed = 128 * ((W * 64 + 127) / 128) + 8 * R.max_rows * vsz + 4 * R.max_rows + 16 + 1024;
-      // (the budget never exceeds the 200 KB the streamed apply may use)
-      const int64_t budget = std::min<int64_t>((int64_t)(227 * 1024) / per_sm, (int64_t)(200 * 1024));
-      int64_t SB = (budget - fixed) / (W * nst * stride * vsz);
-      SB = std::max<int64_t>(W > 1 ? 8 : 16, std::min<int64_t>(SB, cp->mixed ? 128 : 64));
-      if (o.stage_blocks > 0) SB = o.stage_blocks;
+      rs.L_cnt = cp->upload(S.L_cnt);
+      rs.U_cnt = cp->upload(S.U_cnt);
+      rs.L_off = cp->upload(S.L_off);
+      rs.U_off = cp->upload(S.U_off);
+      rs.nblk = (int64_t)S.src.size();
+      rs.src = cp->upload(S.src);
+      rs.col = cp->upload(S.col);
+      rs.piv = cp->upload(S.piv);
+      rs.code = cp->upload(S.code);
+      rs.code_off = cp->upload(S.code_off);
+      rs.stage = cp->upload(S.stage);
+      rs.stage_off = cp->upload(S.stage_off);
       rs.nst = nst;
       rs.stall = o.fault_test == 1 ? 1 : 0;
       rs.stage_blocks = (int32_t)SB;
+      rs.chain_blocks = (int32_t)CB;
       rs.max_rows = R.max_rows;
       const size_t sm = cp->mixed ? ras_stream_smem<float>(rs) : ras_stream_smem<double>(rs);
       // (the apply keeps each row's block counts as 16-bit values in shared memory)
-      const bool fits = sm <= 200 * 1024 && maxblk <= 65535;
+      const bool fits = sm <= 200 * 1024 && S.max_row_blocks <= 65535;
       if (o.apply_mode == 1 && !fits)
         throw StatusError{FSI_ERR_ARG, "apply_mode 1: the streamed apply's shared memory does not fit"};
       cp->use_stream = o.apply_mode == 2 ? false : fits;
       if (cp->use_stream) {
         CK(cp->mixed ? ras_stream_init<float>(rs) : ras_stream_init<double>(rs));
-        rs.Lpack = cp->dalloc<char>((int64_t)(stride * vs) * std::max<int64_t>(rs.nL, 1));
-        rs.Upack = cp->dalloc<char>((int64_t)(stride * vs) * std::max<int64_t>(rs.nU, 1));
+        rs.pack = cp->dalloc<char>((int64_t)(stride * vs) * std::max<int64_t>(rs.nblk, 1));
       }
     }
     CK(cudaStreamSynchronize(cp->s));

@@ -111,16 +111,18 @@ struct RasStreamDev {
   const int64_t* L_cnt;   // [rows] L blocks of each row
   const int64_t* U_cnt;   // [rows] 1 (inverted pivot) + U blocks of each row
   const int64_t* L_off;   // [np+1] first packed L block of each subdomain
-  const int64_t* U_off;   // [np+1] first packed U block of each subdomain
-  void* Lpack;
-  void* Upack;
-  int64_t nL, nU;
-  const int64_t* Lsrc;    // [nL] factor block copied into each packed L block
-  const int32_t* Lcol;    // [nL] subdomain-relative column row
-  const int64_t* Usrc;
-  const int32_t* Ucol;
-  const int64_t* Upiv;    // [nU] factor block of the row's inverted pivot, -1 for the pivot itself
+  const int64_t* U_off;   // [np+1] first packed U block of each subdomain (its U part follows its L part)
+  void* pack;
+  int64_t nblk;           // packed blocks
+  const int64_t* src;     // [nblk] factor block copied into each packed block
+  const int32_t* col;     // [nblk] subdomain-relative column row
+  const int64_t* piv;     // [nblk] factor block of the row's inverted pivot; -1: copied as it is
+  const uint32_t* code;   // entry codes of the chain apply (setup.h, StreamPlan)
+  const int64_t* code_off;// [np+1] first code word of each subdomain
+  const uint8_t* stage;   // blocks of each stage of the chain apply
+  const int64_t* stage_off;// [np+1] first stage of each subdomain
   int32_t stage_blocks;   // blocks per ring stage (one bulk copy; rows may straddle stages)
+  int32_t chain_blocks;   // chain apply: blocks per ring stage
   int64_t max_rows;       // rows of the largest subdomain
   int32_t nst;            // ring stages in flight per warp (2..8)
   int32_t stall;          // tests only: the producer issues nothing (bounded waits run out)
@@ -138,7 +140,8 @@ void launch_pack_factors(const RasStreamDev& r, const TF* fac, cudaStream_t s);
 // once per context: allow the apply kernel its dynamic shared memory
 template <class TF>
 cudaError_t ras_stream_init(const RasStreamDev& r);
-// z = B^{-1} r; z32 (optional) receives an FP32 copy; guard as for the SpMV
+// z = B^{-1} r; z32 (optional) receives an FP32 copy; guard as for the SpMV. Takes
+// the chain kernel, or the ring kernel for dissected subdomains
 template <class TF>
 cudaError_t launch_ras_apply_stream(const RasStreamDev& r, const double* rin, double* z, float* z32, int32_t* err,
                                     const int* guard, cudaStream_t s);

@@ -1,26 +1,22 @@
-// Streamed RAS apply (Sec. 3, Eq. 16) for GB300: one CTA per subdomain, two
-// warps. Warp 1 (one elected lane) is a producer that streams the packed factor
-// with 1-D bulk copies (cp.async.bulk, the TMA engine) into a ring of
-// shared-memory stages guarded by mbarriers; warp 0 is the consumer that walks
-// the rows in order (forward solve with the unit lower factor, then backward
-// solve with the upper factor and inverted pivots) on the subdomain vector held
-// in shared memory. The dependency chain of an ILU solve on an RCM-ordered
-// subdomain is nearly the row count, so the rows are processed one after the
-// other by 28 lanes (4 blocks at a time x 7 components) while the factor bytes
-// for the rows ahead are already in flight.
+// Streamed RAS apply (Sec. 3, Eq. 16) for GB300: one CTA per subdomain; the packed
+// factor streams through shared memory (1-D bulk copies, cp.async.bulk, guarded by
+// mbarriers) past the subdomain vector, which stays there. The dependency chain of
+// an ILU solve on an RCM-ordered subdomain is nearly the row count, so the rows are
+// worked off one after the other (forward with the unit lower factor, then backward
+// with the upper factor and inverted pivots) by one warp: lane 8 j + c takes row c
+// of the blocks j, j + 4, ... of a row. Two kernels:
+//   k_ras_apply_chain: subdomains in one piece (every ordering but the dissected);
+//   k_ras_apply_stream: nested-dissection subdomains, one warp and ring per part.
 //
-// Packed layout (built by k_pack_factors after each factorisation):
-//   L stream: for every row in increasing order, its L blocks;
-//   U stream: for every row in decreasing order, its inverted pivot D_q^{-1}, then
-//             its U blocks premultiplied and negated, -D_q^{-1} U_qj.
-// Each packed block holds its 7 rows as 8-wide, 16-byte aligned rows (56 values):
-// the row's 7 entries, then one slot; row 0's slot holds the subdomain-relative
-// column row (as int bits). The subdomain vector in shared memory is 8 wide too,
-// so each 7-term product is four 16-byte loads (FP32) instead of fourteen.
-// Stages are fixed slices of stage_blocks blocks of a subdomain's L stream, then
-// of its U stream; a row may straddle stages (its partial sums carry over), so
-// the stage size is independent of the row length and can be chosen for
-// occupancy.
+// Packed layout (built by k_pack_factors after each factorisation), per subdomain:
+//   L part: for every row in increasing order, its L blocks;
+//   U part: for every row in decreasing order, its inverted pivot D_q^{-1}, then
+//           its U blocks premultiplied and negated, -D_q^{-1} U_qj.
+// Each packed block holds its 7 rows as 8-wide rows (the 7 entries, then the
+// block's column), cut into 16-byte pieces: the first pieces of the 7 rows, then
+// the second pieces, and so on, so that the 7 lanes of a block read consecutive 16
+// bytes (8-wide rows in one piece put lanes c and c + 4 on the same banks). The
+// subdomain vector in shared memory is 8 wide too.
 //
 // Every wait on an mbarrier is bounded; on timeout the kernel records
 // FSI_ERR_TIMEOUT-style status in *err, drains (bounded) and returns.
@@ -29,6 +25,7 @@
 #include <cstdint>
 
 #include "kernels.cuh"
+#include "setup.h"
 
 namespace fsi {
 
@@ -77,20 +74,20 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 
 template <class TF> struct Pack;
-// packed block: 7 rows of 8 values (the 7 entries of the row, then one slot),
-// 16-byte aligned rows; the slot of row 0 holds the column (as int bits), the
-// other slots are zero
+// packed block: 7 rows of 8 values in 16-byte pieces (see above)
 template <class TF> struct Pack { static constexpr int stride = 56; };
 
+// the block's column (a row of the subdomain)
 template <class TF>
 __device__ __forceinline__ int blk_col(const TF* blk) {
-  return *reinterpret_cast<const int*>(blk + 7);
+  constexpr int V = 16 / sizeof(TF);  // row 0's last value, in its last piece
+  return *reinterpret_cast<const int*>(blk + (8 / V - 1) * 7 * V + V - 1);
 }
 
 // the 7-term product of row c of a packed block with the node vector x (8 wide):
 // 16-byte loads of the row and of x
 __device__ __forceinline__ float row7(const float* a, const float* x) {
-  const float4 a0 = *reinterpret_cast<const float4*>(a), a1 = *reinterpret_cast<const float4*>(a + 4);
+  const float4 a0 = *reinterpret_cast<const float4*>(a), a1 = *reinterpret_cast<const float4*>(a + 28);
   const float4 x0 = *reinterpret_cast<const float4*>(x), x1 = *reinterpret_cast<const float4*>(x + 4);
   const float p01 = a0.x * x0.x + a0.y * x0.y;
   const float p23 = a0.z * x0.z + a0.w * x0.w;
@@ -98,8 +95,8 @@ __device__ __forceinline__ float row7(const float* a, const float* x) {
   return (p01 + p23) + (p45 + a1.z * x1.z);
 }
 __device__ __forceinline__ double row7(const double* a, const double* x) {
-  const double2 a0 = *reinterpret_cast<const double2*>(a), a1 = *reinterpret_cast<const double2*>(a + 2);
-  const double2 a2 = *reinterpret_cast<const double2*>(a + 4), a3 = *reinterpret_cast<const double2*>(a + 6);
+  const double2 a0 = *reinterpret_cast<const double2*>(a), a1 = *reinterpret_cast<const double2*>(a + 14);
+  const double2 a2 = *reinterpret_cast<const double2*>(a + 28), a3 = *reinterpret_cast<const double2*>(a + 42);
   const double2 x0 = *reinterpret_cast<const double2*>(x), x1 = *reinterpret_cast<const double2*>(x + 2);
   const double2 x2 = *reinterpret_cast<const double2*>(x + 4), x3 = *reinterpret_cast<const double2*>(x + 6);
   const double p01 = a0.x * x0.x + a0.y * x0.y;
@@ -129,7 +126,7 @@ __device__ __forceinline__ TF row_dot(const TF* stg, int nb, const TF* w, int j,
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        if (cols[i] >= 0) acc += row7(stg + (b + 4 * i) * STR + 8 * c, w + 8 * cols[i]);
+        if (cols[i] >= 0) acc += row7(stg + (b + 4 * i) * STR + (16 / (int)sizeof(TF)) * c, w + 8 * cols[i]);
       }
     }
   }
@@ -197,7 +194,7 @@ __device__ __forceinline__ void feed_issue(WarpFeed& f, const int32_t* ib, const
 // solve (leaves, then the separators level by level up to the root's) every item
 // of the phase is solved by its own warp, the items of a phase being independent
 // (no edge and no fill between them); the backward solve runs the phases in
-// reverse. Subdomains in the other orderings are one item (depth 0): one warp.
+// reverse. (Subdomains of a few nodes are one item, depth 0: one warp.)
 // Each warp is its own producer: lane 0 streams the packed factor blocks of the
 // warp's items through a ring of NST stages of SB blocks (cp.async.bulk with
 // mbarrier completion); the warp solves the rows of the current stage (rows may
@@ -226,8 +223,8 @@ __global__ void __launch_bounds__(256) k_ras_apply_stream(RasStreamDev R, const 
   const int D = R.sd_depth[s];
   const int32_t* ib = R.item_blk + 4 * R.sd_item[s];        // per item: L begin, L end, U begin, U end
   const int64_t* irow = R.item_row + R.sd_item[s];          // per item: end row
-  const TF* Lpack = reinterpret_cast<const TF*>(R.Lpack) + (size_t)R.L_off[s] * STR;
-  const TF* Upack = reinterpret_cast<const TF*>(R.Upack) + (size_t)R.U_off[s] * STR;
+  const TF* Lpack = reinterpret_cast<const TF*>(R.pack) + (size_t)R.L_off[s] * STR;
+  const TF* Upack = reinterpret_cast<const TF*>(R.pack) + (size_t)R.U_off[s] * STR;
 
   if (lane == 0)
     for (int i = 0; i < NST; ++i) mbar_init(&full[i], 1);
@@ -388,45 +385,252 @@ __global__ void __launch_bounds__(256) k_ras_apply_stream(RasStreamDev R, const 
   }
 }
 
-// copy the factor blocks into the packed streams (7 rows of 8: the row's 7
-// entries, then the column index in row 0's last slot, zeros in the others); a
-// U block with a pivot (Upiv >= 0) is stored as -D_q^{-1} U_qj, the row's
-// inverted pivot itself as it is
+__device__ __forceinline__ int row_col(const float (&v)[8]) { return __float_as_int(v[7]); }
+__device__ __forceinline__ int row_col(const double (&v)[8]) { return __double2loint(v[7]); }
+
+__device__ __forceinline__ void load16(float* v, const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+}
+__device__ __forceinline__ void load16(double* v, const double* p) {
+  const double2 t = *reinterpret_cast<const double2*>(p);
+  v[0] = t.x, v[1] = t.y;
+}
+
+// acc + (row . x): FP32 in row7's order, so that the chain and the ring kernel give the same bits
+__device__ __forceinline__ float row_fma(const float (&a)[8], const float (&x)[8], float acc) {
+  const float p01 = a[0] * x[0] + a[1] * x[1];
+  const float p23 = a[2] * x[2] + a[3] * x[3];
+  const float p45 = a[4] * x[4] + a[5] * x[5];
+  return acc + ((p01 + p23) + (p45 + a[6] * x[6]));
+}
+__device__ __forceinline__ double row_fma(const double (&a)[8], const double (&x)[8], double acc) {
+#pragma unroll
+  for (int e = 0; e < 7; ++e) acc = fma(a[e], x[e], acc);
+  return acc;
+}
+
+// Chain apply: one warp per subdomain, the host's entry codes (setup.h, StreamPlan)
+// in place of row counts and ring arithmetic. What bounds it is the latency of the
+// row chain: with 1,088 subdomains an SM holds 7 warps, and a row costs its
+// instructions times 5 to 6 cycles each. So an entry (up to 16 blocks of a row,
+// FP64 8) is straight-line code: all its vector loads together, then its products;
+// the next entry's rows are read into registers during this entry's reduction;
+// entries never straddle a stage, so their rows lie at fixed offsets; columns come
+// with the rows, not by a load of their own. Two stages of whole entries, refilled
+// by the warp's lane 0.
+// Measured against the ring kernel on one-piece subdomains (same bits in mixed
+// precision): 174k-node tree, ILU(2), 1,088 subdomains, mixed 757 -> 526 us (2.75 GB:
+// 5.2 TB/s); 46,657-node tube, ILU(1), 512 subdomains, FP64 1,243 -> 870 us (the FP64
+// pipe: one warp alone issues an FP64 instruction every 64 cycles, and a 4-block
+// product takes 7 fused instructions where the tree sum took 10).
 template <class TF>
-__global__ void k_pack_factors(int64_t nL, const int64_t* __restrict__ Lsrc, const int32_t* __restrict__ Lcol,
-                               int64_t nU, const int64_t* __restrict__ Usrc, const int32_t* __restrict__ Ucol,
-                               const int64_t* __restrict__ Upiv, const TF* __restrict__ fac, TF* __restrict__ Lpack,
-                               TF* __restrict__ Upack) {
+__global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const double* __restrict__ rin,
+                                                        double* __restrict__ z, float* __restrict__ z32,
+                                                        int32_t* err, const int* __restrict__ guard) {
+  if (guard && *guard == 0) return;
   constexpr int STR = Pack<TF>::stride;
-  const int64_t total = (nL + nU) * STR;
+  constexpr int V = 16 / sizeof(TF), NV = 8 / V;  // values per 16-byte piece, pieces per block row
+  constexpr int G = sizeof(TF) == 4 ? 4 : 2;      // groups of 4 blocks per entry
+  constexpr uint32_t BLK = STR * sizeof(TF);
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);  // [2]
+  unsigned char* ring = smem + 128;
+  const uint32_t cap = R.chain_blocks * BLK;  // bytes of one stage's slot
+  TF* w = reinterpret_cast<TF*>(ring + 2 * cap);
+  const int lane = threadIdx.x, s = blockIdx.x;
+  const int c = lane & 7;
+  const int j = c < 7 ? lane >> 3 : 64;  // block of a group this lane works on (c = 7: none)
+  const int64_t r0 = R.sd_row[s];
+  const int m = (int)(R.sd_row[s + 1] - r0);
+  const uint32_t* cw = R.code + R.code_off[s];
+  const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
+  const TF* src = reinterpret_cast<const TF*>(R.pack) + (size_t)R.L_off[s] * STR;
+  const uint8_t* sz = R.stage + R.stage_off[s];
+  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);  // stages not yet asked for
+  int nsz = left > 0 ? sz[0] : 0;                                       // blocks of the next one
+  uint64_t win = cw[0] | (uint64_t)cw[1] << 32;  // entry codes ahead
+  uint32_t ahead = cw[2];
+
+  // lane 0: ask for the next stage
+  auto feed = [&](int slot) {
+    if (lane == 0 && left > 0) {
+      mbar_arrive_expect_tx(&full[slot], nsz * BLK);
+      bulk_g2s(ring + slot * cap, src, nsz * BLK, &full[slot]);
+      src += (size_t)nsz * STR;
+      ++sz;
+      if (--left > 0) nsz = *sz;
+    }
+  };
+  if (lane == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  feed(0);
+  feed(1);
+
+  // restriction R_i^delta r into shared memory
+#pragma unroll 4
+  for (int q = lane; q < m; q += 32) {
+    const double* sr = rin + 7 * (int64_t)R.gnode[r0 + q];
+    double v[7];
+#pragma unroll
+    for (int e = 0; e < 7; ++e) v[e] = sr[e];
+#pragma unroll
+    for (int e = 0; e < 7; ++e) w[8 * q + e] = (TF)v[e];
+    w[8 * q + 7] = TF(0);
+  }
+  __syncwarp();
+
+  int slot = 0, phase = 0;  // stage being worked off and its barrier's phase
+  const unsigned char* at = ring + 16 * c + (lane >> 3) * BLK;  // this lane's row of the next entry's first group
+  bool ok = true;
+  // rows of an entry's blocks into registers; what lies behind its blocks is read too and not used
+  auto fetch = [&](TF (&A)[G][8], uint32_t code) {
+    auto rows = [&](int g) {
+#pragma unroll
+      for (int e = 0; e < NV; ++e) load16(&A[g][V * e], reinterpret_cast<const TF*>(at + g * 4 * BLK + 112 * e));
+    };
+#pragma unroll
+    for (int g = 0; g < G / 2; ++g) rows(g);
+    if (code & (2 * G)) {
+#pragma unroll
+      for (int g = G / 2; g < G; ++g) rows(g);
+    }
+    at += ((code & 15) + 1) * BLK;
+  };
+  auto xrow = [&](TF (&x)[8], const TF (&A)[8]) {
+    const TF* xp = w + 8 * min((uint32_t)row_col(A), (uint32_t)m - 1);
+#pragma unroll
+    for (int e = 0; e < NV; ++e) load16(&x[V * e], xp + V * e);
+  };
+
+  int q = 0, dq = 1;
+  TF acc = TF(0), tot = TF(-0.0);
+  TF A0[G][8], A1[G][8];
+  // work off the entry whose rows are in A, fetch the next one's into N
+  auto step = [&](TF (&A)[G][8], TF (&N)[G][8], uint32_t code, uint32_t ncode) {
+    if (code < ENTRY_NONE) {
+      const int nb = (int)(code & 15) + 1 - j;  // this lane: blocks 0, 4, 8, .. below nb
+      const TF old = w[8 * q + c];
+      TF x[G][8];
+#pragma unroll
+      for (int g = 0; g < G / 2; ++g) xrow(x[g], A[g]);
+      if (code & (2 * G)) {
+#pragma unroll
+        for (int g = G / 2; g < G; ++g) xrow(x[g], A[g]);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const TF t = row_fma(A[g], x[g], acc);
+          if (4 * g < nb) acc = t;
+        }
+      } else {
+#pragma unroll
+        for (int g = 0; g < G / 2; ++g) {
+          const TF t = row_fma(A[g], x[g], acc);
+          if (4 * g < nb) acc = t;
+        }
+      }
+      if (code & ENTRY_STAGE) {
+        // every lane has read the stage: its slot takes the next but one
+        __syncwarp();
+        feed(slot);
+        phase ^= slot;
+        slot ^= 1;
+        at = ring + slot * cap + 16 * c + (lane >> 3) * BLK;
+        ok = ok && mbar_wait(&full[slot], (uint32_t)phase);
+      }
+      if (ncode < ENTRY_NONE) fetch(N, ncode);
+      if (code & ENTRY_PIECE) {
+        TF r = acc + __shfl_xor_sync(0xffffffffu, acc, 16);
+        r += __shfl_xor_sync(0xffffffffu, r, 8);
+        acc = TF(0);
+        if (sizeof(TF) == 4) tot += r;
+        else tot = r;
+        if (code & ENTRY_ROW) {
+          if (lane < 7) w[8 * q + lane] = dq > 0 ? old - tot : tot;
+          __syncwarp();
+          tot = TF(-0.0);
+          q += dq;
+        }
+      }
+    } else {
+      if (code == ENTRY_EMPTY) {
+        q += dq;
+      } else if (code == ENTRY_BACKWARD) {
+        q = m - 1;
+        dq = -1;
+      }
+      if (ncode < ENTRY_NONE) fetch(N, ncode);
+    }
+  };
+  ok = mbar_wait(&full[0], 0u);
+  if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
+  for (int it = 0; it < 2 * nw && ok; ++it) {
+    const uint32_t w3 = (uint32_t)win;
+    step(A0, A1, w3 & 255, (w3 >> 8) & 255);
+    step(A1, A0, (w3 >> 8) & 255, (w3 >> 16) & 255);
+    win >>= 16;
+    if (it & 1) {
+      win |= (uint64_t)ahead << 32;
+      ahead = cw[min((it >> 1) + 3, nw + 1)];
+    }
+  }
+  if (!ok) {
+    // a wait gave up: record it and let the copy still in flight in the other slot land (bounded)
+    if (lane == 0) atomicExch(err, 2);
+    mbar_wait(&full[slot ^ 1], (uint32_t)(phase ^ slot));
+  }
+
+  // restricted prolongation (R_i^0)^T: owned rows only
+#pragma unroll 4
+  for (int q = lane; q < m; q += 32) {
+    if (R.owned[r0 + q]) {
+      const int64_t g7 = 7 * (int64_t)R.gnode[r0 + q];
+#pragma unroll
+      for (int e = 0; e < 7; ++e) z[g7 + e] = (double)w[8 * q + e];
+      if (z32) {
+#pragma unroll
+        for (int e = 0; e < 7; ++e) z32[g7 + e] = (float)w[8 * q + e];
+      }
+    }
+  }
+}
+
+// copy the factor blocks into the packed stream (7 rows of 8: the row's 7
+// entries, then the block's column); a U block with a pivot (piv >= 0) is stored as -D_q^{-1} U_qj, the
+// row's inverted pivot and the L blocks as they are
+template <class TF>
+__global__ void k_pack_factors(int64_t nblk, const int64_t* __restrict__ src, const int32_t* __restrict__ col,
+                               const int64_t* __restrict__ pivs, const TF* __restrict__ fac, TF* __restrict__ pack) {
+  constexpr int STR = Pack<TF>::stride;
+  const int64_t total = nblk * STR;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = idx / STR;
     const int e = (int)(idx - STR * b);
-    const int r = e >> 3, k = e & 7;
-    const bool isL = b < nL;
-    const int64_t bb = isL ? b : b - nL;
-    const int64_t src = isL ? Lsrc[bb] : Usrc[bb];
-    TF* dst = (isL ? Lpack : Upack) + bb * STR;
+    constexpr int V = 16 / sizeof(TF);
+    const int r = (e % (7 * V)) / V, k = (e / (7 * V)) * V + e % V;
+    const int64_t sb = src[b];
     if (k < 7) {
-      const int64_t piv = isL ? -1 : Upiv[bb];
+      const int64_t piv = pivs[b];
       if (piv < 0) {
-        dst[e] = fac[49 * src + 7 * r + k];
+        pack[idx] = fac[49 * sb + 7 * r + k];
       } else {
         // -(D_q^{-1} U_qj)[r][k]
         const TF* Dq = fac + 49 * piv + 7 * r;
-        const TF* U = fac + 49 * src + k;
+        const TF* U = fac + 49 * sb + k;
         TF v = TF(0);
 #pragma unroll
         for (int mm = 0; mm < 7; ++mm) v += Dq[mm] * U[7 * mm];
-        dst[e] = -v;
+        pack[idx] = -v;
       }
-    } else if (r == 0) {
-      TF v = TF(0);
-      *reinterpret_cast<int*>(&v) = isL ? Lcol[bb] : Ucol[bb];
-      dst[e] = v;
     } else {
-      dst[e] = TF(0);
+      TF v = TF(0);
+      *reinterpret_cast<int*>(&v) = col[b];
+      pack[idx] = v;
     }
   }
 }
@@ -442,27 +646,40 @@ size_t ras_stream_smem(const RasStreamDev& r) {
 
 template <class TF>
 void launch_pack_factors(const RasStreamDev& r, const TF* fac, cudaStream_t s) {
-  const int64_t total = (r.nL + r.nU) * Pack<TF>::stride;
+  const int64_t total = r.nblk * Pack<TF>::stride;
   int64_t g = (total + 255) / 256;
   if (g > 152 * 64) g = 152 * 64;
-  k_pack_factors<TF><<<(int)g, 256, 0, s>>>(r.nL, r.Lsrc, r.Lcol, r.nU, r.Usrc, r.Ucol, r.Upiv, fac,
-                                            (TF*)r.Lpack, (TF*)r.Upack);
+  k_pack_factors<TF><<<(int)g, 256, 0, s>>>(r.nblk, r.src, r.col, r.piv, fac, (TF*)r.pack);
+}
+
+// the ring kernel runs dissected subdomains
+static bool takes_ring(const RasStreamDev& r) { return r.max_depth > 0; }
+
+template <class TF>
+size_t chain_smem(const RasStreamDev& r) {
+  // (an entry's last rows are read up to 15 (FP64: 7) blocks beyond its own)
+  const size_t over = (sizeof(TF) == 4 ? 15 : 7) * Pack<TF>::stride, vec = (size_t)8 * r.max_rows;
+  return 128 + ((size_t)2 * r.chain_blocks * Pack<TF>::stride + (vec > over ? vec : over)) * sizeof(TF);
 }
 
 template <class TF>
 cudaError_t ras_stream_init(const RasStreamDev& r) {
-  // all of the unified L1/shared storage as shared memory: several CTAs per SM
-  cudaError_t e = cudaFuncSetAttribute(k_ras_apply_stream<TF>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  const void* k = takes_ring(r) ? (const void*)k_ras_apply_stream<TF> : (const void*)k_ras_apply_chain<TF>;
+  // all of the unified L1/shared storage as shared memory: several CTAs per SM;
+  // the limit is the kernel's, not the context's: contexts of different sizes share it
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_ras_apply_stream<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)ras_stream_smem<TF>(r));
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 template <class TF>
 cudaError_t launch_ras_apply_stream(const RasStreamDev& r, const double* rin, double* z, float* z32, int32_t* err,
                                     const int* guard, cudaStream_t s) {
-  k_ras_apply_stream<TF><<<r.np, 32 << r.max_depth, ras_stream_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
+  if (takes_ring(r))
+    k_ras_apply_stream<TF><<<r.np, 32 << r.max_depth, ras_stream_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
+  else
+    k_ras_apply_chain<TF><<<r.np, 32, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   return cudaGetLastError();
 }
 

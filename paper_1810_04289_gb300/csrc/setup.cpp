@@ -527,4 +527,100 @@ RasPlan build_ras(const BsrPattern& P, const double* X, int64_t n, const int32_t
   return R;
 }
 
+StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage) {
+  StreamPlan S;
+  const int32_t np = R.np;
+  const int64_t rows = (int64_t)R.gnode.size();
+  S.L_cnt.resize(rows);
+  S.U_cnt.resize(rows);
+  S.L_off.assign(np + 1, 0);
+  S.U_off.assign(np + 1, 0);
+  S.code_off.assign(np + 1, 0);
+  S.stage_off.assign(np + 1, 0);
+  std::vector<std::vector<uint32_t>> words(np);
+  std::vector<std::vector<uint8_t>> stages(np);
+  int64_t at = 0;
+  for (int32_t s = 0; s < np; ++s) {
+    int64_t nL = 0, nB = 0;
+    for (int64_t q = R.sd_row[s]; q < R.sd_row[s + 1]; ++q) {
+      S.L_cnt[q] = R.diag[q] - R.row_ptr[q];
+      S.U_cnt[q] = R.row_ptr[q + 1] - R.diag[q];
+      S.max_row_blocks = std::max(S.max_row_blocks, std::max(S.L_cnt[q], S.U_cnt[q]));
+      nL += S.L_cnt[q];
+      nB += S.L_cnt[q] + S.U_cnt[q];
+    }
+    S.L_off[s] = at;
+    S.U_off[s] = at + nL;
+    at += nB;
+  }
+  S.L_off[np] = S.U_off[np] = at;
+  S.src.resize(at);
+  S.col.resize(at);
+  S.piv.resize(at);
+#pragma omp parallel for schedule(dynamic, 4)
+  for (int32_t s = 0; s < np; ++s) {
+    const int64_t a = R.sd_row[s], b = R.sd_row[s + 1];
+    int64_t k = S.L_off[s];
+    auto put = [&](int64_t e, int64_t piv) {
+      S.src[k] = e;
+      S.col[k] = (int32_t)(R.col[e] - a);
+      S.piv[k++] = piv;
+    };
+    std::vector<uint32_t>& W = words[s];
+    std::vector<uint8_t>& C = stages[s];
+    int64_t n = 0;          // entries so far
+    int64_t last = -1;      // the last one with blocks
+    auto code = [&](uint32_t v) {
+      if (n % 4 == 0) W.push_back(0);
+      W.back() |= v << (8 * (n % 4));
+      if (v < ENTRY_NONE) {
+        const int64_t nb = (v & 15) + 1;
+        if (C.empty() || C.back() + nb > stage) {
+          if (last >= 0) W[last / 4] |= ENTRY_STAGE << (8 * (last % 4));
+          C.push_back(0);
+        }
+        C.back() = (uint8_t)(C.back() + nb);
+        last = n;
+      }
+      ++n;
+    };
+    int64_t pos = 0;  // blocks of this part so far
+    auto row = [&](int64_t nb) {
+      while (nb > 0) {
+        const int64_t piece = std::min(nb, cut - pos % cut);
+        nb -= piece;
+        pos += piece;
+        for (int64_t r = piece; r > 0; r -= most)
+          code((uint32_t)(std::min(r, most) - 1) | (r > most ? 0u : (nb > 0 ? ENTRY_PIECE : ENTRY_PIECE | ENTRY_ROW)));
+      }
+    };
+    for (int64_t q = a; q < b; ++q) {
+      for (int64_t e = R.row_ptr[q]; e < R.diag[q]; ++e) put(e, -1);
+      if (S.L_cnt[q] > 0) row(S.L_cnt[q]);
+      else code(ENTRY_EMPTY);
+    }
+    code(ENTRY_BACKWARD);
+    pos = 0;
+    for (int64_t q = b - 1; q >= a; --q) {
+      put(R.diag[q], -1);
+      for (int64_t e = R.diag[q] + 1; e < R.row_ptr[q + 1]; ++e) put(e, R.diag[q]);
+      row(S.U_cnt[q]);
+    }
+    while (n % 4 != 0) code(ENTRY_NONE);
+    for (int i = 0; i < 8; ++i) code(ENTRY_NONE);
+  }
+  for (int32_t s = 0; s < np; ++s) {
+    S.code_off[s + 1] = S.code_off[s] + (int64_t)words[s].size();
+    S.stage_off[s + 1] = S.stage_off[s] + (int64_t)stages[s].size();
+  }
+  S.code.resize(S.code_off[np]);
+  S.stage.resize(S.stage_off[np]);
+#pragma omp parallel for schedule(dynamic, 16)
+  for (int32_t s = 0; s < np; ++s) {
+    std::copy(words[s].begin(), words[s].end(), S.code.begin() + S.code_off[s]);
+    std::copy(stages[s].begin(), stages[s].end(), S.stage.begin() + S.stage_off[s]);
+  }
+  return S;
+}
+
 }  // namespace fsi

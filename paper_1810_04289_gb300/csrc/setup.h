@@ -88,4 +88,35 @@ RasPlan build_ras(const BsrPattern& P, const double* X, int64_t n_nodes, const i
                   int32_t n_problems, int32_t np, int32_t overlap, int32_t fill_level, int32_t ordering,
                   const uint8_t* node_rank);
 
+// Packed factor stream of every subdomain: for each row in increasing order its
+// L blocks, then for each row in decreasing order its inverted pivot and its U
+// blocks (premultiplied by it when they are packed). The stream is walked in
+// entries of up to `most` (8 or 16) consecutive blocks of one row. An entry never
+// crosses a multiple of `cut` blocks of the L (resp. U) part: a row's sum is formed
+// in the pieces those multiples cut it into, the pieces being added in order.
+// Consecutive entries of up to `stage` (>= most) blocks together form a stage, the
+// unit that is copied to shared memory.
+//
+// Entry codes, one byte each, 4 per word, first entry in the low bits:
+//   bits 0-3: blocks minus 1; bit 4: the entry ends a piece of its row; bit 5: it
+//   ends the row (bit 4 is set too); bit 6: it ends its stage; no blocks: 128
+//   nothing (padding), 129 a row without L blocks, 130 the backward part begins.
+// Every subdomain's words are followed by two words of padding.
+struct StreamPlan {
+  std::vector<int64_t> L_cnt, U_cnt;  // [rows] L blocks; inverted pivot and U blocks
+  std::vector<int64_t> L_off, U_off;  // [np+1] first packed L / U block of each subdomain (one array)
+  std::vector<int64_t> src;           // [blocks] factor block copied into each packed block
+  std::vector<int32_t> col;           // [blocks] subdomain-relative column row
+  std::vector<int64_t> piv;           // [blocks] the row's inverted pivot, -1 for L blocks and the pivot itself
+  std::vector<uint32_t> code;         // entry codes
+  std::vector<int64_t> code_off;      // [np+1] first code word of each subdomain
+  std::vector<uint8_t> stage;         // blocks of each stage
+  std::vector<int64_t> stage_off;     // [np+1] first stage of each subdomain
+  int64_t max_row_blocks = 1;         // most blocks of one row in either part
+};
+constexpr uint32_t ENTRY_PIECE = 16, ENTRY_ROW = 32, ENTRY_STAGE = 64, ENTRY_NONE = 128, ENTRY_EMPTY = 129,
+                   ENTRY_BACKWARD = 130;
+constexpr int64_t STAGE_MOST = 255;  // a stage's blocks are kept in a byte
+StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage);
+
 }  // namespace fsi
