@@ -922,6 +922,7 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
 
     // packed factor streams for the TMA-fed apply
     {
+      RasStreamDev& rs = cp->rs;
       // stage geometry: NST (2) stages of SB blocks. The target is ceil(np / 152)
       // CTAs per SM, at most 8 (all subdomains resident at once up to 1,216), and
       // the ring gets what the shared memory per CTA leaves after the vector; the
@@ -939,7 +940,10 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       // the chain apply's two stages get what the vector leaves of the same budget. Mixed: it forms a
       // row's sum in the pieces the ring's stages cut it into, so that both kernels give the same bits;
       // in FP64 whole rows
-      const int64_t most = cp->mixed ? 16 : 8;
+      // four warps per subdomain where there are too few subdomains to fill the SMs' schedulers
+      // with one warp each (measured at 32 to 1,088 subdomains, ILU(1) and ILU(2): k_ras_apply_team)
+      rs.team = R.max_depth == 0 && R.np <= (cp->mixed ? 256 : 384);
+      const int64_t most = cp->mixed || rs.team ? 16 : 8;
       int64_t CB = (budget - 2048 - 8 * R.max_rows * vsz) / (2 * stride * vsz);
       CB = std::max<int64_t>(most, std::min<int64_t>(CB, 64));
       const StreamPlan S = build_stream(R, cp->mixed ? SB : (int64_t)1 << 40, most, CB);
@@ -967,7 +971,6 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
         }
         (void)Utot;
       }
-      RasStreamDev& rs = cp->rs;
       rs.sd_depth = cp->upload(R.sd_depth);
       rs.sd_item = cp->upload(R.sd_item);
       rs.item_row = cp->upload(R.item_row);

@@ -122,7 +122,8 @@ struct RasStreamDev {
   const uint8_t* stage;   // blocks of each stage of the chain apply
   const int64_t* stage_off;// [np+1] first stage of each subdomain
   int32_t stage_blocks;   // blocks per ring stage (one bulk copy; rows may straddle stages)
-  int32_t chain_blocks;   // chain apply: blocks per ring stage
+  int32_t chain_blocks;   // chain and team apply: most blocks of a stage
+  int32_t team;           // the team apply runs (four warps per subdomain)
   int64_t max_rows;       // rows of the largest subdomain
   int32_t nst;            // ring stages in flight per warp (2..8)
   int32_t stall;          // tests only: the producer issues nothing (bounded waits run out)

@@ -4,8 +4,9 @@
 // an ILU solve on an RCM-ordered subdomain is nearly the row count, so the rows are
 // worked off one after the other (forward with the unit lower factor, then backward
 // with the upper factor and inverted pivots) by one warp: lane 8 j + c takes row c
-// of the blocks j, j + 4, ... of a row. Two kernels:
+// of the blocks j, j + 4, ... of a row. Three kernels:
 //   k_ras_apply_chain: subdomains in one piece (every ordering but the dissected);
+//   k_ras_apply_team: the same where subdomains are few, four warps each;
 //   k_ras_apply_stream: nested-dissection subdomains, one warp and ring per part.
 //
 // Packed layout (built by k_pack_factors after each factorisation), per subdomain:
@@ -599,6 +600,215 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
   }
 }
 
+// Team apply: four warps per subdomain, for runs with few subdomains, where one warp
+// per SM sub-partition is all there is and a row's latency is the whole cost. The
+// blocks of an entry (up to 16 of a row) are dealt to the warps, one per 8-lane
+// group; the warps hand their products (FP32) or sums (FP64) over in shared memory,
+// meet at one barrier, and every warp adds them up and writes the row by itself (the
+// same bits), so that the row needs no second barrier. FP32 keeps the chain kernel's
+// order of additions (sums over the blocks 0..3 mod 4): the same bits. FP64 spreads
+// the work over the four sub-partitions' FP64 units (64 cycles per instruction each).
+// Measured, 46,657-node tube, ILU(1), us per apply, one warp / team:
+//   FP64  64 subdomains 4,334 / 2,797, 256: 1,545 / 1,174, 384: 1,026 / 965, 512: 940 / 1,015;
+//   mixed 64 subdomains 1,050 / 842, 256: 386 / 349, 384: 275 / 275, 512: 251 / 287.
+template <class TF>
+__global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const double* __restrict__ rin,
+                                                        double* __restrict__ z, float* __restrict__ z32,
+                                                        int32_t* err, const int* __restrict__ guard) {
+  if (guard && *guard == 0) return;
+  constexpr bool F32 = sizeof(TF) == 4;
+  constexpr int STR = Pack<TF>::stride;
+  constexpr int V = 16 / sizeof(TF), NV = 8 / V;  // values per 16-byte piece, pieces per block row
+  constexpr uint32_t BLK = STR * sizeof(TF);
+  constexpr int PT = F32 ? 7 * 20 : 7 * 4;  // values handed over per entry: FP32 [c][v][g] (20 per c), FP64 [c][v]
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);           // [2]
+  TF* part = reinterpret_cast<TF*>(smem + 128);                 // [2][PT]
+  unsigned char* ring = smem + 128 + 1152;
+  const uint32_t cap = R.chain_blocks * BLK;
+  TF* w = reinterpret_cast<TF*>(ring + 2 * cap);
+  const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, s = blockIdx.x;
+  const int c = lane & 7, g = lane >> 3;
+  const int b = F32 ? 4 * g + v : 4 * v + g;  // this lane's block of an entry
+  const int64_t r0 = R.sd_row[s];
+  const int m = (int)(R.sd_row[s + 1] - r0);
+  const uint32_t* cw = R.code + R.code_off[s];
+  const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
+  const TF* src = reinterpret_cast<const TF*>(R.pack) + (size_t)R.L_off[s] * STR;
+  const uint8_t* sz = R.stage + R.stage_off[s];
+  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
+  int nsz = left > 0 ? sz[0] : 0;
+  uint64_t win = cw[0] | (uint64_t)cw[1] << 32;
+  uint32_t ahead = cw[2];
+
+  auto feed = [&](int slot) {
+    if (threadIdx.x == 0 && left > 0) {
+      mbar_arrive_expect_tx(&full[slot], nsz * BLK);
+      bulk_g2s(ring + slot * cap, src, nsz * BLK, &full[slot]);
+      src += (size_t)nsz * STR;
+      ++sz;
+      if (--left > 0) nsz = *sz;
+    }
+  };
+  if (threadIdx.x == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    feed(0);
+    feed(1);
+  }
+  for (int q = threadIdx.x; q < m; q += 128) {
+    const double* sr = rin + 7 * (int64_t)R.gnode[r0 + q];
+    double x[7];
+#pragma unroll
+    for (int e = 0; e < 7; ++e) x[e] = sr[e];
+#pragma unroll
+    for (int e = 0; e < 7; ++e) w[8 * q + e] = (TF)x[e];
+    w[8 * q + 7] = TF(0);
+  }
+  __syncthreads();
+
+  int slot = 0, phase = 0, par = 0;
+  const unsigned char* at = ring + 16 * c + b * BLK;
+  bool ok = true;
+  auto fetch = [&](TF (&A)[8], uint32_t code) {
+    const int nb = (int)(code & 15) + 1;
+    if (F32 || 4 * v < nb) {
+#pragma unroll
+      for (int e = 0; e < NV; ++e) load16(&A[V * e], reinterpret_cast<const TF*>(at + 112 * e));
+    }
+    at += nb * BLK;
+  };
+  int q = 0, dq = 1;
+  int hi = 0;  // most blocks of an entry of the row so far (0: the row begins)
+  // FP32: the four partial sums of a row (blocks 0..3 mod 4), in every warp; FP64: this lane's sum
+  TF acc[4] = {TF(0), TF(0), TF(0), TF(0)}, tot = TF(-0.0);
+  TF A0[8], A1[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) A0[e] = A1[e] = TF(0);
+  const int cc = c < 7 ? c : 6;
+  int fslot = 0, fphase = 0;
+  auto wait = [&]() {
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
+      ok = false;
+      left = 0;
+      fslot = slot;
+      fphase = phase;
+    }
+  };
+  auto step = [&](TF (&A)[8], TF (&N)[8], uint32_t code, uint32_t ncode) {
+    if (code < ENTRY_NONE) {
+      const int nb = (int)(code & 15) + 1;
+      const bool piece = code & ENTRY_PIECE;
+      const TF old = w[8 * q + c];
+      TF* const pb = part + par * PT;
+      if (F32 || 4 * v < nb) {
+        const TF* xp = w + 8 * min((uint32_t)row_col(A), (uint32_t)m - 1);
+        TF x[8];
+#pragma unroll
+        for (int e = 0; e < NV; ++e) load16(&x[V * e], xp + V * e);
+        if (F32) {
+          const TF t = row_fma(A, x, TF(0));
+          if (c < 7) pb[20 * c + 4 * v + g] = b < nb ? t : TF(0);
+        } else {
+          // (the forward result is old - sum: the row's first block starts from -old)
+          const TF t = row_fma(A, x, hi == 0 && dq > 0 && b == 0 ? -old : acc[0]);
+          if (b < nb && c < 7) acc[0] = t;
+        }
+      }
+      hi = max(hi, nb);
+      if (!F32 && piece && 4 * v < hi) {
+        TF r = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 16);
+        r += __shfl_xor_sync(0xffffffffu, r, 8);
+        if (lane < 7) pb[4 * c + v] = r;
+        acc[0] = TF(0);
+      }
+      if (F32 || piece || (code & ENTRY_STAGE)) __syncthreads();
+      if (code & ENTRY_STAGE) {
+        feed(slot);
+        phase ^= slot;
+        slot ^= 1;
+        at = ring + slot * cap + 16 * c + b * BLK;
+        wait();
+      }
+      if (ncode < ENTRY_NONE) fetch(N, ncode);
+      if (F32) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          TF t[4];
+          load16(t, pb + 20 * cc + 4 * i);
+          if (V == 2) load16(t + 2, pb + 20 * cc + 4 * i + 2);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[i] += t[e];
+        }
+        par ^= 1;
+      }
+      if (piece) {
+        if (F32) {
+          tot += (acc[0] + acc[2]) + (acc[1] + acc[3]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[i] = TF(0);
+        } else {
+          tot = pb[4 * cc];
+          if (hi > 4) tot += pb[4 * cc + 1];
+          if (hi > 8) {
+            TF t = pb[4 * cc + 2];
+            if (hi > 12) t += pb[4 * cc + 3];
+            tot += t;
+          }
+          par ^= 1;
+        }
+        if (code & ENTRY_ROW) {
+          if (lane < 7) w[8 * q + lane] = dq > 0 ? (F32 ? old - tot : -tot) : tot;
+          __syncwarp();
+          tot = TF(-0.0);
+          hi = 0;
+          q += dq;
+        }
+      }
+    } else {
+      if (code == ENTRY_EMPTY) {
+        q += dq;
+      } else if (code == ENTRY_BACKWARD) {
+        q = m - 1;
+        dq = -1;
+      }
+      if (ncode < ENTRY_NONE) fetch(N, ncode);
+    }
+  };
+  wait();
+  if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
+  // a warp whose wait gave up goes on to the end (the data do not decide any address or barrier)
+  for (int it = 0; it < 2 * nw; ++it) {
+    const uint32_t w3 = (uint32_t)win;
+    step(A0, A1, w3 & 255, (w3 >> 8) & 255);
+    step(A1, A0, (w3 >> 8) & 255, (w3 >> 16) & 255);
+    win >>= 16;
+    if (it & 1) {
+      win |= (uint64_t)ahead << 32;
+      ahead = cw[min((it >> 1) + 3, nw + 1)];
+    }
+  }
+  if (!ok) {
+    // record it and let the copies that may still be in flight land (bounded)
+    if (lane == 0) atomicExch(err, 2);
+    mbar_wait(&full[fslot], (uint32_t)fphase);
+    mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < m; q += 128) {
+    if (R.owned[r0 + q]) {
+      const int64_t g7 = 7 * (int64_t)R.gnode[r0 + q];
+#pragma unroll
+      for (int e = 0; e < 7; ++e) z[g7 + e] = (double)w[8 * q + e];
+      if (z32) {
+#pragma unroll
+        for (int e = 0; e < 7; ++e) z32[g7 + e] = (float)w[8 * q + e];
+      }
+    }
+  }
+}
+
 // copy the factor blocks into the packed stream (7 rows of 8: the row's 7
 // entries, then the block's column); a U block with a pivot (piv >= 0) is stored as -D_q^{-1} U_qj, the
 // row's inverted pivot and the L blocks as they are
@@ -657,14 +867,17 @@ static bool takes_ring(const RasStreamDev& r) { return r.max_depth > 0; }
 
 template <class TF>
 size_t chain_smem(const RasStreamDev& r) {
-  // (an entry's last rows are read up to 15 (FP64: 7) blocks beyond its own)
-  const size_t over = (sizeof(TF) == 4 ? 15 : 7) * Pack<TF>::stride, vec = (size_t)8 * r.max_rows;
-  return 128 + ((size_t)2 * r.chain_blocks * Pack<TF>::stride + (vec > over ? vec : over)) * sizeof(TF);
+  // (an entry's last rows are read up to 15 (FP64, one warp: 7) blocks beyond its own)
+  const size_t over = (sizeof(TF) == 4 || r.team ? 15 : 7) * Pack<TF>::stride, vec = (size_t)8 * r.max_rows;
+  return (r.team ? 128 + 1152 : 128) +
+         ((size_t)2 * r.chain_blocks * Pack<TF>::stride + (vec > over ? vec : over)) * sizeof(TF);
 }
 
 template <class TF>
 cudaError_t ras_stream_init(const RasStreamDev& r) {
-  const void* k = takes_ring(r) ? (const void*)k_ras_apply_stream<TF> : (const void*)k_ras_apply_chain<TF>;
+  const void* k = takes_ring(r) ? (const void*)k_ras_apply_stream<TF>
+                  : r.team      ? (const void*)k_ras_apply_team<TF>
+                                : (const void*)k_ras_apply_chain<TF>;
   // all of the unified L1/shared storage as shared memory: several CTAs per SM;
   // the limit is the kernel's, not the context's: contexts of different sizes share it
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -678,6 +891,8 @@ cudaError_t launch_ras_apply_stream(const RasStreamDev& r, const double* rin, do
                                     const int* guard, cudaStream_t s) {
   if (takes_ring(r))
     k_ras_apply_stream<TF><<<r.np, 32 << r.max_depth, ras_stream_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
+  else if (r.team)
+    k_ras_apply_team<TF><<<r.np, 128, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   else
     k_ras_apply_chain<TF><<<r.np, 32, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   return cudaGetLastError();
