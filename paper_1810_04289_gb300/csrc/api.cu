@@ -65,7 +65,7 @@ struct fsi_ctx {
   double* Fe = nullptr;
   void* Ke = nullptr;
   int64_t ke_tets = 0;        // tets per chunk of the element Jacobian buffer
-  void* Xl = nullptr;         // per-tet local reference coordinates, Jacobian type
+  void* Xl = nullptr;         // mixed: per-tet local reference coordinates, FP32
   float* y32 = nullptr;       // mixed: FP32 copies of y, y_n, y_{n-1} for the Jacobian
   int64_t* row_ptr = nullptr;
   int32_t* col = nullptr;
@@ -247,8 +247,8 @@ void jacobian(fsi_ctx* c, const double* y) {
     launch_states_to_float(c->n, y, c->yn, c->ynm1, c->y32, c->s);
     for (int64_t t0 = 0; t0 < c->T; t0 += c->ke_tets) {
       const int64_t t1 = std::min(c->T, t0 + c->ke_tets);
-      launch_elem_jacobian<float>(c->mesh, c->mc, (const float*)c->Xl, c->y32, c->y32 + c->n, c->y32 + 2 * c->n,
-                                  (float*)c->Ke, t0, t1, c->s);
+      launch_elem_jacobian(c->mesh, c->mc, (const float*)c->Xl, c->y32, c->y32 + c->n, c->y32 + 2 * c->n,
+                           (float*)c->Ke, t0, t1, c->s);
       launch_gather_jacobian<float>(c->nnzb, c->bptr, c->bsrc, (const float*)c->Ke, (float*)c->vals, t0, t1, c->s);
       c->launches += t0 > 0 ? 2 : 0;
     }
@@ -256,11 +256,10 @@ void jacobian(fsi_ctx* c, const double* y) {
   } else {
     for (int64_t t0 = 0; t0 < c->T; t0 += c->ke_tets) {
       const int64_t t1 = std::min(c->T, t0 + c->ke_tets);
-      launch_elem_jacobian<double>(c->mesh, c->mc, (const double*)c->Xl, y, c->yn, c->ynm1, (double*)c->Ke, t0, t1,
-                                   c->s);
-      launch_gather_jacobian<double>(c->nnzb, c->bptr, c->bsrc, (const double*)c->Ke, (double*)c->vals, t0, t1,
-                                     c->s);
-      c->launches += t0 > 0 ? 2 : 0;
+      double* Ke = (double*)c->Ke;
+      launch_elem_jacobian(c->mesh, c->mc, y, c->yn, Ke + 784 * c->ke_tets, Ke, t0, t1, c->s);
+      launch_gather_jacobian<double>(c->nnzb, c->bptr, c->bsrc, Ke, (double*)c->vals, t0, t1, c->s);
+      c->launches += t0 > 0 ? 3 : 1;
     }
     launch_constraint_jacobian<double>(c->mesh, c->mc, c->diag, (double*)c->vals, c->s);
   }
@@ -752,27 +751,26 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     cp->diag = cp->upload(P.diag);
     const size_t vs = cp->mixed ? sizeof(float) : sizeof(double);
     cp->Fe = cp->dalloc<double>(28 * T0);
-    {
-      std::vector<double> xl(12 * T0);
+    if (cp->mixed) {
+      std::vector<float> xl(12 * T0);
       for (int64_t t = 0; t < T0; ++t)
         for (int a = 0; a < 4; ++a)
           for (int i = 0; i < 3; ++i)
-            xl[12 * t + 3 * a + i] = mesh->X[3 * (int64_t)tets[4 * t + a] + i] - mesh->X[3 * (int64_t)tets[4 * t] + i];
-      if (cp->mixed) {
-        std::vector<float> xf(xl.begin(), xl.end());
-        cp->Xl = cp->upload(xf);
-        cp->y32 = cp->dalloc<float>(3 * 7 * N);
-      } else {
-        cp->Xl = cp->upload(xl);
-      }
+            xl[12 * t + 3 * a + i] = (float)(mesh->X[3 * (int64_t)tets[4 * t + a] + i] -
+                                             mesh->X[3 * (int64_t)tets[4 * t] + i]);
+      cp->Xl = cp->upload(xl);
+      cp->y32 = cp->dalloc<float>(3 * 7 * N);
     }
+    double* geo = cp->dalloc<double>(GEO * T0);
     // the element Jacobian buffer Ke and the subdomain factors share one
     // allocation (sized below, once the factor size is known): Ke is live only
     // inside a Jacobian assembly, the factors only from the preconditioner
     // setup that follows it (every assembly marks the preconditioner stale)
     cp->vals = cp->dalloc<char>((int64_t)(49 * vs) * cp->nnzb);
     CK(cudaMemsetAsync(cp->vals, 0, 49 * vs * cp->nnzb, cp->s));
-    cp->mesh = MeshDev{N, T0, Tf, cp->X, cp->tets, cp->nflag, cp->nprobid, cp->inlet};
+    cp->mesh = MeshDev{N, T0, Tf, cp->X, cp->tets, cp->nflag, cp->nprobid, cp->inlet, geo};
+    launch_geometry(cp->mesh, geo, cp->s);
+    check_launch();
     cp->nwss = (int64_t)wface.size();
     cp->wface = cp->upload(wface);
     cp->wfb = cp->upload(wfb);
@@ -909,7 +907,7 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     // the factors' size (or 1 GB): the shared buffer is as large as the factors
     {
       const int64_t fac_bytes = (int64_t)(49 * vs) * rd.nblocks;
-      const int64_t per_tet = (int64_t)(784 * vs);
+      const int64_t per_tet = (int64_t)((784 + (cp->mixed ? 0 : JAC_VALUES)) * vs);
       const int64_t room = std::max<int64_t>(fac_bytes, (int64_t)1 << 30);
       cp->ke_tets = std::max<int64_t>(1, std::min<int64_t>(T0, room / per_tet));
       if (o.jac_chunk > 0) cp->ke_tets = std::min<int64_t>(T0, o.jac_chunk);

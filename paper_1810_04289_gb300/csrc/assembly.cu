@@ -27,46 +27,88 @@ __device__ __forceinline__ void load_tet(const MeshDev& m, int64_t t, int n[4], 
   }
 }
 
-// reference coordinates relative to vertex 0 (translation-invariant element
-// routines; keeps full relative precision of the edges in FP32)
-template <class T>
-__device__ __forceinline__ void load_X(const MeshDev& m, const int n[4], T Xl[4][3]) {
-  const double x0 = m.X[3 * (int64_t)n[0]], y0 = m.X[3 * (int64_t)n[0] + 1], z0 = m.X[3 * (int64_t)n[0] + 2];
+__device__ __forceinline__ void load_edges(const MeshDev& m, const int n[4], double e[3][3]) {
+  const double* x0 = m.X + 3 * (int64_t)n[0];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    Xl[a][0] = T(m.X[3 * (int64_t)n[a]] - x0);
-    Xl[a][1] = T(m.X[3 * (int64_t)n[a] + 1] - y0);
-    Xl[a][2] = T(m.X[3 * (int64_t)n[a] + 2] - z0);
+  for (int k = 0; k < 3; ++k) {
+    const double* x = m.X + 3 * (int64_t)n[k + 1];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) e[k][i] = x[i] - x0[i];
   }
 }
 
-__global__ void k_elem_residual(MeshDev m, MatConst mc, const double* __restrict__ y,
-                                const double* __restrict__ y1, const double* __restrict__ y2,
-                                double* __restrict__ Fe) {
+// reference geometry from the [GEO][T] array: gradients of vertices 1..3 and volume
+__device__ __forceinline__ void load_geo(const MeshDev& m, int64_t t, double g0[3][3], double& vol0) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) g0[k / 3][k % 3] = m.geo[k * m.T + t];
+  vol0 = m.geo[9 * m.T + t];
+}
+
+__global__ void k_geometry(MeshDev m, double* __restrict__ geo) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m.T; t += (int64_t)gridDim.x * blockDim.x) {
     int n[4];
     uint32_t f[4];
     load_tet(m, t, n, f);
-    double Xl[4][3];
-    load_X<double>(m, n, Xl);
+    double e[3][3], X[4][3], out[GEO];
+    load_edges(m, n, e);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      X[0][i] = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) X[k + 1][i] = e[k][i];
+    }
+    reference_geometry(X, out);
+#pragma unroll
+    for (int k = 0; k < GEO; ++k) geo[k * m.T + t] = out[k];
+  }
+}
+
+// the fluid tet's fields at its vertices
+struct FluidFields {
+  double u[4][3], p[4], d[4][3], u1[4][3], d1[4][3], de[3][3];
+  __device__ __forceinline__ FluidFields(const int n[4], const double* __restrict__ y, const double* __restrict__ y1) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const double* ya = y + 7 * (int64_t)n[a];
+      const double* y1a = y1 + 7 * (int64_t)n[a];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        u[a][i] = ya[i];
+        d[a][i] = ya[4 + i];
+        u1[a][i] = y1a[i];
+        d1[a][i] = y1a[4 + i];
+      }
+      p[a] = ya[3];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) de[k][i] = d[k + 1][i] - d[0][i];
+  }
+};
+
+// One thread per tet. Bound by the FP64 pipe; closed-form integrals and stored
+// reference geometry (see element.cuh)
+__global__ void __launch_bounds__(128) k_elem_residual(MeshDev m, MatConst mc, const double* __restrict__ y,
+                                                       const double* __restrict__ y1, const double* __restrict__ y2,
+                                                       double* __restrict__ Fe) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m.T; t += (int64_t)gridDim.x * blockDim.x) {
+    int n[4];
+    uint32_t f[4];
+    load_tet(m, t, n, f);
+    double g0[3][3], vol0;
+    load_geo(m, t, g0, vol0);
     double out[4][7];
     if (t < m.Tf) {
-      double u[4][3], p[4], d[4][3], u1[4][3], d1[4][3];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const double* ya = y + 7 * (int64_t)n[a];
-        const double* y1a = y1 + 7 * (int64_t)n[a];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          u[a][i] = ya[i];
-          d[a][i] = ya[4 + i];
-          u1[a][i] = y1a[i];
-          d1[a][i] = y1a[4 + i];
-        }
-        p[a] = ya[3];
-      }
-      double Rm[4][3], Rc[4], Rh[4][3];
-      fluid_element<double, double>(Xl, u, p, d, u1, d1, mc, Rm, Rc, Rh);
+      const FluidFields q(n, y, y1);
+      double Xe[3][3];
+      load_edges(m, n, Xe);
+      FluidValues v;
+      fluid_values(Xe, q.de, q.u, q.p, q.d, q.u1, q.d1, m.geo[10 * m.T + t], m.geo[11 * m.T + t], mc, v);
+      double F[4][3], Rm[4][3], gr[4], Rc[4], Rh[4][3];
+      fluid_momentum(v, F, Rm);
+      fluid_continuity(v, gr, Rc);
+      mesh_motion(q.de, g0, vol0, Rh);
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
         const bool uc = f[a] & NF_U_CONSTR, pc = f[a] & NF_P_IDENT, dz = f[a] & NF_D_ZERO, itf = f[a] & NF_ITF;
@@ -78,7 +120,7 @@ __global__ void k_elem_residual(MeshDev m, MatConst mc, const double* __restrict
         out[a][3] = pc ? 0.0 : Rc[a];
       }
     } else {
-      double d[4][3], d1[4][3], d2[4][3];
+      double d[4][3], d1[4][3], d2[4][3], de[3][3];
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -87,8 +129,12 @@ __global__ void k_elem_residual(MeshDev m, MatConst mc, const double* __restrict
           d1[a][i] = y1[7 * (int64_t)n[a] + 4 + i];
           d2[a][i] = y2[7 * (int64_t)n[a] + 4 + i];
         }
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) de[k][i] = d[k + 1][i] - d[0][i];
       double Rw[4][3];
-      wall_element<double, double>(Xl, d, d1, d2, mc, Rw);
+      wall_residual(de, g0, vol0, d, d1, d2, mc, Rw);
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
         const bool dz = f[a] & NF_D_ZERO;
@@ -148,11 +194,11 @@ __global__ void k_constraint_residual(MeshDev m, MatConst mc, double t, const do
   }
 }
 
-// One Jacobian column per thread: 28 threads per tet (column = node b, dof k),
-// forward-mode derivative of the element residual along that column. Inputs
-// are already in the arithmetic type T: per-tet reference coordinates relative
-// to vertex 0 (Xl, 12 per tet) and node states (y, y_old, y_older), so the FP32
-// kernel runs no FP64 instruction.
+// Mixed form: one Jacobian column per thread, 28 threads per tet (column = node b,
+// dof k), forward-mode derivative of the element residual along that column in
+// T = float. Inputs are already in T: per-tet reference coordinates relative to
+// vertex 0 (Xl, 12 per tet) and node states (y, y_old, y_older), so the kernel runs
+// no FP64 instruction.
 constexpr int JAC_TETS_PER_BLOCK = 8;
 
 template <class T>
@@ -236,6 +282,250 @@ k_elem_jacobian(MeshDev m, MatConst mc, const T* __restrict__ Xl, const T* __res
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP64 element Jacobian in closed form, two kernels. With column (b, k) of a
+// fluid tet the derivatives of every intermediate are of rank one in g_b:
+//   dG_ij = alpha_i g_b,j, d(grad p) = gamma g_b, d(a_b,k) = eta, d|K| = nu |K|,
+//   dg_a = -zeta_a g_b, dD = theta D,
+// (u column: alpha = e_k, eta = 1; p: gamma = 1; d: alpha = -G e_k, gamma = -grad p_k,
+// eta = -1/dt, nu = g_b,k, zeta_a = g_a,k), so a column is a handful of products of
+// per-tet and per-(a, b) values. k_jac_values computes those once per tet (one
+// thread per tet), k_elem_jacobian64 one column per thread from them: 28 x ~170
+// FP64 instructions per tet in place of 28 x ~1,900 with dual numbers, each of which
+// redid the value part. Bound by the FP64 pipe all the same.
+// ---------------------------------------------------------------------------
+enum : int {  // per-tet values, laid out [JV][tets of the chunk]; fluid tets:
+  JV_G = 0,       // gradients g[4][3]
+  JV_GU = 12,     // velocity gradient G[3][3]
+  JV_GP = 21,     // pressure gradient
+  JV_S = 24,      // S_a = sum_c a_c . g_a
+  JV_E1 = 28,     // [b][a] factor of alpha_i in the momentum rows
+  JV_E2 = 44,     // [b][a] factor of beta_i (the direct part of the inertia's derivative)
+  JV_H = 60,      // n_b + W
+  JV_Q = 72,      // c Q g_a
+  JV_RM = 84,     // momentum residual
+  JV_F = 96,      // P g_b
+  JV_RC = 108,    // continuity residual
+  JV_GR = 112,    // g_a . r |K|/D
+  JV_K = 116,     // mesh-motion stiffness [b][a]
+  JV_TH = 132,    // theta per unit eta, k = 0..2
+  JV_SC = 135,    // |K|, c, |K|/D, |K| tau_C rho div u, |K| tau_C rho
+  JV = JAC_VALUES,
+  // wall tets: F g0_a, |K0| mu F F^T, [b][a] diagonal part, [b][a] g0_a . g0_b
+  JW_F = 0, JW_B = 12, JW_D = 21, JW_GG = 37
+};
+
+__global__ void __launch_bounds__(128) k_jac_values(MeshDev m, MatConst mc, const double* __restrict__ y,
+                                                    const double* __restrict__ y1, double* __restrict__ val,
+                                                    int64_t t0, int64_t t1) {
+  const int64_t nt = t1 - t0;
+  for (int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < t1;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    double* o = val + (t - t0);
+    auto put = [&](int k, double v) { o[k * nt] = v; };
+    int n[4];
+    uint32_t f[4];
+    load_tet(m, t, n, f);
+    double g0[3][3], vol0, ga[4][3];
+    load_geo(m, t, g0, vol0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) ga[k + 1][i] = g0[k][i];
+      ga[0][i] = rest(g0[0][i], g0[1][i], g0[2][i]);
+    }
+    if (t < m.Tf) {
+      FluidValues v;
+      {
+        const FluidFields q(n, y, y1);
+        double Xe[3][3];
+        load_edges(m, n, Xe);
+        fluid_values(Xe, q.de, q.u, q.p, q.d, q.u1, q.d1, m.geo[10 * m.T + t], m.geo[11 * m.T + t], mc, v);
+      }
+      const double rho = mc.rho_f, k20 = 0.05 * v.vol;
+      {
+        double F[4][3], Rm[4][3], gr[4], Rc[4];
+        fluid_momentum(v, F, Rm);
+        fluid_continuity(v, gr, Rc);
+        const double tv = v.ip * v.vol;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            put(JV_RM + 3 * a + i, Rm[a][i]);
+            put(JV_F + 3 * a + i, F[a][i]);
+            put(JV_H + 3 * a + i, v.n[a][i] + v.W[i]);
+            put(JV_G + 3 * a + i, v.g[a][i]);
+            put(JV_Q + 3 * a + i,
+                v.c * (v.Q[i][0] * v.g[a][0] + v.Q[i][1] * v.g[a][1] + v.Q[i][2] * v.g[a][2]));
+          }
+          put(JV_RC + a, Rc[a]);
+          put(JV_GR + a, tv * gr[a]);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) put(JV_GU + 3 * i + j, v.G[i][j]);
+          put(JV_GP + i, v.gp[i]);
+          // dD/D per unit of d(a_b,k): (2 rho / h)^2 (A_k/4) / (4 D^2)
+          put(JV_TH + i, 0.25 * rho * rho * m.geo[11 * m.T + t] * v.A[i] * (v.ip * v.ip));
+        }
+        put(JV_SC + 0, v.vol);
+        put(JV_SC + 1, v.c);
+        put(JV_SC + 2, tv);
+        put(JV_SC + 3, v.vol * v.tc * v.div);
+        put(JV_SC + 4, v.vol * v.tc);
+      }
+      double s[4][4], S[4];  // s[c][a] = a_c . g_a
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c][a] = v.a[c][0] * v.g[a][0] + v.a[c][1] * v.g[a][1] + v.a[c][2] * v.g[a][2];
+        S[a] = (s[0][a] + s[1][a]) + (s[2][a] + s[3][a]);
+        put(JV_S + a, S[a]);
+      }
+      const double rc = rho * v.c, rk = rho * k20, vm = v.vol * mc.mu_f;
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          double zz = S[a] * S[b];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) zz += s[c][a] * s[c][b];
+          const double gg = v.g[a][0] * v.g[b][0] + v.g[a][1] * v.g[b][1] + v.g[a][2] * v.g[b][2];
+          put(JV_E1 + 4 * b + a, rc * zz + rk * (S[b] + s[a][b]) + vm * gg);
+          put(JV_E2 + 4 * b + a, v.c * (s[b][a] + S[a]) + (a == b ? 2.0 * k20 : k20));
+          put(JV_K + 4 * b + a, vol0 * (ga[a][0] * ga[b][0] + ga[a][1] * ga[b][1] + ga[a][2] * ga[b][2]));
+        }
+    } else {
+      double de[3][3], F[3][3], S[3][3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) de[k][i] = y[7 * (int64_t)n[k + 1] + 4 + i] - y[7 * (int64_t)n[0] + 4 + i];
+      wall_stress(de, g0, mc, F, S);
+      const double idt = 1.0 / mc.dt, k20 = vol0 * (1.0 / 20.0) * (mc.rho_s * idt * idt + mc.eta_s * idt);
+      double fa[4][3], Sg[4][3];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          fa[a][i] = F[i][0] * ga[a][0] + F[i][1] * ga[a][1] + F[i][2] * ga[a][2];
+          Sg[a][i] = S[i][0] * ga[a][0] + S[i][1] * ga[a][1] + S[i][2] * ga[a][2];
+          put(JW_F + 3 * a + i, fa[a][i]);
+        }
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          put(JW_B + 3 * i + j, vol0 * mc.mu_s * (F[i][0] * F[j][0] + F[i][1] * F[j][1] + F[i][2] * F[j][2]));
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const double gSg = ga[a][0] * Sg[b][0] + ga[a][1] * Sg[b][1] + ga[a][2] * Sg[b][2];
+          put(JW_D + 4 * b + a, vol0 * gSg + (a == b ? 2.0 * k20 : k20));
+          put(JW_GG + 4 * b + a, ga[a][0] * ga[b][0] + ga[a][1] * ga[b][1] + ga[a][2] * ga[b][2]);
+        }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(28 * JAC_TETS_PER_BLOCK)
+k_elem_jacobian64(MeshDev m, MatConst mc, const double* __restrict__ val, double* __restrict__ Ke, int64_t t0,
+                  int64_t t1) {
+  __shared__ double sv[JAC_TETS_PER_BLOCK][JV + 1];  // odd row length: the tets of a block on other banks
+  const int64_t nt = t1 - t0;
+  const int tl = threadIdx.x / 28;
+  const int colid = threadIdx.x - 28 * tl;
+  const int b = colid / 7, k = colid - 7 * (colid / 7);
+  for (int64_t tb = t0 + blockIdx.x * (int64_t)JAC_TETS_PER_BLOCK; tb < t1;
+       tb += (int64_t)gridDim.x * JAC_TETS_PER_BLOCK) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < JV * JAC_TETS_PER_BLOCK; i += 28 * JAC_TETS_PER_BLOCK) {
+      const int v = i / JAC_TETS_PER_BLOCK, q = i % JAC_TETS_PER_BLOCK;
+      if (tb + q < t1) sv[q][v] = val[v * nt + (tb - t0) + q];
+    }
+    __syncthreads();
+    const int64_t t = tb + tl;
+    if (t >= t1) continue;  // (the loop's barriers come before this point for every thread: tb is the block's)
+    const double* s = sv[tl];
+    int n[4];
+    uint32_t f[4];
+    load_tet(m, t, n, f);
+    double* o = Ke + 784 * (t - t0) + 49 * b + k;
+    if (t < m.Tf) {
+      const bool isu = k < 3, isp = k == 3, isd = k > 3;
+      const int kk = isu ? k : (isd ? k - 4 : 0);
+      const double idt = 1.0 / mc.dt, rho = mc.rho_f;
+      const double eta = isu ? 1.0 : (isd ? -idt : 0.0);
+      const double gam = isp ? 1.0 : (isd ? -s[JV_GP + kk] : 0.0);
+      const double* gb = s + JV_G + 3 * b;
+      const double nu = isd ? gb[kk] : 0.0;
+      const double vol = s[JV_SC], c = s[JV_SC + 1], tv = s[JV_SC + 2];
+      const double theta = eta * s[JV_TH + kk];
+      double al[3], be[3], h[3], dr[3];
+      const double rq = 0.25 * rho * s[JV_S + b];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const double Gik = s[JV_GU + 3 * i + kk];
+        al[i] = isu ? (i == kk ? 1.0 : 0.0) : (isd ? -Gik : 0.0);
+        be[i] = rho * eta * Gik + (isu && i == kk ? rho * idt : 0.0);
+        h[i] = s[JV_H + 3 * b + i];
+        dr[i] = tv * (rq * al[i] + 0.25 * be[i] + gam * gb[i]);
+      }
+      const double om = al[0] * gb[0] + al[1] * gb[1] + al[2] * gb[2];
+      const double gac = theta * s[JV_SC + 3] + om * s[JV_SC + 4] - (isp ? 0.25 * vol : 0.0);
+      const double cg5 = 5.0 * c * gam, ceta = c * eta, vmu = vol * mc.mu_f, q4 = 0.25 * vol * om;
+      const double grb = s[JV_GR + b];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const double* ga = s + JV_G + 3 * a;
+        const double g0 = ga[0], g1 = ga[1], g2 = ga[2];
+        const double gk = ga[kk];
+        const double zeta = isd ? gk : 0.0, hc = ceta * gk;
+        const double gbc = vmu * (al[0] * g0 + al[1] * g1 + al[2] * g2) + cg5 * s[JV_S + a];
+        const double e1 = s[JV_E1 + 4 * b + a], e2 = s[JV_E2 + 4 * b + a];
+        const bool uc = f[a] & NF_U_CONSTR, pc = f[a] & NF_P_IDENT, dz = f[a] & NF_D_ZERO, itf = f[a] & NF_ITF;
+        const double K = isd ? s[JV_K + 4 * b + a] : 0.0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          double r = nu * s[JV_RM + 3 * a + i] - theta * s[JV_Q + 3 * a + i];
+          r += al[i] * e1;
+          r += be[i] * e2;
+          r += h[i] * hc;
+          r += gb[i] * gbc;
+          r += (i == 0 ? g0 : i == 1 ? g1 : g2) * gac;
+          r -= zeta * s[JV_F + 3 * b + i];
+          o[196 * a + 7 * i] = uc ? 0.0 : r;
+          o[196 * a + 7 * (4 + i)] = dz ? 0.0 : (itf ? r : (i == kk ? K : 0.0));
+        }
+        const double rc = nu * s[JV_RC + a] + q4 - theta * s[JV_GR + a] - zeta * grb + g0 * dr[0] + g1 * dr[1] +
+                          g2 * dr[2];
+        o[196 * a + 7 * 3] = pc ? 0.0 : rc;
+      }
+    } else {
+      // d column k of node b: |K0| (F S)' g0_a and the inertia
+      const int kk = k > 3 ? k - 4 : 0;
+      const double vmu = mc.mu_s * m.geo[9 * m.T + t], vlam = mc.lam_s * m.geo[9 * m.T + t];
+      const double fbk = s[JW_F + 3 * b + kk];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const bool z = (f[a] & NF_D_ZERO) || k < 4;
+        const double gg = s[JW_GG + 4 * b + a], fak = vmu * s[JW_F + 3 * a + kk], lb = vlam * fbk;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          double r = s[JW_B + 3 * i + kk] * gg + s[JW_F + 3 * b + i] * fak + lb * s[JW_F + 3 * a + i];
+          if (i == kk) r += s[JW_D + 4 * b + a];
+          o[196 * a + 7 * i] = 0.0;
+          o[196 * a + 7 * (4 + i)] = z ? 0.0 : r;
+        }
+        o[196 * a + 7 * 3] = 0.0;
+      }
+    }
+  }
+}
+
 __global__ void k_states_to_float(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
                                   const double* __restrict__ c, float* __restrict__ out) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -308,13 +598,26 @@ void launch_constraint_residual(const MeshDev& m, const MatConst& mc, double t, 
   k_constraint_residual<<<grid_for(m.N, 256), 256, 0, s>>>(m, mc, t, y, y1, F);
 }
 
-template <class T>
-void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const T* Xl, const T* y, const T* y1, const T* y2,
-                          T* Ke, int64_t t0, int64_t t1, cudaStream_t s) {
+inline int jac_blocks(int64_t nt) {
+  const int64_t blocks = (nt + JAC_TETS_PER_BLOCK - 1) / JAC_TETS_PER_BLOCK;
+  return (int)(blocks > 152 * 256 ? 152 * 256 : blocks);
+}
+
+void launch_geometry(const MeshDev& m, double* geo, cudaStream_t s) {
+  if (m.T > 0) k_geometry<<<grid_for(m.T, 128), 128, 0, s>>>(m, geo);
+}
+
+void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const float* Xl, const float* y, const float* y1,
+                          const float* y2, float* Ke, int64_t t0, int64_t t1, cudaStream_t s) {
   if (t1 <= t0) return;
-  int64_t blocks = (t1 - t0 + JAC_TETS_PER_BLOCK - 1) / JAC_TETS_PER_BLOCK;
-  if (blocks > 152 * 256) blocks = 152 * 256;
-  k_elem_jacobian<T><<<(int)blocks, 28 * JAC_TETS_PER_BLOCK, 0, s>>>(m, mc, Xl, y, y1, y2, Ke, t0, t1);
+  k_elem_jacobian<float><<<jac_blocks(t1 - t0), 28 * JAC_TETS_PER_BLOCK, 0, s>>>(m, mc, Xl, y, y1, y2, Ke, t0, t1);
+}
+
+void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const double* y, const double* y1, double* val,
+                          double* Ke, int64_t t0, int64_t t1, cudaStream_t s) {
+  if (t1 <= t0) return;
+  k_jac_values<<<grid_for(t1 - t0, 128), 128, 0, s>>>(m, mc, y, y1, val, t0, t1);
+  k_elem_jacobian64<<<jac_blocks(t1 - t0), 28 * JAC_TETS_PER_BLOCK, 0, s>>>(m, mc, val, Ke, t0, t1);
 }
 
 void launch_states_to_float(int64_t n, const double* a, const double* b, const double* c, float* out,
@@ -334,10 +637,6 @@ void launch_constraint_jacobian(const MeshDev& m, const MatConst& mc, const int3
   k_constraint_jacobian<T><<<grid_for(m.N, 256), 256, 0, s>>>(m, mc, diag, vals);
 }
 
-template void launch_elem_jacobian<double>(const MeshDev&, const MatConst&, const double*, const double*,
-                                           const double*, const double*, double*, int64_t, int64_t, cudaStream_t);
-template void launch_elem_jacobian<float>(const MeshDev&, const MatConst&, const float*, const float*,
-                                          const float*, const float*, float*, int64_t, int64_t, cudaStream_t);
 template void launch_gather_jacobian<double>(int64_t, const int64_t*, const int32_t*, const double*, double*,
                                              int64_t, int64_t, cudaStream_t);
 template void launch_gather_jacobian<float>(int64_t, const int64_t*, const int32_t*, const float*, float*,

@@ -17,6 +17,10 @@
 //   D = sqrt((2 rho/dt)^2 + (2 rho |a_c|/h)^2 + (4 mu/h^2)^2), a_c = (u - w) at the
 //   centroid, tau_M = rho/D (SUPG), tau_M/rho = 1/D (PSPG), tau_C rho = h^2 D/12.
 // The 4-point degree-2 rule integrates every term exactly for P1 fields.
+//
+// fluid_element / wall_element evaluate that rule as it stands; in Dual<float> they
+// give the mixed form's Jacobian columns. The FP64 residual and Jacobian take the
+// integrals in closed form instead (fluid_values and the functions after it).
 #pragma once
 #include "dual.cuh"
 
@@ -223,6 +227,213 @@ __device__ __forceinline__ void wall_element(const T X[4][3], const S d[4][3], c
       S sum = acc[0][i] + acc[1][i] + acc[2][i] + acc[3][i] + acc[a][i];
       Rw[a][i] = vol0 * ((T(1) / T(20)) * sum + P[i][0] * g0[a][0] + P[i][1] * g0[a][1] + P[i][2] * g0[a][2]);
     }
+}
+
+// ---------------------------------------------------------------------------
+// FP64: the same residuals with the integrals in closed form
+// ---------------------------------------------------------------------------
+// Every integrand is a product of at most two P1 fields, and for nodal values
+// f_b, g_b: int f g = |K|/20 (sum f sum g + sum_b f_b g_b). With the advection
+// velocity a_b and the inertia n_b = rho ((u_b - u1_b)/dt + G a_b) at the vertices
+// (G constant), A = sum a_b, N = sum n_b, W = N + 5 grad p and
+//   Q_ij = A_j W_i + sum_b n_b,i a_b,j,
+//   P_ij = |K| sigma_ij + c Q_ij,   c = tau_M |K|/20,
+//   sigma_ij = mu (G_ij + G_ji) + delta_ij (tau_C rho div u - mean p),
+// the momentum row is Rm_a = P g_a + |K|/20 (N + n_a): about half the FP64
+// instructions of the quadrature loop. The FP64 pipe bounds both kernels (4 warps
+// of an SM issue one FP64 instruction per 19 cycles), so it is instructions that count.
+
+// reference geometry of a tet, laid out [GEO][T] at creation
+constexpr int GEO = 12;  // gradients of vertices 1..3 (9), volume, h^2, 1/h^2
+
+__device__ __forceinline__ void reference_geometry(const double X[4][3], double out[GEO]) {
+  double g[4][3], vol;
+  tet_gradients<double>(X, g, vol);
+  const double h = cbrt(6.0 * sqrt(2.0) * vol);
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[3 * k + i] = g[k + 1][i];
+  out[9] = vol;
+  out[10] = h * h;
+  out[11] = 1.0 / (h * h);
+}
+
+struct FluidValues {
+  double g[4][3], vol;       // current gradients and volume
+  double G[3][3], gp[3], div;
+  double a[4][3], A[3];      // advection velocity at the vertices, its sum
+  double n[4][3], W[3];      // inertia at the vertices, N + 5 grad p
+  double arg, ip;            // D^2, 1/D
+  double c, tc;              // tau_M |K|/20, tau_C rho
+  double Q[3][3], P[3][3];
+  double r[3];               // mean strong residual N/4 + grad p
+};
+
+// v_0 = -(v_1 + v_2 + v_3) of quantities that sum to zero over the vertices
+__device__ __forceinline__ double rest(double a, double b, double c) { return -(a + b + c); }
+
+// Xe, de: edges from vertex 0 of the reference tet and of d; ue, pe those of u and p
+__device__ __forceinline__ void fluid_values(const double Xe[3][3], const double de[3][3], const double u[4][3],
+                                             const double p[4], const double d[4][3], const double u1[4][3],
+                                             const double d1[4][3], double h2, double ih2, const MatConst& m,
+                                             FluidValues& v) {
+  const double rho = m.rho_f, idt = 1.0 / m.dt;
+  double e[3][3], x[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) e[k][i] = Xe[k][i] + de[k][i];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int q = (k + 1) % 3, s = (k + 2) % 3;
+    x[k][0] = e[q][1] * e[s][2] - e[q][2] * e[s][1];
+    x[k][1] = e[q][2] * e[s][0] - e[q][0] * e[s][2];
+    x[k][2] = e[q][0] * e[s][1] - e[q][1] * e[s][0];
+  }
+  const double det = e[0][0] * x[0][0] + e[0][1] * x[0][1] + e[0][2] * x[0][2];
+  const double inv = 1.0 / det;
+  v.vol = det * (1.0 / 6.0);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v.g[k + 1][i] = x[k][i] * inv;
+    v.g[0][i] = rest(v.g[1][i], v.g[2][i], v.g[3][i]);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double w1 = u[1][i] - u[0][i], w2 = u[2][i] - u[0][i], w3 = u[3][i] - u[0][i];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) v.G[i][j] = w1 * v.g[1][j] + w2 * v.g[2][j] + w3 * v.g[3][j];
+    v.gp[i] = (p[1] - p[0]) * v.g[1][i] + (p[2] - p[0]) * v.g[2][i] + (p[3] - p[0]) * v.g[3][i];
+  }
+  v.div = v.G[0][0] + v.G[1][1] + v.G[2][2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) v.a[b][i] = u[b][i] - (d[b][i] - d1[b][i]) * idt;
+    v.A[i] = (v.a[0][i] + v.a[1][i]) + (v.a[2][i] + v.a[3][i]);
+  }
+  // D^2 with the centroid's advection velocity A/4
+  const double ct = 2.0 * rho * idt, cv = 4.0 * m.mu_f * ih2;
+  v.arg = (ct * ct + cv * cv) +
+          (0.25 * rho * rho * ih2) * (v.A[0] * v.A[0] + v.A[1] * v.A[1] + v.A[2] * v.A[2]);
+  v.ip = rsqrt(v.arg);
+  v.tc = (h2 * (1.0 / 12.0)) * (v.arg * v.ip);
+  v.c = rho * v.ip * v.vol * 0.05;
+  const double ridt = rho * idt;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double r0 = rho * v.G[i][0], r1 = rho * v.G[i][1], r2 = rho * v.G[i][2];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      v.n[b][i] = ridt * (u[b][i] - u1[b][i]) + r0 * v.a[b][0] + r1 * v.a[b][1] + r2 * v.a[b][2];
+    const double N = (v.n[0][i] + v.n[1][i]) + (v.n[2][i] + v.n[3][i]);
+    v.W[i] = N + 5.0 * v.gp[i];
+    v.r[i] = 0.25 * N + v.gp[i];
+  }
+  const double pc = 0.25 * ((p[0] + p[1]) + (p[2] + p[3]));
+  const double iso = v.vol * (v.tc * v.div - pc), vm = v.vol * m.mu_f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      double q = v.A[j] * v.W[i];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) q += v.n[b][i] * v.a[b][j];
+      v.Q[i][j] = q;
+      const double s = vm * (v.G[i][j] + v.G[j][i]) + v.c * q;
+      v.P[i][j] = i == j ? s + iso : s;
+    }
+}
+
+// Rm_a = P g_a + |K|/20 (N + n_a); F = P g_a
+__device__ __forceinline__ void fluid_momentum(const FluidValues& v, double F[4][3], double Rm[4][3]) {
+  const double k20 = 0.05 * v.vol;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+#pragma unroll
+    for (int a = 1; a < 4; ++a) F[a][i] = v.P[i][0] * v.g[a][0] + v.P[i][1] * v.g[a][1] + v.P[i][2] * v.g[a][2];
+    F[0][i] = rest(F[1][i], F[2][i], F[3][i]);
+    const double N = v.W[i] - 5.0 * v.gp[i];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) Rm[a][i] = k20 * (N + v.n[a][i]) + F[a][i];
+  }
+}
+
+// Rc_a = |K| div u/4 + |K| gr_a / D, gr_a = g_a . r
+__device__ __forceinline__ void fluid_continuity(const FluidValues& v, double gr[4], double Rc[4]) {
+#pragma unroll
+  for (int a = 1; a < 4; ++a) gr[a] = v.g[a][0] * v.r[0] + v.g[a][1] * v.r[1] + v.g[a][2] * v.r[2];
+  gr[0] = rest(gr[1], gr[2], gr[3]);
+  const double t = v.ip * v.vol, q = 0.25 * v.vol * v.div;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) Rc[a] = t * gr[a] + q;
+}
+
+// harmonic mesh motion Rh_a = |K0| (sum_b d_b (x) g0_b) g0_a; g0: vertices 1..3
+__device__ __forceinline__ void mesh_motion(const double de[3][3], const double g0[3][3], double vol0,
+                                            double Rh[4][3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    double H[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      H[j] = vol0 * (de[0][i] * g0[0][j] + de[1][i] * g0[1][j] + de[2][i] * g0[2][j]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) Rh[k + 1][i] = H[0] * g0[k][0] + H[1] * g0[k][1] + H[2] * g0[k][2];
+    Rh[0][i] = rest(Rh[1][i], Rh[2][i], Rh[3][i]);
+  }
+}
+
+// Wall tet: F, second Piola-Kirchhoff S and first P on the reference gradients
+__device__ __forceinline__ void wall_stress(const double de[3][3], const double g0[3][3], const MatConst& m,
+                                            double F[3][3], double S[3][3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      F[i][j] = de[0][i] * g0[0][j] + de[1][i] * g0[1][j] + de[2][i] * g0[2][j] + (i == j ? 1.0 : 0.0);
+  double E[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) {
+      E[i][j] = 0.5 * (F[0][i] * F[0][j] + F[1][i] * F[1][j] + F[2][i] * F[2][j] - (i == j ? 1.0 : 0.0));
+      E[j][i] = E[i][j];
+    }
+  const double tr = m.lam_s * (E[0][0] + E[1][1] + E[2][2]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) S[i][j] = 2.0 * m.mu_s * E[i][j] + (i == j ? tr : 0.0);
+}
+
+// Rw_a = |K0| (sum_b acc_b + acc_a)/20 + |K0| F S g0_a, acc = rho (d - 2 d1 + d2)/dt^2 + eta (d - d1)/dt
+__device__ __forceinline__ void wall_residual(const double de[3][3], const double g0[3][3], double vol0,
+                                              const double d[4][3], const double d1[4][3], const double d2[4][3],
+                                              const MatConst& m, double Rw[4][3]) {
+  double F[3][3], S[3][3];
+  wall_stress(de, g0, m, F, S);
+  const double idt = 1.0 / m.dt;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    double P[3], acc[4];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) P[j] = vol0 * (F[i][0] * S[0][j] + F[i][1] * S[1][j] + F[i][2] * S[2][j]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const double vs = (d[b][i] - d1[b][i]) * idt, vs1 = (d1[b][i] - d2[b][i]) * idt;
+      acc[b] = m.rho_s * (vs - vs1) * idt + m.eta_s * vs;
+    }
+    const double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]), k20 = vol0 * (1.0 / 20.0);
+    double f[4];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f[k + 1] = P[0] * g0[k][0] + P[1] * g0[k][1] + P[2] * g0[k][2];
+    f[0] = rest(f[1], f[2], f[3]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) Rw[a][i] = k20 * (sum + acc[a]) + f[a];
+  }
 }
 
 }  // namespace fsi

@@ -18,6 +18,7 @@ struct MeshDev {
   const uint32_t* nflag;     // [N]
   const int32_t* nprob;      // [N]
   const double* inlet;       // [nprob*INLET_STRIDE]
+  const double* geo;         // [GEO][T] reference geometry of every tet (element.cuh)
 };
 
 // ---- wall shear stress (wss.cu): face = 4 * fluid tet + local index of the
@@ -32,12 +33,17 @@ void launch_gather_residual(const MeshDev& m, const int64_t* nptr, const int32_t
                             double* F, cudaStream_t s);
 void launch_constraint_residual(const MeshDev& m, const MatConst& mc, double t, const double* y,
                                 const double* y1, double* F, cudaStream_t s);
-// Xl: per-tet reference coordinates relative to vertex 0 (12 per tet); y, y1, y2
-// node states, all in the arithmetic type T
-// element Jacobians of the tets [t0, t1) into Ke (784 values per tet, from tet t0)
-template <class T>
-void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const T* Xl, const T* y, const T* y1, const T* y2,
-                          T* Ke, int64_t t0, int64_t t1, cudaStream_t s);
+// reference geometry of every tet into geo ([GEO][T])
+void launch_geometry(const MeshDev& m, double* geo, cudaStream_t s);
+// element Jacobians of the tets [t0, t1) into Ke (784 values per tet, from tet t0).
+// Mixed form: Xl per-tet reference coordinates relative to vertex 0 (12 per tet), all
+// inputs FP32
+void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const float* Xl, const float* y, const float* y1,
+                          const float* y2, float* Ke, int64_t t0, int64_t t1, cudaStream_t s);
+// FP64: val holds JAC_VALUES values per tet of the chunk
+constexpr int JAC_VALUES = 140;
+void launch_elem_jacobian(const MeshDev& m, const MatConst& mc, const double* y, const double* y1, double* val,
+                          double* Ke, int64_t t0, int64_t t1, cudaStream_t s);
 // out = [a | b | c] converted to FP32 (3 n floats)
 void launch_states_to_float(int64_t n, const double* a, const double* b, const double* c, float* out,
                             cudaStream_t s);
