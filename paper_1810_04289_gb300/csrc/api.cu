@@ -318,6 +318,7 @@ void pc_setup(fsi_ctx* c) {
   CK(cudaMemcpyAsync(&c->hbuf[1], c->errflag, sizeof(int32_t), cudaMemcpyDeviceToHost, c->s));
   CK(cudaStreamSynchronize(c->s));
   std::memcpy(&e, &c->hbuf[1], sizeof(int32_t));
+  if (e == 2) throw StatusError{FSI_ERR_TIMEOUT, "a bounded wait in the subdomain factorisation gave up"};
   if (e) throw StatusError{FSI_ERR_ZERO_PIVOT, "singular pivot block in the subdomain ILU factorisation"};
   c->pc_stale = false;
 }
@@ -859,9 +860,6 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     rd.lent_ptr = cp->upload(R.lent_ptr);
     rd.lent_pos = cp->upload(R.lent_pos);
     rd.lent_kdiag = cp->upload(R.lent_kdiag);
-    rd.upd_ptr = cp->upload(R.upd_ptr);
-    rd.upd_tgt = cp->upload(R.upd_tgt);
-    rd.upd_src = cp->upload(R.upd_src);
     rd.sd_lvlL = cp->upload(R.sd_lvlL);
     rd.sd_lvlU = cp->upload(R.sd_lvlU);
     rd.lvlL_ptr = cp->upload(R.lvlL_ptr);
@@ -889,7 +887,26 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       auto fits = [&](int mode) { return cp->mixed ? ras_factor_fits<float>(rd, mode) : ras_factor_fits<double>(rd, mode); };
       // automatic: nested-dissection groups when the subdomains are dissected and
       // the groups' rows fit, else the row-only sequential kernel
-      const int want = o.factor_mode > 0 ? o.factor_mode - 1 : (R.max_depth > 0 && fits(3) ? 3 : 2);
+      int want = o.factor_mode > 0 ? o.factor_mode - 1 : (R.max_depth > 0 && fits(3) ? 3 : 2);
+      FactorPipe FP;
+      if (o.factor_mode == 0 && want == 2) {
+        // the pipelined kernel (sparse.cu, k_ras_factor_pipe) where its slots fit, two CTAs per SM
+        // (one where there are few subdomains): up to 8 L blocks in flight, of up to 32 blocks or
+        // the mean row length each (longer ones are read directly)
+        const int64_t cap = std::max<int64_t>(32, rd.nblocks / std::max<int64_t>(1, (int64_t)R.gnode.size()));
+        FP = build_factor_pipe(R, cap, (int64_t)vs);
+        rd.pipe_meta = (int32_t)(16 * FP.max_meta);
+        rd.pipe_data = (int32_t)(16 * ((49 * vs * FP.max_len + 31 + 15) / 16));
+        for (int per_sm = 2; per_sm >= (R.np > 304 ? 2 : 1) && want == 2; --per_sm)
+          for (int ns : {8, 6, 4}) {
+            rd.pipe_slots = ns;
+            const size_t need = (cp->mixed ? ras_factor_smem<float>(rd, 4) : ras_factor_smem<double>(rd, 4)) + 1024;
+            if (need <= FACTOR_SMEM_MAX / per_sm) {
+              want = 4;
+              break;
+            }
+          }
+      }
       rd.factor_mode = want;
       if (fits(2) && !fits(want)) throw StatusError{FSI_ERR_ARG, "factor_mode needs more shared memory than fits"};
       if (!fits(2)) {
@@ -900,7 +917,16 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
                       rd.max_row_blocks);
         throw StatusError{FSI_ERR_ARG, msg};
       }
-
+      if (want == 4) {
+        rd.ent_k = cp->upload(FP.ent_k);
+        rd.ent_len = cp->upload(FP.ent_len);
+        rd.meta_off = cp->upload(FP.meta_off);
+        rd.meta = cp->upload(FP.meta);
+      } else {
+        rd.upd_ptr = cp->upload(R.upd_ptr);
+        rd.upd_tgt = cp->upload(R.upd_tgt);
+        rd.upd_src = cp->upload(R.upd_src);
+      }
     }
     cp->ras = rd;
     // the Jacobian is assembled in chunks of tets so that Ke needs no more than
@@ -911,7 +937,8 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       const int64_t room = std::max<int64_t>(fac_bytes, (int64_t)1 << 30);
       cp->ke_tets = std::max<int64_t>(1, std::min<int64_t>(T0, room / per_tet));
       if (o.jac_chunk > 0) cp->ke_tets = std::min<int64_t>(T0, o.jac_chunk);
-      cp->fac = cp->dalloc<char>(std::max<int64_t>(fac_bytes, per_tet * cp->ke_tets));
+      // (+ 16: the pipelined factorisation copies whole 16-byte units)
+      cp->fac = cp->dalloc<char>(std::max<int64_t>(fac_bytes, per_tet * cp->ke_tets) + 16);
       cp->Ke = cp->fac;
     }
     cp->work = cp->dalloc<char>((int64_t)(7 * vs) * (int64_t)R.gnode.size());

@@ -90,7 +90,16 @@ struct RasDev {
   int32_t max_row_lent;    // most L blocks in one row
   int32_t max_row_upd;     // most elimination updates in one row
   int32_t max_entry_upd;   // most updates of one L block
-  int32_t factor_mode;     // factorisation kernel: 0..2 rows in order (shared-memory modes), 3 nested-dissection groups
+  int32_t factor_mode;     // factorisation kernel: 0..2 rows in order (shared-memory modes), 3 nested-dissection groups,
+                           // 4 rows in order, pipelined
+  // pipelined factorisation (setup.h, FactorPipe)
+  const int32_t* ent_k;
+  const int32_t* ent_len;
+  const int64_t* meta_off;
+  const uint32_t* meta;
+  int32_t pipe_slots;      // L blocks in flight
+  int32_t pipe_meta;       // bytes of a slot's word list
+  int32_t pipe_data;       // bytes of a slot's blocks
   const int32_t* sd_depth; // [np] nested-dissection depth of each subdomain (0: one item)
   const int64_t* sd_item;  // [np+1] first item of each subdomain
   const int64_t* item_row; // [items] end row of each item (subdomain-relative)
@@ -101,7 +110,10 @@ void launch_ras_extract(const RasDev& r, const TJ* vals, TF* fac, cudaStream_t s
 template <class TF>
 void launch_ras_factor(const RasDev& r, TF* fac, int32_t* err, cudaStream_t s);
 template <class TF>
-bool ras_factor_fits(const RasDev& r, int mode);  // mode 0..3 fits one CTA
+bool ras_factor_fits(const RasDev& r, int mode);  // mode 0..4 fits one CTA
+// shared memory of the factorisation CTA
+template <class TF>
+size_t ras_factor_smem(const RasDev& r, int mode);
 // shared-memory limit of the factorisation CTA (the opt-in maximum)
 constexpr size_t FACTOR_SMEM_MAX = 227 * 1024;
 template <class TF>

@@ -623,4 +623,38 @@ StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t sta
   return S;
 }
 
+FactorPipe build_factor_pipe(const RasPlan& R, int64_t cap, int64_t value_bytes) {
+  FactorPipe F;
+  const int64_t nL = (int64_t)R.lent_pos.size();
+  const int64_t V = 16 / value_bytes;
+  F.ent_k.resize(nL);
+  F.ent_len.resize(nL);
+  F.meta_off.assign(nL + 1, 0);
+  for (int64_t e = 0; e < nL; ++e)
+    F.meta_off[e + 1] = F.meta_off[e] + (R.upd_ptr[e + 1] - R.upd_ptr[e] + 2 + 3) / 4;
+  F.meta.assign(4 * F.meta_off[nL], 0);
+  int64_t ml = 1, mm = 1;
+#pragma omp parallel for schedule(dynamic, 4) reduction(max : ml, mm)
+  for (int32_t s = 0; s < R.np; ++s)
+    for (int64_t q = R.sd_row[s]; q < R.sd_row[s + 1]; ++q)
+      for (int64_t e = R.lent_ptr[q]; e < R.lent_ptr[q + 1]; ++e) {
+        const int64_t k = R.col[R.lent_pos[e]], kd = R.lent_kdiag[e];
+        uint32_t* w = F.meta.data() + 4 * F.meta_off[e];
+        int64_t len = 1, n = 0;
+        for (int64_t u = R.upd_ptr[e]; u < R.upd_ptr[e + 1]; ++u, ++n) {
+          w[2 + n] = (uint32_t)(R.upd_tgt[u] - R.row_ptr[q]) << 16 | (uint32_t)(R.upd_src[u] - kd);
+          len = std::max(len, R.upd_src[u] - kd + 1);
+        }
+        const uint32_t kind = k == q - 1 ? PIPE_PREV : (len > cap ? PIPE_DIRECT : 0);
+        w[0] = (uint32_t)n | (uint32_t)((49 * kd) % V) << 16 | kind << 28;
+        F.ent_k[e] = (int32_t)(k - R.sd_row[s]);
+        F.ent_len[e] = kind ? 0 : (int32_t)len;
+        ml = std::max(ml, (int64_t)F.ent_len[e]);
+        mm = std::max(mm, F.meta_off[e + 1] - F.meta_off[e]);
+      }
+  F.max_len = ml;
+  F.max_meta = mm;
+  return F;
+}
+
 }  // namespace fsi

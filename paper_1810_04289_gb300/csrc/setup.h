@@ -119,4 +119,22 @@ constexpr uint32_t ENTRY_PIECE = 16, ENTRY_ROW = 32, ENTRY_STAGE = 64, ENTRY_NON
 constexpr int64_t STAGE_MOST = 255;  // a stage's blocks are kept in a byte
 StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage);
 
+// What the pipelined factorisation (sparse.cu, k_ras_factor_pipe) copies to shared
+// memory ahead of each L block (i,k), in elimination order: a word list
+//   [ updates | shift << 16 | kind << 28, 0, then per update target << 16 | source ]
+// padded to 16 bytes (target: block of row i; source: block after the pivot of row
+// k), and the blocks of row k from its pivot to the last source. kind 0: copied;
+// PIPE_PREV: k is the row before i, which is still in shared memory; PIPE_DIRECT:
+// more than `cap` blocks, read from global memory. shift: values between the copy's
+// 16-byte aligned start and the pivot.
+struct FactorPipe {
+  std::vector<int32_t> ent_k;      // [nL] subdomain-relative row k
+  std::vector<int32_t> ent_len;    // [nL] blocks copied (0: kind is not 0)
+  std::vector<int64_t> meta_off;   // [nL+1] first 16-byte unit of the word list
+  std::vector<uint32_t> meta;
+  int64_t max_len = 1, max_meta = 1;  // most blocks copied; most 16-byte units of a list
+};
+constexpr uint32_t PIPE_PREV = 1, PIPE_DIRECT = 2;
+FactorPipe build_factor_pipe(const RasPlan& R, int64_t cap, int64_t value_bytes);
+
 }  // namespace fsi

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.cuh"
+#include "setup.h"
 
 namespace fsi {
 
@@ -261,6 +262,336 @@ __global__ void __launch_bounds__(256) k_ras_factor_cta(RasDev R, TF* __restrict
   }
 }
 
+// 1 / x, correctly rounded (what the division gives), without its call
+__device__ __forceinline__ float rcp_rn(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
+
+// In-place inverse of the 7x7 block B by one warp, the same arithmetic as
+// warp_invert7 with a column of [B | I] in each lane's registers (lanes 0..13).
+template <class TF>
+__device__ __forceinline__ void warp_invert7_regs(TF* B, int32_t* err) {
+  const int lane = threadIdx.x & 31;
+  TF a[7];
+#pragma unroll
+  for (int r = 0; r < 7; ++r) a[r] = lane < 7 ? B[7 * r + lane] : (lane - 7 == r ? TF(1) : TF(0));
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    int piv = k;
+    TF best = fabs(a[k]);
+#pragma unroll
+    for (int r = k + 1; r < 7; ++r) {
+      const TF v = fabs(a[r]);
+      if (v > best) {
+        best = v;
+        piv = r;
+      }
+    }
+    if (lane == k && !(best > tiny_pivot<TF>())) atomicExch(err, 1);
+    piv = __shfl_sync(0xffffffffu, piv, k);
+    const TF ak = a[k];
+#pragma unroll
+    for (int r = k + 1; r < 7; ++r)
+      if (r == piv) {
+        a[k] = a[r];
+        a[r] = ak;
+      }
+    const TF inv = rcp_rn(__shfl_sync(0xffffffffu, a[k], k));
+    a[k] *= inv;
+#pragma unroll
+    for (int r = 0; r < 7; ++r)
+      if (r != k) {
+        const TF f = __shfl_sync(0xffffffffu, a[r], k);
+        a[r] -= f * a[k];
+      }
+  }
+  if (lane >= 7 && lane < 14) {
+#pragma unroll
+    for (int r = 0; r < 7; ++r) B[7 * r + lane - 7] = a[r];
+  }
+}
+
+__device__ __forceinline__ void pipe_bar_init(uint64_t* b, uint32_t n) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(n)
+               : "memory");
+}
+__device__ __forceinline__ void pipe_bar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
+}
+// bounded wait: false if the phase did not complete in time
+__device__ __forceinline__ bool pipe_bar_wait(uint64_t* b, uint32_t parity) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(b);
+  for (uint32_t it = 0; it < (1u << 20); ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// Pipelined block ILU, one CTA per subdomain, rows in order: the arithmetic of
+// k_ras_factor_cta in its order (same bits). That kernel is bound by latency: for
+// every L block it reads index lists, the pivot, the update lists and the source
+// blocks from L2, one after the other, between two barriers. Here
+//   - a producer warp copies what each L block needs (the host's word list and row
+//     k's blocks from the pivot on) into a ring of slots, up to 8 L blocks ahead and
+//     across rows, as soon as row k is finished; the row before stays in shared memory;
+//   - the pivot of a row is inverted by a warp of its own, in registers, beside the
+//     next row's elimination, which needs it last;
+//   - the row's own values are read a row ahead; FP32 has one barrier per L block
+//     (every warp forms A_ik D_k^{-1} for itself) and a thread takes a column of a
+//     target block with A_ik D_k^{-1} in registers (57 loads per 343 products; one
+//     element per thread took 15 instructions per product).
+// Measured, us: FP32 14,350-node tube, 64 subdomains, ILU(1) 12,850 -> 4,420; 6-tube
+// batch, 255 subdomains, ILU(2) 8,050 -> 3,460; 174k-node tree, 1,088 subdomains, ILU(2)
+// 23,750 -> 17,400; FP64 429-node tube, 4 subdomains 7,960 -> 3,130, 14,350-node tube
+// 30,870 -> 12,340 (FP64 pipe). The slots must leave two CTAs per SM (one up to 304
+// subdomains: 46,657-node tube, FP64, 512 subdomains, one CTA 25,000, the kernel
+// above 20,300).
+// threads that eliminate (then one producer warp and one warp that inverts the
+// pivots). FP32: a thread updates a whole column of a target block; FP64: an element
+constexpr int PIPE_HEAD = 160;         // barriers and the row counter
+constexpr int PIPE_SCL = 4 * 56 * 4;  // bytes of the scaled L blocks
+template <class TF> constexpr int PIPE_THREADS = sizeof(TF) == 4 ? 128 : 256;
+
+template <class TF>
+__global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2) k_ras_factor_pipe(RasDev R, TF* fac, int32_t* err) {
+  constexpr bool F32 = sizeof(TF) == 4;
+  constexpr int NT = PIPE_THREADS<TF>, MAXSLOT = 8, PF = F32 ? 12 : 8;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(fsm);        // [MAXSLOT]
+  uint64_t* empty = full + MAXSLOT;                         // [MAXSLOT]
+  uint64_t* inv = empty + MAXSLOT;                          // a row's pivot is inverted
+  volatile int* done = reinterpret_cast<volatile int*>(inv + 1);  // rows finished and stored
+  TF* sScl = reinterpret_cast<TF*>(fsm + PIPE_HEAD);              // FP32 [4][56], rows of 8; FP64 [49]
+  const int NS = R.pipe_slots;
+  const uint32_t slot_bytes = R.pipe_meta + R.pipe_data;
+  unsigned char* slots = fsm + PIPE_HEAD + PIPE_SCL;
+  TF* sRow = reinterpret_cast<TF*>(slots + NS * slot_bytes);  // [2][max_row_blocks * 49]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int s = blockIdx.x;
+  const int64_t qb = R.sd_row[s], qe = R.sd_row[s + 1];
+  if (tid == 0) {
+    for (int i = 0; i < NS; ++i) {
+      pipe_bar_init(&full[i], 32);
+      pipe_bar_init(&empty[i], 1);
+    }
+    pipe_bar_init(inv, 1);
+    *done = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  bool ok = true;
+  int slot = 0, phase = 0;
+  auto next_slot = [&]() {
+    if (++slot == NS) {
+      slot = 0;
+      phase ^= 1;
+    }
+  };
+
+  if (w == NT / 32) {
+    // producer warp: for every L block in elimination order, its word list and row k's
+    // blocks into the next free slot, once row k is finished
+    const int64_t e0 = R.lent_ptr[qb], e1 = R.lent_ptr[qe];
+    int fin = 0, issued = 0;
+    for (int64_t eb = e0; eb < e1 && ok; eb += 32) {
+      const int64_t em = eb + lane < e1 ? eb + lane : e1 - 1;
+      const int mk = R.ent_k[em], ml = R.ent_len[em];
+      const int64_t mkd = R.lent_kdiag[em], mo = R.meta_off[em];
+      const int mn = (int)(R.meta_off[em + 1] - mo);
+      const int cnt = (int)(e1 - eb < 32 ? e1 - eb : 32);
+      for (int i = 0; i < cnt && ok; ++i) {
+        const int k = __shfl_sync(0xffffffffu, mk, i), len = __shfl_sync(0xffffffffu, ml, i);
+        const int n16 = __shfl_sync(0xffffffffu, mn, i);
+        const int64_t kd = __shfl_sync(0xffffffffu, mkd, i), off = __shfl_sync(0xffffffffu, mo, i);
+        if (issued >= NS) ok = pipe_bar_wait(&empty[slot], (uint32_t)(phase ^ 1));
+        if (len > 0 && fin <= k) {
+          for (uint32_t it = 0; it < (1u << 24) && (fin = *done) <= k; ++it) __nanosleep(20);
+          ok = ok && fin > k;
+          __threadfence_block();
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        unsigned char* d = slots + slot * slot_bytes;
+        const unsigned char* ms = reinterpret_cast<const unsigned char*>(R.meta) + 16 * off;
+        for (int x = lane; x < n16; x += 32) cp_async16(d + 16 * x, ms + 16 * x);
+        if (len > 0) {
+          const int64_t b0 = 49 * kd * (int64_t)sizeof(TF), a0 = b0 & ~(int64_t)15;
+          const int n = (int)((49 * (kd + len) * (int64_t)sizeof(TF) - a0 + 15) >> 4);
+          const unsigned char* ds = reinterpret_cast<const unsigned char*>(fac) + a0;
+          for (int x = lane; x < n; x += 32) cp_async16(d + R.pipe_meta + 16 * x, ds + 16 * x);
+        }
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&full[slot]))
+                     : "memory");
+        ++issued;
+        next_slot();
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok && lane == 0) atomicExch(err, 2);
+    return;
+  }
+
+  if (w == NT / 32 + 1) {
+    // inverts each row's pivot when its updates are done (named barrier 2), beside the
+    // next row's elimination
+    for (int64_t q = qb; q < qe; ++q) {
+      asm volatile("bar.sync 2, %0;" ::"n"(NT + 32) : "memory");
+      TF* B = sRow + (q & 1) * 49 * R.max_row_blocks + 49 * (int)(R.diag[q] - R.row_ptr[q]);
+      warp_invert7_regs<TF>(B, err);
+      __syncwarp();
+      TF* out = fac + 49 * R.diag[q];
+      for (int x = lane; x < 49; x += 32) out[x] = B[x];
+      __threadfence_block();
+      __syncwarp();
+      if (lane == 0) {
+        *done = (int)(q - qb) + 1;  // (the row's other blocks were stored before barrier 2)
+        pipe_bar_arrive(inv);
+      }
+    }
+    return;
+  }
+
+  auto bar = []() { asm volatile("bar.sync 1, %0;" ::"n"(PIPE_THREADS<TF>) : "memory"); };
+  // the row's values a row ahead in registers, its offsets two rows ahead
+  int64_t rp = R.row_ptr[qb], rp1 = R.row_ptr[qb + 1], rp2 = R.row_ptr[qb + 1 < qe ? qb + 2 : qb + 1];
+  int64_t lp = R.lent_ptr[qb], lp1 = R.lent_ptr[qb + 1];
+  TF pre[PF];
+#pragma unroll
+  for (int i = 0; i < PF; ++i) {
+    const int64_t x = 49 * rp + tid + NT * i;
+    pre[i] = x < 49 * rp1 ? fac[x] : TF(0);
+  }
+  // FP32: elements lane, lane + 32 of the scaled block
+  const int r0 = lane / 7, c0 = lane - 7 * r0, r1 = (lane + 32) / 7, c1 = lane + 32 - 7 * r1;
+  int nl_prev = 0;
+  for (int64_t q = qb; q < qe; ++q) {
+    const int nv = 49 * (int)(rp1 - rp), nl = (int)(lp1 - lp);
+    TF* row = sRow + (q & 1) * 49 * R.max_row_blocks;
+    const TF* prow = sRow + ((q & 1) ^ 1) * 49 * R.max_row_blocks + 49 * nl_prev;  // previous row, from its pivot on
+#pragma unroll
+    for (int i = 0; i < PF; ++i)
+      if (tid + NT * i < nv) row[tid + NT * i] = pre[i];
+    for (int x = tid + NT * PF; x < nv; x += NT) row[x] = fac[49 * rp + x];
+    const int64_t rp3 = R.row_ptr[q + 3 <= qe ? q + 3 : qe], lp2 = R.lent_ptr[q + 2 <= qe ? q + 2 : qe];
+#pragma unroll
+    for (int i = 0; i < PF; ++i) {
+      const int64_t x = 49 * rp1 + tid + NT * i;
+      pre[i] = q + 1 < qe && x < 49 * rp2 ? fac[x] : TF(0);
+    }
+    bar();
+    bool inverted = q == qb;  // the previous row's pivot
+    auto wait_inverse = [&]() {
+      if (!inverted && ok) ok = pipe_bar_wait(inv, (uint32_t)((q - qb - 1) & 1));
+      inverted = true;
+    };
+    for (int e = 0; e < nl; ++e) {
+      if (ok) ok = pipe_bar_wait(&full[slot], (uint32_t)phase);
+      const uint32_t* meta = reinterpret_cast<const uint32_t*>(slots + slot * slot_bytes);
+      const uint32_t head = ok ? meta[0] : 0;
+      const int ne = (int)(head & 0xffff);
+      const uint32_t kind = head >> 28;
+      if (kind == PIPE_PREV) wait_inverse();
+      // A_ik D_k^{-1}: FP32 in every warp for itself (one barrier per L block), FP64 once
+      auto both = [&](const TF* D) {
+        const TF* A = row + 49 * e;
+        if constexpr (F32) {
+          TF* scl = sScl + 56 * w;
+          if (ok) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int x = lane + 32 * h;
+              if (x < 49) {
+                const int r = h ? r1 : r0, c = h ? c1 : c0;
+                TF v = TF(0);
+#pragma unroll
+                for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
+                scl[8 * r + c] = v;
+                if (w == 0) fac[49 * (rp + e) + x] = v;
+              }
+            }
+          }
+          __syncwarp();
+          if (ok && tid < 7 * ne) {
+            float4 sv[14];  // the scaled block, rows of 8
+#pragma unroll
+            for (int i = 0; i < 14; ++i) sv[i] = *reinterpret_cast<const float4*>(scl + 4 * i);
+            const TF* sc = reinterpret_cast<const TF*>(sv);
+            for (int x = tid; x < 7 * ne; x += NT) {
+              const int u = x / 7, c = x - 7 * u;
+              const uint32_t ts = meta[2 + u];
+              TF* T = row + 49 * (ts >> 16) + c;
+              const TF* S = D + 49 * (ts & 0xffff) + c;
+              TF col[7], acc[7];
+#pragma unroll
+              for (int mm = 0; mm < 7; ++mm) col[mm] = S[7 * mm], acc[mm] = T[7 * mm];
+#pragma unroll
+              for (int mm = 0; mm < 7; ++mm)
+#pragma unroll
+                for (int r = 0; r < 7; ++r) acc[r] -= sc[8 * r + mm] * col[mm];
+#pragma unroll
+              for (int r = 0; r < 7; ++r) T[7 * r] = acc[r];
+            }
+          }
+        } else {
+          if (ok && tid < 49) {
+            const int r = tid / 7, c = tid - 7 * r;
+            TF v = TF(0);
+#pragma unroll
+            for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
+            sScl[tid] = v;
+            fac[49 * (rp + e) + tid] = v;
+          }
+          bar();
+          if (ok)
+            for (int x = tid; x < 49 * ne; x += NT) {
+              const int u = x / 49, el = x - 49 * u;
+              const int r = el / 7, c = el - 7 * r;
+              const uint32_t ts = meta[2 + u];
+              TF* T = row + 49 * (ts >> 16) + el;
+              const TF* S = D + 49 * (ts & 0xffff) + c;
+              TF acc = *T;
+#pragma unroll
+              for (int mm = 0; mm < 7; ++mm) acc -= sScl[7 * r + mm] * S[7 * mm];
+              *T = acc;
+            }
+        }
+      };
+      if (kind == PIPE_DIRECT)
+        both(fac + 49 * R.lent_kdiag[lp + e]);
+      else
+        both(kind == PIPE_PREV ? prow
+                               : reinterpret_cast<const TF*>(slots + slot * slot_bytes + R.pipe_meta) +
+                                     ((head >> 16) & 15));
+      bar();
+      if (tid == 0) pipe_bar_arrive(&empty[slot]);
+      next_slot();
+    }
+    // the pivot goes to the inverting warp, the blocks after it to global memory; the other
+    // row buffer may be overwritten once the previous pivot has left it
+    for (int x = 49 * (nl + 1) + tid; x < nv; x += NT) fac[49 * rp + x] = row[x];
+    wait_inverse();
+    __threadfence_block();
+    asm volatile("bar.arrive 2, %0;" ::"n"(NT + 32) : "memory");
+    nl_prev = nl;
+    rp = rp1;
+    rp1 = rp2;
+    rp2 = rp3;
+    lp = lp1;
+    lp1 = lp2;
+  }
+  if (!ok && lane == 0) atomicExch(err, 2);
+}
+
 // Block ILU on nested-dissection ordered subdomains: the CTA's 256 threads
 // form G = 2^D groups (D the subdomain's dissection depth); in each phase (the
 // leaves, then the separators level by level) every item of the phase is
@@ -447,7 +778,10 @@ void launch_ras_extract(const RasDev& r, const TJ* vals, TF* fac, cudaStream_t s
 }
 
 template <class TF>
-size_t ras_factor_cta_smem(const RasDev& r, int mode) {
+size_t ras_factor_smem(const RasDev& r, int mode) {
+  if (mode == 4)
+    return PIPE_HEAD + PIPE_SCL + (size_t)r.pipe_slots * (r.pipe_meta + r.pipe_data) +
+           (size_t)2 * r.max_row_blocks * 49 * sizeof(TF);
   if (mode == 3)  // one row, scaled block and inversion scratch per group
     return ((size_t)1 << r.max_depth) * (((size_t)r.max_row_blocks + 1) * 49 + 98) * sizeof(TF);
   size_t blocks = (size_t)r.max_row_blocks + 1;  // the row and the scaled L block
@@ -462,7 +796,7 @@ size_t ras_factor_cta_smem(const RasDev& r, int mode) {
 // source reads better than prefetching them does.
 template <class TF>
 bool ras_factor_fits(const RasDev& r, int mode) {
-  return ras_factor_cta_smem<TF>(r, mode) <= FACTOR_SMEM_MAX;
+  return ras_factor_smem<TF>(r, mode) <= FACTOR_SMEM_MAX;
 }
 
 template <class TF, int MODE>
@@ -475,7 +809,7 @@ void launch_factor_mode(const RasDev& r, TF* fac, int32_t* err, size_t smem, cud
 
 template <class TF>
 void launch_ras_factor(const RasDev& r, TF* fac, int32_t* err, cudaStream_t s) {
-  const size_t smem = ras_factor_cta_smem<TF>(r, r.factor_mode);
+  const size_t smem = ras_factor_smem<TF>(r, r.factor_mode);
   switch (r.factor_mode) {
     case 0: launch_factor_mode<TF, 0>(r, fac, err, smem, s); break;
     case 1: launch_factor_mode<TF, 1>(r, fac, err, smem, s); break;
@@ -486,10 +820,18 @@ void launch_ras_factor(const RasDev& r, TF* fac, int32_t* err, cudaStream_t s) {
       cudaFuncSetAttribute(k_ras_factor_nd<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       k_ras_factor_nd<TF><<<r.np, 256, smem, s>>>(r, fac, err);
       break;
+    case 4:
+      cudaFuncSetAttribute(k_ras_factor_pipe<TF>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           (int)cudaSharedmemCarveoutMaxShared);
+      cudaFuncSetAttribute(k_ras_factor_pipe<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k_ras_factor_pipe<TF><<<r.np, PIPE_THREADS<TF> + 64, smem, s>>>(r, fac, err);
+      break;
     default: break;  // fsi_create rejects such plans
   }
 }
 
+template size_t ras_factor_smem<float>(const RasDev&, int);
+template size_t ras_factor_smem<double>(const RasDev&, int);
 template bool ras_factor_fits<float>(const RasDev&, int);
 template bool ras_factor_fits<double>(const RasDev&, int);
 

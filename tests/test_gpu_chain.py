@@ -43,7 +43,7 @@ def apply(case, precision, mode, **opt):
     fsi.fsi_pc_apply(S.ctx, S.vec(r), z)
     out, kind = z.cpu().numpy(), S.info().apply_kernel
     S.close()
-    assert kind == (2 if mode == 2 else 1)
+    assert mode == 0 or kind == mode
     return out
 
 
@@ -60,6 +60,15 @@ def test_chain_and_team_match_the_level_scheduled_kernel(case, nsub, ilu, orderi
     assert all(v <= 1e-10 for v in d64.values()), d64
     level, chain = far(apply(case, 1, 2, **opt), ref), far(apply(case, 1, 1, **opt), ref)
     assert all(chain[g] <= 2 * level[g] + 1e-6 for g in GROUPS), (chain, level)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nsub,ilu,ordering", [(1, 0, 0), (1, 3, 1), (4, 1, 2), (64, 2, 1), (305, 1, 1), (900, 2, 0)])
+def test_pipelined_factors_are_the_row_kernels_bits(case, precision, nsub, ilu, ordering):
+    """factor_mode 0 (pipelined) does factor_mode 3's arithmetic in its order."""
+    opt = dict(n_subdomains=nsub, ilu_level=ilu, ordering=ordering)
+    a, b = (apply(case, precision, 0, factor_mode=k, **opt) for k in (0, 3))
+    assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("precision,nsub", [(0, 500), (1, 500), (1, 8)])
