@@ -100,8 +100,6 @@ struct fsi_ctx {
   int* reorth = nullptr;         // [1] some problem needs a second Gram-Schmidt pass (orth = 1), or
                                  // its new norm from the updated vector (orth = 0 fallback)
   double* gs_inv = nullptr;      // [P] reciprocal of H[j+1][j] (orth 0)
-  double* gs_nrm = nullptr;      // [P] norms formed from the updated vector (its fallback)
-  double* gs_scal = nullptr;     // [P] their divisors
   int* gs_unsafe = nullptr;      // [P] the norm is taken from the updated vector
   int* pmask = nullptr;          // [P] problem already converged (Newton)
   double* palpha = nullptr;      // [P] line-search step per problem
@@ -278,10 +276,10 @@ void spmv_on(fsi_ctx* c, const double* x, const float* x32, double* y, const int
       launch_to_float(c->n, x, c->zf, guard, st);
       x32 = c->zf;
     }
-    launch_bsr_spmv<float, float>(c->N, c->row_ptr, c->col, (const float*)c->vals, x32, y, c->opt.threads_per_row,
+    launch_bsr_spmv<float>(c->N, c->row_ptr, c->col, (const float*)c->vals, x32, y, c->opt.threads_per_row,
                                   guard, st);
   } else {
-    launch_bsr_spmv<double, double>(c->N, c->row_ptr, c->col, (const double*)c->vals, x, y, c->opt.threads_per_row,
+    launch_bsr_spmv<double>(c->N, c->row_ptr, c->col, (const double*)c->vals, x, y, c->opt.threads_per_row,
                                     guard, st);
   }
   c->launches += 1;
@@ -381,12 +379,10 @@ void arnoldi_step(fsi_ctx* c, int32_t j, const int* guard, cudaStream_t st) {
     launch_seg_norm_pythagoras(P, c->hB, ldh, j, hj, (int64_t)ldh * m, c->gs_inv, c->gs_unsafe, c->reorth,
                                c->opt.fault_test == 2 ? 1 : 0, guard, st);
     launch_seg_maxpy(c->seg, n, j + 1, c->V, n, c->hB, ldh, w, guard, st, c->gs_inv);
-    launch_seg_norm(c->seg, w, c->partial, c->gs_nrm, 1, c->reorth, st);
-    launch_seg_norm_fix(P, c->gs_nrm, c->gs_unsafe, hj, (int64_t)ldh * m, c->gs_scal, c->reorth, st);
-    launch_seg_scale_inv(c->seg, n, w, c->gs_scal, 1, w, c->reorth, st);
+    launch_seg_norm_fallback(c->seg, w, c->gs_unsafe, hj, (int64_t)ldh * m, c->reorth, st);
     launch_seg_givens(P, c->hA, c->hB, ldh, c->H, ldh, m, j, c->cs, c->sn, c->g, c->gres, c->gtarget, c->active,
                       c->kcols, c->anyact, st);
-    c->launches += 7 + nk;
+    c->launches += 5 + nk;
     return;
   }
   // orth 2: dots, update, dots, update, norm, scale
@@ -810,7 +806,10 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     cp->hB = cp->dalloc<double>(NP * (m + 1));
     // reduction chunks: each problem's dofs cut into chunks of at most CH dofs
     {
-      const int64_t CH = std::max<int64_t>(1024, (7 * N + 1215) / 1216);
+      // as many as keep the SMs busy: about two blocks per SM on small vectors (256 to 1,024 dofs
+      // each), 1,216 on large ones
+      const int64_t CH = std::max(std::min<int64_t>(1024, std::max<int64_t>(256, (7 * N + 303) / 304)),
+                                  (7 * N + 1215) / 1216);
       std::vector<int64_t> cb{0}, pc{0};
       std::vector<int64_t> pstart(NP + 1, 0);
       for (int64_t i = 0; i < N; ++i) pstart[prob[i] + 1]++;
@@ -836,8 +835,6 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     cp->anyact = cp->dalloc<int>(1);
     cp->reorth = cp->dalloc<int>(1);
     cp->gs_inv = cp->dalloc<double>(n_problems);
-    cp->gs_nrm = cp->dalloc<double>(n_problems);
-    cp->gs_scal = cp->dalloc<double>(n_problems);
     cp->gs_unsafe = cp->dalloc<int>(n_problems);
     cp->pmask = cp->dalloc<int>(n_problems);
     cp->palpha = cp->dalloc<double>(n_problems);

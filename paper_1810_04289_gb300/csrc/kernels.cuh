@@ -59,8 +59,8 @@ void launch_constraint_jacobian(const MeshDev& m, const MatConst& mc, const int3
 // ---- sparse (sparse.cu)
 // y = J x; threads_per_row 32 (one warp per block row) or 16 (two rows per
 // warp); guard: optional device flag, the kernel does nothing while *guard == 0
-template <class TV, class TX>
-void launch_bsr_spmv(int64_t n, const int64_t* row_ptr, const int32_t* col, const TV* vals, const TX* x,
+template <class TV>
+void launch_bsr_spmv(int64_t n, const int64_t* row_ptr, const int32_t* col, const TV* vals, const TV* x,
                      double* y, int threads_per_row, const int* guard, cudaStream_t s);
 void launch_to_float(int64_t n, const double* x, float* y, const int* guard, cudaStream_t s);
 
@@ -193,8 +193,10 @@ void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, 
 // the new Arnoldi vector's norm as sqrt(||w||^2 - ||h2||^2) where that is safe (see krylov.cu)
 void launch_seg_norm_pythagoras(int32_t P, const double* hb, int32_t lda, int32_t j, double* hsub, int64_t ldsub,
                                 double* inv, int* unsafe, int* flag, int force, const int* guard, cudaStream_t s);
-void launch_seg_norm_fix(int32_t P, const double* nrm, const int* unsafe, double* hsub, int64_t ldsub, double* scal,
-                         const int* guard, cudaStream_t s);
+// where *guard says so: the norms of the problems with unsafe[p] formed from w itself into
+// hsub, and w divided by them
+void launch_seg_norm_fallback(const SegDev& sg, double* w, const int* unsafe, double* hsub,
+                              int64_t ldsub, const int* guard, cudaStream_t s);
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
                           double* y, const int* guard, cudaStream_t s);
 

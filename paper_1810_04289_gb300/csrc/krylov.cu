@@ -31,6 +31,27 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums of v[0..W) over the warp's lanes: every step halves the vectors a lane
+// still carries, so 8 vectors take 9 FP64 additions instead of 40 (the FP64 pipe
+// bounds the dots; the additions of a plain butterfly per vector cost as much as the
+// products: 8 vectors of 326k dofs 31 -> 22 us). Afterwards v[0] of the lanes with
+// lane / (32 / W) == k holds vector k's sum.
+template <int W>
+__device__ __forceinline__ void warp_sums(double (&v)[W]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int h = W / 2; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? v[i + h] : v[i], other = up ? v[i] : v[i + h];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+    }
+  }
+  for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+
 // out[p * ldo + k] = sum over the dofs of problem p of V_k . w (V null: w . w,
 // and take_sqrt gives the 2-norm). Block (c, y) forms the partials of chunk c
 // for the vectors of group g = g0 + y, 8g .. 8g + W - 1 (those below nv); the
@@ -78,18 +99,16 @@ __global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, int32_t 
         if (k0 + k < nv) acc[k] += v[u][k] * wv[u];
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < W; ++k) {
-    if (k0 + k < nv) {
-      const double v = warp_sum(acc[k]);
-      if (lane == 0) red[k][warp] = v;
-    }
-  }
+  warp_sums<W>(acc);
+  if (lane % (32 / W) == 0) red[lane / (32 / W)][warp] = acc[0];
   __syncthreads();
-  if (threadIdx.x < W && k0 + threadIdx.x < nv) {
-    double v = 0.0;
-    for (int q = 0; q < RB / 32; ++q) v += red[threadIdx.x][q];
-    partial[(int64_t)c * nv + k0 + threadIdx.x] = v;
+  // the 8 warps' sums of vector k: lanes 8 k .. 8 k + 7 of the first W / 4 (at least one) warps
+  if (threadIdx.x < (W < 4 ? 32 : 8 * W)) {
+    const int k = threadIdx.x >> 3;
+    double v = k < W ? red[k][threadIdx.x & 7] : 0.0;
+#pragma unroll
+    for (int o = 4; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (k < W && (threadIdx.x & 7) == 0 && k0 + k < nv) partial[(int64_t)c * nv + k0 + k] = v;
   }
   // publish the partials, then count this block in
   __threadfence();
@@ -156,7 +175,7 @@ __global__ void k_seg_scale_inv(SegDev sg, int64_t n, const double* __restrict__
 // the reciprocal (0 for a zero norm); elsewhere (only as a Krylov space is
 // exhausted; for every problem with force = 1, tests of that path) inv[p] = 1,
 // unsafe[p] = 1 and *flag = 1: the norm is then formed from the updated vector
-// by the guarded k_seg_norm_fix path.
+// by k_seg_norm_fallback.
 __global__ void k_seg_norm_pythagoras(int32_t P, const double* __restrict__ hb, int32_t lda, int32_t j,
                                       double* __restrict__ hsub, int64_t ldsub, double* __restrict__ inv,
                                       int* __restrict__ unsafe, int* __restrict__ flag, int force,
@@ -168,42 +187,53 @@ __global__ void k_seg_norm_pythagoras(int32_t P, const double* __restrict__ hb, 
   }
   if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+  // one warp per problem
+  for (int p = threadIdx.x >> 5; p < P; p += blockDim.x >> 5) {
+    const int lane = threadIdx.x & 31;
     const double* h = hb + (int64_t)p * lda;
     const double s = h[j + 1];
     double q = 0.0;
-    for (int k = 0; k <= j; ++k) q += h[k] * h[k];
-    const double b2 = s - q;
-    if (!force && b2 >= 0.75 * s) {
-      const double b = sqrt(b2);
-      hsub[(int64_t)p * ldsub] = b;
-      inv[p] = b > 0.0 ? 1.0 / b : 0.0;
-      unsafe[p] = 0;
-    } else {
-      inv[p] = 1.0;
-      unsafe[p] = 1;
-      atomicOr(&s_any, 1);
+    for (int k = lane; k <= j; k += 32) q += h[k] * h[k];
+    q = warp_sum(q);
+    if (lane == 0) {
+      const double b2 = s - q;
+      if (!force && b2 >= 0.75 * s) {
+        const double b = sqrt(b2);
+        hsub[(int64_t)p * ldsub] = b;
+        inv[p] = b > 0.0 ? 1.0 / b : 0.0;
+        unsafe[p] = 0;
+      } else {
+        inv[p] = 1.0;
+        unsafe[p] = 1;
+        atomicOr(&s_any, 1);
+      }
     }
   }
   __syncthreads();
   if (threadIdx.x == 0) *flag = s_any;
 }
 
-// the fallback of k_seg_norm_pythagoras, after nrm[p] = ||w_p|| of the updated
-// vector: H[p][j+1][j] = nrm[p] and scal[p] = nrm[p] where unsafe[p], scal[p] = 1
-// elsewhere (the vector is then divided by scal)
-__global__ void k_seg_norm_fix(int32_t P, const double* __restrict__ nrm, const int* __restrict__ unsafe,
-                               double* __restrict__ hsub, int64_t ldsub, double* __restrict__ scal,
-                               const int* guard) {
+// the fallback of k_seg_norm_pythagoras, one block per problem (a rare path: one
+// launch that mostly returns at once in place of three): where unsafe[p],
+// H[p][j+1][j] = ||w_p|| of the updated vector and w_p /= it (0 for a zero norm)
+__global__ void __launch_bounds__(1024) k_seg_norm_fallback(SegDev sg, double* __restrict__ w,
+                                                            const int* __restrict__ unsafe,
+                                                            double* __restrict__ hsub, int64_t ldsub,
+                                                            const int* guard) {
   if (off(guard)) return;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    if (unsafe[p]) {
-      hsub[(int64_t)p * ldsub] = nrm[p];
-      scal[p] = nrm[p];
-    } else {
-      scal[p] = 1.0;
-    }
-  }
+  const int p = blockIdx.x;
+  if (!unsafe[p]) return;
+  __shared__ double red[32];
+  const int64_t i0 = sg.chunk_beg[sg.prob_chunk[p]], i1 = sg.chunk_beg[sg.prob_chunk[p + 1]];
+  double s = 0.0;
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += w[i] * w[i];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = warp_sum(red[threadIdx.x & 31]);
+  const double nrm = sqrt(s), inv = nrm != 0.0 ? 1.0 / nrm : 0.0;
+  if (threadIdx.x == 0) hsub[(int64_t)p * ldsub] = nrm;
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] *= inv;
 }
 
 // start of a cycle for every problem: g = beta e_1, active while beta > target
@@ -251,65 +281,95 @@ __global__ void k_seg_reorth_decide(int32_t P, const double* __restrict__ ws, co
 // previous rotations, form the one that zeroes H[j+1][j], rotate g; |g[j+1]|
 // is that problem's GMRES residual. A problem stops at its target or when its
 // Krylov space is exhausted (H[j+1][j] = 0). *any = some problem still active.
-__global__ void k_seg_givens(int32_t P, const double* __restrict__ ha, const double* __restrict__ hb, int32_t lda,
-                             double* __restrict__ H, int32_t ldh, int32_t m, int32_t j,
-                             double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-                             double* __restrict__ res, const double* __restrict__ target, int* __restrict__ active,
-                             int* __restrict__ kcols, int* __restrict__ any) {
+// One warp per problem (up to 32 at a time): the lanes read the column's sums and the
+// rotations at once and hand them to the chain by shuffles (read one by one inside the
+// chain of rotations they cost an L2 latency each: 7.3 -> 5.9 us for one problem).
+__global__ void __launch_bounds__(1024) k_seg_givens(int32_t P, const double* __restrict__ ha,
+                                                     const double* __restrict__ hb, int32_t lda,
+                                                     double* __restrict__ H, int32_t ldh, int32_t m, int32_t j,
+                                                     double* __restrict__ cs, double* __restrict__ sn,
+                                                     double* __restrict__ g, double* __restrict__ res,
+                                                     const double* __restrict__ target, int* __restrict__ active,
+                                                     int* __restrict__ kcols, int* __restrict__ any) {
   __shared__ int s_any;
+  const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    if (active[p]) {
-      double* h = H + (int64_t)p * ldh * m + (int64_t)j * ldh;
-      for (int i = 0; i <= j; ++i) h[i] = ha[(int64_t)p * lda + i] + hb[(int64_t)p * lda + i];
-      double* c_ = cs + (int64_t)p * m;
-      double* s_ = sn + (int64_t)p * m;
-      double* gp = g + (int64_t)p * ldh;
-      const double sub = h[j + 1];
-      for (int i = 0; i < j; ++i) {
-        const double a = h[i], b = h[i + 1];
-        h[i] = c_[i] * a + s_[i] * b;
-        h[i + 1] = -s_[i] * a + c_[i] * b;
-      }
-      const double a = h[j], b = h[j + 1];
-      const double r = hypot(a, b);
-      double c = 1.0, sv = 0.0;
-      if (r > 0.0) {
-        c = a / r;
-        sv = b / r;
-      }
+  for (int p = threadIdx.x >> 5; p < P; p += blockDim.x >> 5) {
+    if (!active[p]) continue;
+    double* h = H + (int64_t)p * ldh * m + (int64_t)j * ldh;
+    double* c_ = cs + (int64_t)p * m;
+    double* s_ = sn + (int64_t)p * m;
+    double* gp = g + (int64_t)p * ldh;
+    // entries lane and lane + 32 (restart <= 64)
+    double hv[2], cv[2], sv[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int i = lane + 32 * t;
+      hv[t] = i <= j ? ha[(int64_t)p * lda + i] + hb[(int64_t)p * lda + i] : 0.0;
+      cv[t] = i < j ? c_[i] : 0.0;
+      sv[t] = i < j ? s_[i] : 0.0;
+    }
+    const double sub = h[j + 1], gj = gp[j], tg = target[p];
+    double a = __shfl_sync(0xffffffffu, hv[0], 0);
+    for (int i = 0; i < j; ++i) {
+      const double b = i + 1 < 32 ? __shfl_sync(0xffffffffu, hv[0], i + 1) : __shfl_sync(0xffffffffu, hv[1], i - 31);
+      const double c = i < 32 ? __shfl_sync(0xffffffffu, cv[0], i) : __shfl_sync(0xffffffffu, cv[1], i - 32);
+      const double s = i < 32 ? __shfl_sync(0xffffffffu, sv[0], i) : __shfl_sync(0xffffffffu, sv[1], i - 32);
+      const double hi = c * a + s * b;
+      a = -s * a + c * b;
+      if (lane == (i & 31)) (i < 32 ? hv[0] : hv[1]) = hi;
+    }
+    const double r = hypot(a, sub);
+    double c = 1.0, s = 0.0;
+    if (r > 0.0) {
+      c = a / r;
+      s = sub / r;
+    }
+    if (lane == (j & 31)) (j < 32 ? hv[0] : hv[1]) = r;
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      if (lane + 32 * t <= j) h[lane + 32 * t] = hv[t];
+    if (lane == 0) {
       c_[j] = c;
-      s_[j] = sv;
-      h[j] = r;
+      s_[j] = s;
       h[j + 1] = 0.0;
-      const double gj = gp[j];
       gp[j] = c * gj;
-      gp[j + 1] = -sv * gj;
-      const double rn = fabs(gp[j + 1]);
+      gp[j + 1] = -s * gj;
+      const double rn = fabs(s * gj);
       res[p] = rn;
       kcols[p] = j + 1;
-      if (!(rn > target[p]) || sub == 0.0) active[p] = 0;
+      if (!(rn > tg) || sub == 0.0) active[p] = 0;
+      else atomicOr(&s_any, 1);
     }
-    if (active[p]) atomicOr(&s_any, 1);
   }
   __syncthreads();
   if (threadIdx.x == 0) *any = s_any;
 }
 
-// y[p] = R_p^{-1} g[p] for each problem's kcols[p] x kcols[p] rotated Hessenberg
+// y[p] = R_p^{-1} g[p] for each problem's kcols[p] x kcols[p] rotated Hessenberg, one
+// warp per problem, column by column: lane i holds row i's right-hand side
 __global__ void k_seg_lsq(int32_t P, const double* __restrict__ H, int32_t ldh, int32_t m,
                           const int* __restrict__ kcols, const double* __restrict__ g, double* __restrict__ y) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < P; p += (gridDim.x * blockDim.x) >> 5) {
     const int k = kcols[p];
     const double* Hp = H + (int64_t)p * ldh * m;
-    const double* gp = g + (int64_t)p * ldh;
     double* yp = y + (int64_t)p * m;
-    for (int i = k - 1; i >= 0; --i) {
-      double s = gp[i];
-      for (int jj = i + 1; jj < k; ++jj) s -= Hp[(int64_t)jj * ldh + i] * yp[jj];
-      const double d = Hp[(int64_t)i * ldh + i];
-      yp[i] = d != 0.0 ? s / d : 0.0;
+    double r[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) r[t] = lane + 32 * t < k ? g[(int64_t)p * ldh + lane + 32 * t] : 0.0;
+    for (int jj = k - 1; jj >= 0; --jj) {
+      double c[2];  // column jj
+#pragma unroll
+      for (int t = 0; t < 2; ++t) c[t] = lane + 32 * t <= jj ? Hp[(int64_t)jj * ldh + lane + 32 * t] : 0.0;
+      const double d = jj < 32 ? __shfl_sync(0xffffffffu, c[0], jj) : __shfl_sync(0xffffffffu, c[1], jj - 32);
+      const double s = jj < 32 ? __shfl_sync(0xffffffffu, r[0], jj) : __shfl_sync(0xffffffffu, r[1], jj - 32);
+      const double v = d != 0.0 ? s / d : 0.0;
+      if (lane == 0) yp[jj] = v;
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (lane + 32 * t < jj) r[t] -= c[t] * v;
     }
   }
 }
@@ -408,12 +468,12 @@ void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, 
 
 void launch_seg_norm_pythagoras(int32_t P, const double* hb, int32_t lda, int32_t j, double* hsub, int64_t ldsub,
                                 double* inv, int* unsafe, int* flag, int force, const int* guard, cudaStream_t s) {
-  k_seg_norm_pythagoras<<<1, 256, 0, s>>>(P, hb, lda, j, hsub, ldsub, inv, unsafe, flag, force, guard);
+  k_seg_norm_pythagoras<<<1, 32 * (P < 32 ? P : 32), 0, s>>>(P, hb, lda, j, hsub, ldsub, inv, unsafe, flag, force, guard);
 }
 
-void launch_seg_norm_fix(int32_t P, const double* nrm, const int* unsafe, double* hsub, int64_t ldsub, double* scal,
-                         const int* guard, cudaStream_t s) {
-  k_seg_norm_fix<<<1, 256, 0, s>>>(P, nrm, unsafe, hsub, ldsub, scal, guard);
+void launch_seg_norm_fallback(const SegDev& sg, double* w, const int* unsafe, double* hsub, int64_t ldsub,
+                              const int* guard, cudaStream_t s) {
+  k_seg_norm_fallback<<<sg.P, 1024, 0, s>>>(sg, w, unsafe, hsub, ldsub, guard);
 }
 
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
@@ -429,12 +489,12 @@ void launch_seg_cycle_init(int32_t P, double* g, int32_t ldg, const double* beta
 void launch_seg_givens(int32_t P, const double* a, const double* b, int32_t lda, double* H, int32_t ldh, int32_t m,
                        int32_t j, double* cs, double* sn, double* g, double* res, const double* target, int* active,
                        int* kcols, int* any, cudaStream_t s) {
-  k_seg_givens<<<1, 256, 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res, target, active, kcols, any);
+  k_seg_givens<<<1, 32 * (P < 32 ? P : 32), 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res, target, active, kcols, any);
 }
 
 void launch_seg_lsq(int32_t P, const double* H, int32_t ldh, int32_t m, const int* kcols, const double* g, double* y,
                     cudaStream_t s) {
-  k_seg_lsq<<<(P + 63) / 64, 64, 0, s>>>(P, H, ldh, m, kcols, g, y);
+  k_seg_lsq<<<(P + 1) / 2, 64, 0, s>>>(P, H, ldh, m, kcols, g, y);
 }
 
 void launch_seg_update_x(const SegDev& sg, int64_t n, const double* Z, int64_t ldz, const double* y, int32_t m,

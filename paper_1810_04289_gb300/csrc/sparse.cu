@@ -6,6 +6,8 @@
 // prolongation used when the TMA-fed apply (ras_stream.cu) does not fit.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "setup.h"
 
@@ -20,19 +22,49 @@ inline int grid_for(int64_t work, int block) {
 }
 
 // ---------------------------------------------------------------------------
-// SpMV: one warp per block row. Lane l < 28 owns output component r = l / 4 and
-// every fourth block (q = l % 4) of the row; the four partial sums of a
-// component are combined by two shuffles. Lanes 28..31 idle. FP64: values,
-// vector and sums in FP64. Mixed: FP32 values and an FP32 copy of the vector;
-// each block's 7-term product is formed in FP32 and the block products are
-// accumulated in FP64 (one FP64 add per block and component), result in FP64.
+// SpMV: S block slots x 8 component lanes (7 used) per row, 32 / (8 S) rows per
+// warp; slot q takes every S-th block of the row, the partial sums of a component
+// are combined by shuffles. FP64: values, vector and sums in FP64, one fused
+// multiply-add per product (the FP64 pipe bounds this form: 4 warps of an SM issue one
+// FP64 instruction per 19 cycles; a tree sum per block took 10 instructions where the
+// chain takes 7: 103k-node tree 240 -> 159 us). Mixed: FP32 values and an FP32 copy
+// of the vector; each block's 7-term product is formed in FP32 and the block products
+// are summed in pairs of floats (two_sum: the rounding error of every addition is kept,
+// about 48 bits): a conversion and an FP64 addition per block product bounded the
+// kernel as much as memory did (174k-node tree 104 -> 98 us).
 // ---------------------------------------------------------------------------
-template <class TV, class TX, int S>
+struct SumFloat {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float t) {
+    const float s = __fadd_rn(hi, t), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(t, b)));
+    hi = s;
+  }
+  // (an infinite or NaN sum has no error term)
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  }
+};
+struct SumDouble {
+  double s = 0.0;
+  __device__ __forceinline__ double value() const { return s; }
+};
+__device__ __forceinline__ void add_product(SumFloat& acc, const float* A, const float* x) {
+  const float s0 = A[0] * x[0] + A[1] * x[1];
+  const float s1 = A[2] * x[2] + A[3] * x[3];
+  const float s2 = A[4] * x[4] + A[5] * x[5];
+  acc.add((s0 + s1) + (s2 + A[6] * x[6]));
+}
+__device__ __forceinline__ void add_product(SumDouble& acc, const double* A, const double* x) {
+#pragma unroll
+  for (int k = 0; k < 7; ++k) acc.s = fma(A[k], x[k], acc.s);
+}
+
+template <class TV, class SUM, int S>
 __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __restrict__ row_ptr,
                                                   const int32_t* __restrict__ col, const TV* __restrict__ vals,
-                                                  const TX* __restrict__ x, double* __restrict__ y,
+                                                  const TV* __restrict__ x, double* __restrict__ y,
                                                   const int* __restrict__ guard) {
-  // S block slots x 8 component lanes (7 used) per row; 32 / (8 S) rows per warp
   if (guard && *guard == 0) return;
   constexpr int G = 8 * S;
   const int lane = threadIdx.x & 31;
@@ -42,7 +74,7 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __re
   const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / G;
   for (int64_t base = grp0 - (lane / G); base < n; base += ngrp) {
     const int64_t row = base + (lane / G);
-    double acc = 0.0;
+    SUM sum;
     if (r < 7 && row < n) {
       const int64_t b0 = row_ptr[row], b1 = row_ptr[row + 1];
       // four of this lane's blocks per pass: their column indices first, then
@@ -52,18 +84,11 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __re
 #pragma unroll
         for (int u = 0; u < 4; ++u) cl[u] = b + u * S < b1 ? col[b + u * S] : -1;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (cl[u] >= 0) {
-            const TV* A = vals + 49 * (b + u * S) + 7 * r;
-            const TX* xb = x + 7 * (int64_t)cl[u];
-            TX s0 = TX(A[0]) * xb[0] + TX(A[1]) * xb[1];
-            TX s1 = TX(A[2]) * xb[2] + TX(A[3]) * xb[3];
-            TX s2 = TX(A[4]) * xb[4] + TX(A[5]) * xb[5];
-            acc += (double)((s0 + s1) + (s2 + TX(A[6]) * xb[6]));
-          }
-        }
+        for (int u = 0; u < 4; ++u)
+          if (cl[u] >= 0) add_product(sum, vals + 49 * (b + u * S) + 7 * r, x + 7 * (int64_t)cl[u]);
       }
     }
+    double acc = sum.value();
 #pragma unroll
     for (int o = 1; o < S; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (r < 7 && q == 0 && row < n) y[7 * row + r] = acc;
@@ -73,8 +98,16 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __re
 __global__ void k_to_float(int64_t n, const double* __restrict__ x, float* __restrict__ y,
                            const int* __restrict__ guard) {
   if (guard && *guard == 0) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = (float)x[i];
+  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {  // a caller's vector may start anywhere
+    for (int64_t i = i0; i < (n >> 1); i += st) {
+      const double2 v = reinterpret_cast<const double2*>(x)[i];
+      reinterpret_cast<float2*>(y)[i] = make_float2((float)v.x, (float)v.y);
+    }
+    if ((n & 1) && i0 == 0) y[n - 1] = (float)x[n - 1];
+  } else {
+    for (int64_t i = i0; i < n; i += st) y[i] = (float)x[i];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -759,17 +792,18 @@ __global__ void __launch_bounds__(256) k_ras_apply(RasDev R, const TF* __restric
 
 }  // namespace
 
-template <class TV, class TX>
-void launch_bsr_spmv(int64_t n, const int64_t* row_ptr, const int32_t* col, const TV* vals, const TX* x,
+template <class TV>
+void launch_bsr_spmv(int64_t n, const int64_t* row_ptr, const int32_t* col, const TV* vals, const TV* x,
                      double* y, int threads_per_row, const int* guard, cudaStream_t s) {
+  using SUM = std::conditional_t<sizeof(TV) == 4, SumFloat, SumDouble>;
   if (threads_per_row == 16)
-    k_bsr_spmv<TV, TX, 2><<<grid_for(16 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
+    k_bsr_spmv<TV, SUM, 2><<<grid_for(16 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
   else
-    k_bsr_spmv<TV, TX, 4><<<grid_for(32 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
+    k_bsr_spmv<TV, SUM, 4><<<grid_for(32 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
 }
 
 void launch_to_float(int64_t n, const double* x, float* y, const int* guard, cudaStream_t s) {
-  k_to_float<<<grid_for(n, 256), 256, 0, s>>>(n, x, y, guard);
+  k_to_float<<<grid_for((n + 1) / 2, 256), 256, 0, s>>>(n, x, y, guard);
 }
 
 template <class TF, class TJ>
@@ -841,10 +875,10 @@ void launch_ras_apply(const RasDev& r, const TF* fac, const double* rin, TF* wor
   k_ras_apply<TF><<<r.np, 256, 0, s>>>(r, fac, rin, work, z, z32, guard);
 }
 
-template void launch_bsr_spmv<double, double>(int64_t, const int64_t*, const int32_t*, const double*,
-                                              const double*, double*, int, const int*, cudaStream_t);
-template void launch_bsr_spmv<float, float>(int64_t, const int64_t*, const int32_t*, const float*, const float*,
-                                            double*, int, const int*, cudaStream_t);
+template void launch_bsr_spmv<double>(int64_t, const int64_t*, const int32_t*, const double*, const double*,
+                                      double*, int, const int*, cudaStream_t);
+template void launch_bsr_spmv<float>(int64_t, const int64_t*, const int32_t*, const float*, const float*, double*,
+                                     int, const int*, cudaStream_t);
 template void launch_ras_extract<double, double>(const RasDev&, const double*, double*, cudaStream_t);
 template void launch_ras_extract<float, float>(const RasDev&, const float*, float*, cudaStream_t);
 template void launch_ras_factor<double>(const RasDev&, double*, int32_t*, cudaStream_t);
