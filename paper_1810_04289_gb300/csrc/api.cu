@@ -968,7 +968,8 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       const int64_t most = cp->mixed || rs.team ? 16 : 8;
       int64_t CB = (budget - 2048 - 8 * R.max_rows * vsz) / (2 * stride * vsz);
       CB = std::max<int64_t>(most, std::min<int64_t>(CB, 64));
-      const StreamPlan S = build_stream(R, cp->mixed ? SB : (int64_t)1 << 40, most, CB);
+      const StreamPlan S = rs.team && !cp->mixed ? build_lookahead_stream(R, CB)
+                                                 : build_stream(R, cp->mixed ? SB : (int64_t)1 << 40, most, CB);
       const std::vector<int64_t>&Lcnt = S.L_cnt, &Ucnt = S.U_cnt;
       // per nested-dissection item: its first / end block in the subdomain's L
       // stream (rows ascending) and U stream (rows descending)

@@ -603,38 +603,33 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
 // Team apply: four warps per subdomain, for runs with few subdomains, where one warp
 // per SM sub-partition is all there is and a row's latency is the whole cost. The
 // blocks of an entry (up to 16 of a row) are dealt to the warps, one per 8-lane
-// group; the warps hand their products (FP32) or sums (FP64) over in shared memory,
-// meet at one barrier, and every warp adds them up and writes the row by itself (the
-// same bits), so that the row needs no second barrier. FP32 keeps the chain kernel's
-// order of additions (sums over the blocks 0..3 mod 4): the same bits. FP64 spreads
-// the work over the four sub-partitions' FP64 units (64 cycles per instruction each).
-// Measured, 46,657-node tube, ILU(1), us per apply, one warp / team:
-//   FP64  64 subdomains 4,334 / 2,797, 256: 1,545 / 1,174, 384: 1,026 / 965, 512: 940 / 1,015;
-//   mixed 64 subdomains 1,050 / 842, 256: 386 / 349, 384: 275 / 275, 512: 251 / 287.
-template <class TF>
+// group; the warps hand their products over in shared memory, meet at one barrier, and
+// every warp adds them up and writes the row by itself (the same bits), so that the row
+// needs no second barrier. The additions keep the chain kernel's order (sums over the
+// blocks 0..3 mod 4): the same bits.
+// Measured, mixed, 46,657-node tube, ILU(1), us per apply, one warp / team: 64
+// subdomains 1,050 / 842, 256: 386 / 349, 384: 275 / 275, 512: 251 / 287.
 __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const double* __restrict__ rin,
                                                         double* __restrict__ z, float* __restrict__ z32,
                                                         int32_t* err, const int* __restrict__ guard) {
   if (guard && *guard == 0) return;
-  constexpr bool F32 = sizeof(TF) == 4;
-  constexpr int STR = Pack<TF>::stride;
-  constexpr int V = 16 / sizeof(TF), NV = 8 / V;  // values per 16-byte piece, pieces per block row
-  constexpr uint32_t BLK = STR * sizeof(TF);
-  constexpr int PT = F32 ? 7 * 20 : 7 * 4;  // values handed over per entry: FP32 [c][v][g] (20 per c), FP64 [c][v]
+  constexpr int STR = Pack<float>::stride;
+  constexpr uint32_t BLK = STR * sizeof(float);
+  constexpr int PT = 7 * 20;  // products handed over per entry: [c][v][g], 20 per c (no bank conflicts)
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);           // [2]
-  TF* part = reinterpret_cast<TF*>(smem + 128);                 // [2][PT]
+  float* part = reinterpret_cast<float*>(smem + 128);                 // [2][PT]
   unsigned char* ring = smem + 128 + 1152;
   const uint32_t cap = R.chain_blocks * BLK;
-  TF* w = reinterpret_cast<TF*>(ring + 2 * cap);
+  float* w = reinterpret_cast<float*>(ring + 2 * cap);
   const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, s = blockIdx.x;
   const int c = lane & 7, g = lane >> 3;
-  const int b = F32 ? 4 * g + v : 4 * v + g;  // this lane's block of an entry
+  const int b = 4 * g + v;  // this lane's block of an entry
   const int64_t r0 = R.sd_row[s];
   const int m = (int)(R.sd_row[s + 1] - r0);
   const uint32_t* cw = R.code + R.code_off[s];
   const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
-  const TF* src = reinterpret_cast<const TF*>(R.pack) + (size_t)R.L_off[s] * STR;
+  const float* src = reinterpret_cast<const float*>(R.pack) + (size_t)R.L_off[s] * STR;
   const uint8_t* sz = R.stage + R.stage_off[s];
   int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
   int nsz = left > 0 ? sz[0] : 0;
@@ -663,29 +658,26 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
 #pragma unroll
     for (int e = 0; e < 7; ++e) x[e] = sr[e];
 #pragma unroll
-    for (int e = 0; e < 7; ++e) w[8 * q + e] = (TF)x[e];
-    w[8 * q + 7] = TF(0);
+    for (int e = 0; e < 7; ++e) w[8 * q + e] = (float)x[e];
+    w[8 * q + 7] = float(0);
   }
   __syncthreads();
 
   int slot = 0, phase = 0, par = 0;
   const unsigned char* at = ring + 16 * c + b * BLK;
   bool ok = true;
-  auto fetch = [&](TF (&A)[8], uint32_t code) {
+  auto fetch = [&](float (&A)[8], uint32_t code) {
     const int nb = (int)(code & 15) + 1;
-    if (F32 || 4 * v < nb) {
-#pragma unroll
-      for (int e = 0; e < NV; ++e) load16(&A[V * e], reinterpret_cast<const TF*>(at + 112 * e));
-    }
+    load16(&A[0], reinterpret_cast<const float*>(at));
+    load16(&A[4], reinterpret_cast<const float*>(at + 112));
     at += nb * BLK;
   };
   int q = 0, dq = 1;
-  int hi = 0;  // most blocks of an entry of the row so far (0: the row begins)
-  // FP32: the four partial sums of a row (blocks 0..3 mod 4), in every warp; FP64: this lane's sum
-  TF acc[4] = {TF(0), TF(0), TF(0), TF(0)}, tot = TF(-0.0);
-  TF A0[8], A1[8];
+  // the four partial sums of a row (blocks 0..3 mod 4), in every warp
+  float acc[4] = {float(0), float(0), float(0), float(0)}, tot = float(-0.0);
+  float A0[8], A1[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) A0[e] = A1[e] = TF(0);
+  for (int e = 0; e < 8; ++e) A0[e] = A1[e] = float(0);
   const int cc = c < 7 ? c : 6;
   int fslot = 0, fphase = 0;
   auto wait = [&]() {
@@ -696,34 +688,19 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       fphase = phase;
     }
   };
-  auto step = [&](TF (&A)[8], TF (&N)[8], uint32_t code, uint32_t ncode) {
+  auto step = [&](float (&A)[8], float (&N)[8], uint32_t code, uint32_t ncode) {
     if (code < ENTRY_NONE) {
       const int nb = (int)(code & 15) + 1;
       const bool piece = code & ENTRY_PIECE;
-      const TF old = w[8 * q + c];
-      TF* const pb = part + par * PT;
-      if (F32 || 4 * v < nb) {
-        const TF* xp = w + 8 * min((uint32_t)row_col(A), (uint32_t)m - 1);
-        TF x[8];
-#pragma unroll
-        for (int e = 0; e < NV; ++e) load16(&x[V * e], xp + V * e);
-        if (F32) {
-          const TF t = row_fma(A, x, TF(0));
-          if (c < 7) pb[20 * c + 4 * v + g] = b < nb ? t : TF(0);
-        } else {
-          // (the forward result is old - sum: the row's first block starts from -old)
-          const TF t = row_fma(A, x, hi == 0 && dq > 0 && b == 0 ? -old : acc[0]);
-          if (b < nb && c < 7) acc[0] = t;
-        }
-      }
-      hi = max(hi, nb);
-      if (!F32 && piece && 4 * v < hi) {
-        TF r = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 16);
-        r += __shfl_xor_sync(0xffffffffu, r, 8);
-        if (lane < 7) pb[4 * c + v] = r;
-        acc[0] = TF(0);
-      }
-      if (F32 || piece || (code & ENTRY_STAGE)) __syncthreads();
+      const float old = w[8 * q + c];
+      float* const pb = part + par * PT;
+      const float* xp = w + 8 * min((uint32_t)row_col(A), (uint32_t)m - 1);
+      float x[8];
+      load16(&x[0], xp);
+      load16(&x[4], xp + 4);
+      const float t = row_fma(A, x, float(0));
+      if (c < 7) pb[20 * c + 4 * v + g] = b < nb ? t : float(0);
+      __syncthreads();
       if (code & ENTRY_STAGE) {
         feed(slot);
         phase ^= slot;
@@ -732,37 +709,22 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
         wait();
       }
       if (ncode < ENTRY_NONE) fetch(N, ncode);
-      if (F32) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          TF t[4];
-          load16(t, pb + 20 * cc + 4 * i);
-          if (V == 2) load16(t + 2, pb + 20 * cc + 4 * i + 2);
+      for (int i = 0; i < 4; ++i) {
+        float t4[4];
+        load16(t4, pb + 20 * cc + 4 * i);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc[i] += t[e];
-        }
-        par ^= 1;
+        for (int e = 0; e < 4; ++e) acc[i] += t4[e];
       }
+      par ^= 1;
       if (piece) {
-        if (F32) {
-          tot += (acc[0] + acc[2]) + (acc[1] + acc[3]);
+        tot += (acc[0] + acc[2]) + (acc[1] + acc[3]);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) acc[i] = TF(0);
-        } else {
-          tot = pb[4 * cc];
-          if (hi > 4) tot += pb[4 * cc + 1];
-          if (hi > 8) {
-            TF t = pb[4 * cc + 2];
-            if (hi > 12) t += pb[4 * cc + 3];
-            tot += t;
-          }
-          par ^= 1;
-        }
+        for (int i = 0; i < 4; ++i) acc[i] = float(0);
         if (code & ENTRY_ROW) {
-          if (lane < 7) w[8 * q + lane] = dq > 0 ? (F32 ? old - tot : -tot) : tot;
+          if (lane < 7) w[8 * q + lane] = dq > 0 ? old - tot : tot;
           __syncwarp();
-          tot = TF(-0.0);
-          hi = 0;
+          tot = float(-0.0);
           q += dq;
         }
       }
@@ -801,6 +763,187 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       const int64_t g7 = 7 * (int64_t)R.gnode[r0 + q];
 #pragma unroll
       for (int e = 0; e < 7; ++e) z[g7 + e] = (double)w[8 * q + e];
+      if (z32) {
+#pragma unroll
+        for (int e = 0; e < 7; ++e) z32[g7 + e] = (float)w[8 * q + e];
+      }
+    }
+  }
+}
+
+// FP64 team apply, a step ahead (setup.h, build_lookahead_stream): in step t warp 0
+// solves the step's row from the sum over its far blocks, formed in step t - 1, and
+// from its near block alone, whose vector it still holds in registers (7-term dots
+// spread over its four 8-lane groups: 2 fused multiply-adds, 2 additions), while warps
+// 1 to 3 form the far sum of step t + 1's row (12 blocks at a time, 7 + 2 FP64
+// instructions of 64 cycles each). One barrier per step.
+__global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const double* __restrict__ rin,
+                                                          double* __restrict__ z, float* __restrict__ z32,
+                                                          int32_t* err, const int* __restrict__ guard) {
+  if (guard && *guard == 0) return;
+  constexpr int STR = Pack<double>::stride;
+  constexpr uint32_t BLK = STR * sizeof(double);
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);              // [2]
+  double(*part)[4][8] = reinterpret_cast<double(*)[4][8]>(smem + 128);  // [2][warp][component] far sums
+  unsigned char* ring = smem + 128 + 1152;
+  const uint32_t cap = R.chain_blocks * BLK;
+  double* w = reinterpret_cast<double*>(ring + 2 * cap);
+  const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, s = blockIdx.x;
+  const int c = lane & 7, g = lane >> 3;
+  const int b = 4 * (v - 1) + g;  // this lane's far block of an entry (warps 1 to 3)
+  const int64_t r0 = R.sd_row[s];
+  const int m = (int)(R.sd_row[s + 1] - r0);
+  const uint32_t* cw = R.code + R.code_off[s];
+  const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
+  const double* src = reinterpret_cast<const double*>(R.pack) + (size_t)R.L_off[s] * STR;
+  const uint8_t* sz = R.stage + R.stage_off[s];
+  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
+  int nsz = left > 0 ? sz[0] : 0;
+  uint64_t win = cw[0] | (uint64_t)cw[1] << 32;
+  uint32_t ahead = cw[2];
+
+  auto feed = [&](int slot) {
+    if (threadIdx.x == 0 && left > 0) {
+      mbar_arrive_expect_tx(&full[slot], nsz * BLK);
+      bulk_g2s(ring + slot * cap, src, nsz * BLK, &full[slot]);
+      src += (size_t)nsz * STR;
+      ++sz;
+      if (--left > 0) nsz = *sz;
+    }
+  };
+  if (threadIdx.x == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    feed(0);
+    feed(1);
+  }
+  if (threadIdx.x < 64) reinterpret_cast<double*>(part)[threadIdx.x] = 0.0;
+  for (int q = threadIdx.x; q < m; q += 128) {
+    const double* sr = rin + 7 * (int64_t)R.gnode[r0 + q];
+#pragma unroll
+    for (int e = 0; e < 7; ++e) w[8 * q + e] = sr[e];
+    w[8 * q + 7] = 0.0;
+  }
+  __syncthreads();
+
+  int slot = 0, phase = 0, par = 0, t = 0, fslot = 0, fphase = 0;
+  bool ok = true;
+  const unsigned char* at = ring;  // blocks of the next entry to fetch (warp 0: of the current one)
+  auto wait = [&]() {
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
+      ok = false;
+      left = 0;
+      fslot = slot;
+      fphase = phase;
+    }
+  };
+  auto next_stage = [&]() {
+    feed(slot);
+    phase ^= slot;
+    slot ^= 1;
+    at = ring + slot * cap;
+    wait();
+  };
+  auto size = [](uint32_t code) { return ((code & 15) + ((code & ENTRY_NEAR) ? 1 : 0)) * BLK; };
+  wait();
+
+  if (v == 0) {
+    double r = 0.0;  // component c of the last step's row (0 for c = 7), in all groups
+    const int k1 = g < 3 ? g + 4 : 7;
+    auto step = [&](uint32_t code) {
+      if (code >= ENTRY_NONE) return;
+      if (code & ENTRY_END) {
+        const int q = t < m ? t : 2 * m - 1 - t;
+        double acc = g == 0 ? (t < m ? -w[8 * q + c] : 0.0) : part[par][g][c];
+        if (code & ENTRY_NEAR) {
+          // entries g and g + 4 of row c (c = 7: row 6's, not used) of the near block
+          const double* A = reinterpret_cast<const double*>(at + (code & 15) * BLK) + 2 * (c < 7 ? c : 6);
+          const double x0 = __shfl_sync(0xffffffffu, r, g), x1 = __shfl_sync(0xffffffffu, r, k1);
+          acc = fma(A[14 * (g >> 1) + (g & 1)], x0, acc);
+          const double y1 = fma(A[14 * ((g + 4) >> 1) + (g & 1)], x1, acc);
+          if (g < 3) acc = y1;
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+        r = c < 7 ? (t < m ? -acc : acc) : 0.0;
+        if (lane < 7) w[8 * q + c] = r;
+        par ^= 1;
+        ++t;
+      }
+      if (code & (ENTRY_END | ENTRY_STAGE)) __syncthreads();
+      if (code & ENTRY_STAGE) next_stage();
+      else at += size(code);
+    };
+    for (int it = 0; it < 2 * nw; ++it) {
+      const uint32_t w3 = (uint32_t)win;
+      step(w3 & 255);
+      step((w3 >> 8) & 255);
+      win >>= 16;
+      if (it & 1) {
+        win |= (uint64_t)ahead << 32;
+        ahead = cw[min((it >> 1) + 3, nw + 1)];
+      }
+    }
+  } else {
+    double A0[8], A1[8], acc = 0.0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) A0[e] = A1[e] = 0.0;
+    auto fetch = [&](double (&A)[8], uint32_t code) {
+      if (4 * (v - 1) < (int)(code & 15)) {
+        const double* p = reinterpret_cast<const double*>(at + b * BLK) + 2 * (c < 7 ? c : 6);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) load16(&A[2 * e], p + 14 * e);
+      }
+      at += size(code);
+    };
+    auto step = [&](double (&A)[8], double (&N)[8], uint32_t code, uint32_t ncode) {
+      if (code < ENTRY_NONE) {
+        const int nf = (int)(code & 15);
+        if (4 * (v - 1) < nf) {
+          const double* xp = w + 8 * min((uint32_t)row_col(A), (uint32_t)m - 1);
+          double x[8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) load16(&x[2 * e], xp + 2 * e);
+          const double y = row_fma(A, x, acc);
+          if (b < nf) acc = y;
+        }
+        if (code & ENTRY_END) {
+          acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+          par ^= 1;
+          if (lane < 7) part[par][v][c] = acc;
+          acc = 0.0;
+        }
+        if (code & (ENTRY_END | ENTRY_STAGE)) __syncthreads();
+        if (code & ENTRY_STAGE) next_stage();
+      }
+      if (ncode < ENTRY_NONE) fetch(N, ncode);
+    };
+    if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
+    for (int it = 0; it < 2 * nw; ++it) {
+      const uint32_t w3 = (uint32_t)win;
+      step(A0, A1, w3 & 255, (w3 >> 8) & 255);
+      step(A1, A0, (w3 >> 8) & 255, (w3 >> 16) & 255);
+      win >>= 16;
+      if (it & 1) {
+        win |= (uint64_t)ahead << 32;
+        ahead = cw[min((it >> 1) + 3, nw + 1)];
+      }
+    }
+  }
+  if (!ok) {
+    if (lane == 0) atomicExch(err, 2);
+    mbar_wait(&full[fslot], (uint32_t)fphase);
+    mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < m; q += 128) {
+    if (R.owned[r0 + q]) {
+      const int64_t g7 = 7 * (int64_t)R.gnode[r0 + q];
+#pragma unroll
+      for (int e = 0; e < 7; ++e) z[g7 + e] = w[8 * q + e];
       if (z32) {
 #pragma unroll
         for (int e = 0; e < 7; ++e) z32[g7 + e] = (float)w[8 * q + e];
@@ -874,9 +1017,14 @@ size_t chain_smem(const RasStreamDev& r) {
 }
 
 template <class TF>
+const void* team_kernel() {
+  return sizeof(TF) == 4 ? (const void*)k_ras_apply_team : (const void*)k_ras_apply_team64;
+}
+
+template <class TF>
 cudaError_t ras_stream_init(const RasStreamDev& r) {
   const void* k = takes_ring(r) ? (const void*)k_ras_apply_stream<TF>
-                  : r.team      ? (const void*)k_ras_apply_team<TF>
+                  : r.team      ? team_kernel<TF>()
                                 : (const void*)k_ras_apply_chain<TF>;
   // all of the unified L1/shared storage as shared memory: several CTAs per SM;
   // the limit is the kernel's, not the context's: contexts of different sizes share it
@@ -891,8 +1039,10 @@ cudaError_t launch_ras_apply_stream(const RasStreamDev& r, const double* rin, do
                                     const int* guard, cudaStream_t s) {
   if (takes_ring(r))
     k_ras_apply_stream<TF><<<r.np, 32 << r.max_depth, ras_stream_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
+  else if (r.team && sizeof(TF) == 4)
+    k_ras_apply_team<<<r.np, 128, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   else if (r.team)
-    k_ras_apply_team<TF><<<r.np, 128, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
+    k_ras_apply_team64<<<r.np, 128, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   else
     k_ras_apply_chain<TF><<<r.np, 32, chain_smem<TF>(r), s>>>(r, rin, z, z32, err, guard);
   return cudaGetLastError();

@@ -527,7 +527,12 @@ RasPlan build_ras(const BsrPattern& P, const double* X, int64_t n, const int32_t
   return R;
 }
 
-StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage) {
+namespace {
+
+// Sizes, offsets and the frame common to both orders of the packed stream: `emit(s, put,
+// code)` lists subdomain s's blocks (put) and entries (code, with its blocks)
+template <class Emit>
+StreamPlan make_stream(const RasPlan& R, int64_t stage, Emit&& emit) {
   StreamPlan S;
   const int32_t np = R.np;
   const int64_t rows = (int64_t)R.gnode.size();
@@ -559,22 +564,20 @@ StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t sta
   S.piv.resize(at);
 #pragma omp parallel for schedule(dynamic, 4)
   for (int32_t s = 0; s < np; ++s) {
-    const int64_t a = R.sd_row[s], b = R.sd_row[s + 1];
     int64_t k = S.L_off[s];
     auto put = [&](int64_t e, int64_t piv) {
       S.src[k] = e;
-      S.col[k] = (int32_t)(R.col[e] - a);
+      S.col[k] = (int32_t)(R.col[e] - R.sd_row[s]);
       S.piv[k++] = piv;
     };
     std::vector<uint32_t>& W = words[s];
     std::vector<uint8_t>& C = stages[s];
     int64_t n = 0;          // entries so far
     int64_t last = -1;      // the last one with blocks
-    auto code = [&](uint32_t v) {
+    auto code = [&](uint32_t v, int64_t nb) {
       if (n % 4 == 0) W.push_back(0);
       W.back() |= v << (8 * (n % 4));
-      if (v < ENTRY_NONE) {
-        const int64_t nb = (v & 15) + 1;
+      if (nb > 0) {
         if (C.empty() || C.back() + nb > stage) {
           if (last >= 0) W[last / 4] |= ENTRY_STAGE << (8 * (last % 4));
           C.push_back(0);
@@ -584,30 +587,9 @@ StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t sta
       }
       ++n;
     };
-    int64_t pos = 0;  // blocks of this part so far
-    auto row = [&](int64_t nb) {
-      while (nb > 0) {
-        const int64_t piece = std::min(nb, cut - pos % cut);
-        nb -= piece;
-        pos += piece;
-        for (int64_t r = piece; r > 0; r -= most)
-          code((uint32_t)(std::min(r, most) - 1) | (r > most ? 0u : (nb > 0 ? ENTRY_PIECE : ENTRY_PIECE | ENTRY_ROW)));
-      }
-    };
-    for (int64_t q = a; q < b; ++q) {
-      for (int64_t e = R.row_ptr[q]; e < R.diag[q]; ++e) put(e, -1);
-      if (S.L_cnt[q] > 0) row(S.L_cnt[q]);
-      else code(ENTRY_EMPTY);
-    }
-    code(ENTRY_BACKWARD);
-    pos = 0;
-    for (int64_t q = b - 1; q >= a; --q) {
-      put(R.diag[q], -1);
-      for (int64_t e = R.diag[q] + 1; e < R.row_ptr[q + 1]; ++e) put(e, R.diag[q]);
-      row(S.U_cnt[q]);
-    }
-    while (n % 4 != 0) code(ENTRY_NONE);
-    for (int i = 0; i < 8; ++i) code(ENTRY_NONE);
+    emit(s, put, code);
+    while (n % 4 != 0) code(ENTRY_NONE, 0);
+    for (int i = 0; i < 8; ++i) code(ENTRY_NONE, 0);
   }
   for (int32_t s = 0; s < np; ++s) {
     S.code_off[s + 1] = S.code_off[s] + (int64_t)words[s].size();
@@ -621,6 +603,68 @@ StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t sta
     std::copy(stages[s].begin(), stages[s].end(), S.stage.begin() + S.stage_off[s]);
   }
   return S;
+}
+
+}  // namespace
+
+StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage) {
+  return make_stream(R, stage, [&](int32_t s, auto&& put, auto&& code) {
+    const int64_t a = R.sd_row[s], b = R.sd_row[s + 1];
+    int64_t pos = 0;  // blocks of this part so far
+    auto row = [&](int64_t nb) {
+      while (nb > 0) {
+        const int64_t piece = std::min(nb, cut - pos % cut);
+        nb -= piece;
+        pos += piece;
+        for (int64_t r = piece; r > 0; r -= most)
+          code((uint32_t)(std::min(r, most) - 1) | (r > most ? 0u : (nb > 0 ? ENTRY_PIECE : ENTRY_PIECE | ENTRY_ROW)),
+               std::min(r, most));
+      }
+    };
+    for (int64_t q = a; q < b; ++q) {
+      for (int64_t e = R.row_ptr[q]; e < R.diag[q]; ++e) put(e, -1);
+      if (R.diag[q] > R.row_ptr[q]) row(R.diag[q] - R.row_ptr[q]);
+      else code(ENTRY_EMPTY, 0);
+    }
+    code(ENTRY_BACKWARD, 0);
+    pos = 0;
+    for (int64_t q = b - 1; q >= a; --q) {
+      put(R.diag[q], -1);
+      for (int64_t e = R.diag[q] + 1; e < R.row_ptr[q + 1]; ++e) put(e, R.diag[q]);
+      row(R.row_ptr[q + 1] - R.diag[q]);
+    }
+  });
+}
+
+StreamPlan build_lookahead_stream(const RasPlan& R, int64_t stage) {
+  return make_stream(R, stage, [&](int32_t s, auto&& put, auto&& code) {
+    const int64_t a = R.sd_row[s], m = R.sd_row[s + 1] - a;
+    // the blocks of step t's row: fn(block, its pivot or -1, multiplies the row of step t - 1)
+    auto blocks = [&](int64_t t, auto&& fn) {
+      if (t < m) {
+        const int64_t q = a + t;
+        for (int64_t e = R.row_ptr[q]; e < R.diag[q]; ++e) fn(e, (int64_t)-1, R.col[e] == q - 1);
+      } else {
+        const int64_t q = a + 2 * m - 1 - t;
+        fn(R.diag[q], (int64_t)-1, t == m);
+        for (int64_t e = R.diag[q] + 1; e < R.row_ptr[q + 1]; ++e) fn(e, R.diag[q], R.col[e] == q + 1);
+      }
+    };
+    for (int64_t t = 0; t < 2 * m; ++t) {
+      int64_t far = 0;
+      if (t + 1 < 2 * m)
+        blocks(t + 1, [&](int64_t e, int64_t piv, bool near) {
+          if (!near) put(e, piv), ++far;
+        });
+      for (; far > FAR_MOST; far -= FAR_MOST) code((uint32_t)FAR_MOST, FAR_MOST);
+      uint32_t v = (uint32_t)far | ENTRY_END;
+      int64_t nb = far;
+      blocks(t, [&](int64_t e, int64_t piv, bool near) {
+        if (near) put(e, piv), v |= ENTRY_NEAR, ++nb;
+      });
+      code(v, nb);
+    }
+  });
 }
 
 FactorPipe build_factor_pipe(const RasPlan& R, int64_t cap, int64_t value_bytes) {

@@ -119,6 +119,16 @@ constexpr uint32_t ENTRY_PIECE = 16, ENTRY_ROW = 32, ENTRY_STAGE = 64, ENTRY_NON
 constexpr int64_t STAGE_MOST = 255;  // a stage's blocks are kept in a byte
 StreamPlan build_stream(const RasPlan& R, int64_t cut, int64_t most, int64_t stage);
 
+// The same stream a step ahead (the FP64 team apply): step t solves one row (forward
+// rows in increasing, then backward rows in decreasing order) from its near block, the
+// one that multiplies the row solved in step t - 1, and from the sum over its far
+// blocks, which step t - 1 has formed. Step t's part of the stream: the far blocks of
+// step t + 1's row, then step t's near block. Entry codes as above but bits 0-3: far
+// blocks (0 to 12); bit 4: the entry ends its step; bit 5: a near block follows.
+StreamPlan build_lookahead_stream(const RasPlan& R, int64_t stage);
+constexpr uint32_t ENTRY_END = 16, ENTRY_NEAR = 32;
+constexpr int64_t FAR_MOST = 12;
+
 // What the pipelined factorisation (sparse.cu, k_ras_factor_pipe) copies to shared
 // memory ahead of each L block (i,k), in elimination order: a word list
 //   [ updates | shift << 16 | kind << 28, 0, then per update target << 16 | source ]

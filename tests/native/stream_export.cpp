@@ -18,7 +18,7 @@ extern "C" void* stream_new(int64_t n, const double* X, int64_t T, const int32_t
   auto* b = new Box;
   std::vector<int32_t> tv(tets, tets + 4 * T);
   b->R = build_ras(build_pattern(n, tv), X, n, nullptr, 1, np, 1, fill, ordering, rank);
-  b->S = build_stream(b->R, cut, most, stage);
+  b->S = most > 0 ? build_stream(b->R, cut, most, stage) : build_lookahead_stream(b->R, stage);
   return b;
 }
 

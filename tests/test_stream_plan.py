@@ -117,3 +117,58 @@ def test_walk_solves_the_subdomains(lib, most, stage, ordering, np_, fill, cut):
         assert q == -1 and (S["L_off"][s + 1] == k)
         assert np.abs(w - want).max() <= 1e-12 * max(1.0, np.abs(want).max())
     assert np.all(seen == 1)
+
+
+@pytest.mark.parametrize("ordering", [0, 1, 2])
+@pytest.mark.parametrize("np_,fill,stage", [(4, 1, 16), (1, 2, 64), (64, 0, 13), (7, 3, 29), (200, 1, 16)])
+def test_lookahead_walk_solves_the_subdomains(lib, np_, fill, stage, ordering):
+    """The FP64 team's stream: a step's near block multiplies the row solved just
+    before, its far blocks were summed a step earlier, before that row was known."""
+    m = vm.tube_config("tube-12x8x4")
+    S = plan(lib, m, np_, fill, ordering, 0, 0, stage)
+    rng = np.random.default_rng(5)
+    fac = rng.normal(size=len(S["col"])) * 0.1
+    seen = np.zeros(len(fac), dtype=int)
+    for s in range(len(S["sd_row"]) - 1):
+        a, b = S["sd_row"][s], S["sd_row"][s + 1]
+        n = b - a
+        r = rng.normal(size=n)
+        want = r.copy()
+        for q in range(a, b):
+            e = slice(S["row_ptr"][q], S["diag"][q])
+            want[q - a] -= fac[e] @ want[S["col"][e] - a]
+        for q in range(b - 1, a - 1, -1):
+            e = slice(S["diag"][q] + 1, S["row_ptr"][q + 1])
+            want[q - a] = fac[S["diag"][q]] * (want[q - a] - fac[e] @ want[S["col"][e] - a])
+        w, k, t, far, nxt, in_stage = r.copy(), S["L_off"][s], 0, 0.0, 0.0, 0
+        sizes = S["stage"][S["stage_off"][s]:S["stage_off"][s + 1]].astype(int).tolist()
+        assert max(sizes) <= stage
+        row = lambda i: i if i < n else 2 * n - 1 - i
+        val = lambda i: fac[S["src"][i]] if S["piv"][i] < 0 else -fac[S["piv"][i]] * fac[S["src"][i]]
+        for x in S["code"][S["code_off"][s]:S["code_off"][s + 1]]:
+            for c in [(int(x) >> (8 * i)) & 255 for i in range(4)]:
+                if c == NONE:
+                    continue
+                nf, near, solved = c & 15, 1 if c & 32 else 0, None
+                assert nf <= 12
+                for i in range(k, k + nf):
+                    seen[S["src"][i]] += 1
+                    assert t == 0 or S["bcol"][i] != row(t) or row(t + 1) == row(t)
+                    nxt += val(i) * w[S["bcol"][i]]
+                if near:
+                    seen[S["src"][k + nf]] += 1
+                    assert S["bcol"][k + nf] == row(t - 1)
+                    far += val(k + nf) * w[S["bcol"][k + nf]]
+                k += nf + near
+                in_stage += nf + near
+                if c & STAGE:
+                    assert in_stage == sizes.pop(0)
+                    in_stage = 0
+                if c & 16:
+                    w[row(t)] = w[row(t)] - far if t < n else far
+                    far, nxt, t = nxt, 0.0, t + 1
+                else:
+                    assert not near
+        assert t == 2 * n and k == S["L_off"][s + 1] and sizes == [in_stage]
+        assert np.abs(w - want).max() <= 1e-12 * max(1.0, np.abs(want).max())
+    assert np.all(seen == 1)
