@@ -963,8 +963,9 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       // row's sum in the pieces the ring's stages cut it into, so that both kernels give the same bits;
       // in FP64 whole rows
       // four warps per subdomain where there are too few subdomains to fill the SMs' schedulers
-      // with one warp each (measured at 32 to 1,088 subdomains, ILU(1) and ILU(2): k_ras_apply_team)
-      rs.team = R.max_depth == 0 && R.np <= (cp->mixed ? 256 : 384);
+      // with one warp each (measured at 32 to 1,600 subdomains, ILU(1) and ILU(2): k_ras_apply_team,
+      // k_ras_apply_team64)
+      rs.team = R.max_depth == 0 && R.np <= (cp->mixed ? 256 : 608);
       const int64_t most = cp->mixed || rs.team ? 16 : 8;
       int64_t CB = (budget - 2048 - 8 * R.max_rows * vsz) / (2 * stride * vsz);
       CB = std::max<int64_t>(most, std::min<int64_t>(CB, 64));

@@ -776,7 +776,11 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
 // from its near block alone, whose vector it still holds in registers (7-term dots
 // spread over its four 8-lane groups: 2 fused multiply-adds, 2 additions), while warps
 // 1 to 3 form the far sum of step t + 1's row (12 blocks at a time, 7 + 2 FP64
-// instructions of 64 cycles each). One barrier per step.
+// instructions of 64 cycles each). One barrier per step. Measured against one warp
+// per subdomain (k_ras_apply_chain), us per apply: 46,657-node tube, ILU(1), 64
+// subdomains 4,334 / 2,409, 256: 1,545 / 927, 384: 978 / 708, 512: 890 / 767, 768: 759 / 716,
+// 1,024: 617 / 694; 103k-node tree, ILU(1), 512: 1,199 / 1,041, 768: 989 / 1,115, ILU(2)
+// 512: 1,753 / 1,407, 768: 1,446 / 1,518. Taken up to 608 (four subdomains per SM).
 __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const double* __restrict__ rin,
                                                           double* __restrict__ z, float* __restrict__ z32,
                                                           int32_t* err, const int* __restrict__ guard) {
@@ -953,38 +957,53 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
 }
 
 // copy the factor blocks into the packed stream (7 rows of 8: the row's 7
-// entries, then the block's column); a U block with a pivot (piv >= 0) is stored as -D_q^{-1} U_qj, the
-// row's inverted pivot and the L blocks as they are
+// entries, then the block's column, in 16-byte pieces); a U block with a pivot
+// (piv >= 0) is stored as -D_q^{-1} U_qj, the row's inverted pivot and the L
+// blocks as they are. One warp per block: its index list entries are read once per
+// block and the products take both blocks from shared memory (one thread per value,
+// with 64-bit divisions and the products' 14 operands from L1: 1.27 M blocks 295 -> 195 us).
 template <class TF>
-__global__ void k_pack_factors(int64_t nblk, const int64_t* __restrict__ src, const int32_t* __restrict__ col,
-                               const int64_t* __restrict__ pivs, const TF* __restrict__ fac, TF* __restrict__ pack) {
-  constexpr int STR = Pack<TF>::stride;
-  const int64_t total = nblk * STR;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = idx / STR;
-    const int e = (int)(idx - STR * b);
-    constexpr int V = 16 / sizeof(TF);
-    const int r = (e % (7 * V)) / V, k = (e / (7 * V)) * V + e % V;
-    const int64_t sb = src[b];
-    if (k < 7) {
-      const int64_t piv = pivs[b];
-      if (piv < 0) {
-        pack[idx] = fac[49 * sb + 7 * r + k];
+__global__ void __launch_bounds__(256) k_pack_factors(int64_t nblk, const int64_t* __restrict__ src,
+                                                      const int32_t* __restrict__ col,
+                                                      const int64_t* __restrict__ pivs, const TF* __restrict__ fac,
+                                                      TF* __restrict__ pack) {
+  constexpr int STR = Pack<TF>::stride, V = 16 / sizeof(TF);
+  __shared__ TF sm[8][2][56];
+  const int lane = threadIdx.x & 31;
+  TF* A = sm[threadIdx.x >> 5][0];
+  TF* D = sm[threadIdx.x >> 5][1];
+  // this lane's values e = lane and lane + 32 (below 56): row and entry
+  const int e1 = lane + 32;
+  const int r0 = (lane % (7 * V)) / V, k0 = (lane / (7 * V)) * V + lane % V;
+  const int r1 = (e1 % (7 * V)) / V, k1 = (e1 / (7 * V)) * V + e1 % V;
+  const int64_t step = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nblk; b += step) {
+    const int64_t sb = src[b], piv = pivs[b];
+    const int cb = col[b];
+    A[lane] = fac[49 * sb + lane];
+    if (lane < 17) A[lane + 32] = fac[49 * sb + lane + 32];
+    if (piv >= 0) {
+      D[lane] = fac[49 * piv + lane];
+      if (lane < 17) D[lane + 32] = fac[49 * piv + lane + 32];
+    }
+    __syncwarp();
+    auto value = [&](int r, int k) {
+      TF v = TF(0);
+      if (k == 7) {
+        *reinterpret_cast<int*>(&v) = cb;
+      } else if (piv < 0) {
+        v = A[7 * r + k];
       } else {
         // -(D_q^{-1} U_qj)[r][k]
-        const TF* Dq = fac + 49 * piv + 7 * r;
-        const TF* U = fac + 49 * sb + k;
-        TF v = TF(0);
 #pragma unroll
-        for (int mm = 0; mm < 7; ++mm) v += Dq[mm] * U[7 * mm];
-        pack[idx] = -v;
+        for (int mm = 0; mm < 7; ++mm) v += D[7 * r + mm] * A[7 * mm + k];
+        v = -v;
       }
-    } else {
-      TF v = TF(0);
-      *reinterpret_cast<int*>(&v) = col[b];
-      pack[idx] = v;
-    }
+      return v;
+    };
+    pack[b * STR + lane] = value(r0, k0);
+    if (e1 < STR) pack[b * STR + e1] = value(r1, k1);
+    __syncwarp();
   }
 }
 
@@ -999,8 +1018,7 @@ size_t ras_stream_smem(const RasStreamDev& r) {
 
 template <class TF>
 void launch_pack_factors(const RasStreamDev& r, const TF* fac, cudaStream_t s) {
-  const int64_t total = r.nblk * Pack<TF>::stride;
-  int64_t g = (total + 255) / 256;
+  int64_t g = (r.nblk + 7) / 8;
   if (g > 152 * 64) g = 152 * 64;
   k_pack_factors<TF><<<(int)g, 256, 0, s>>>(r.nblk, r.src, r.col, r.piv, fac, (TF*)r.pack);
 }

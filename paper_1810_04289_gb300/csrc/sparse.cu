@@ -113,15 +113,19 @@ __global__ void k_to_float(int64_t n, const double* __restrict__ x, float* __res
 // ---------------------------------------------------------------------------
 // RAS: extraction of J_i^delta = R_i^delta J (R_i^delta)^T (Eq. 15)
 // ---------------------------------------------------------------------------
+// one warp per block (one index read per block, no division per value)
 template <class TF, class TJ>
-__global__ void k_ras_extract(int64_t nblocks, const int64_t* __restrict__ gblk, const TJ* __restrict__ vals,
-                              TF* __restrict__ fac) {
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < 49 * nblocks;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = idx / 49;
-    const int e = (int)(idx - 49 * b);
+__global__ void __launch_bounds__(256) k_ras_extract(int64_t nblocks, const int64_t* __restrict__ gblk,
+                                                     const TJ* __restrict__ vals, TF* __restrict__ fac) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = ((int64_t)gridDim.x * blockDim.x) >> 5;
+#pragma unroll 2
+  for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nblocks; b += step) {
     const int64_t gb = gblk[b];
-    fac[idx] = gb >= 0 ? (TF)vals[49 * gb + e] : TF(0);
+    const TJ* v = vals + 49 * gb;
+    const TF x0 = gb >= 0 ? (TF)v[lane] : TF(0), x1 = gb >= 0 && lane < 17 ? (TF)v[lane + 32] : TF(0);
+    fac[49 * b + lane] = x0;
+    if (lane < 17) fac[49 * b + lane + 32] = x1;
   }
 }
 
@@ -808,7 +812,7 @@ void launch_to_float(int64_t n, const double* x, float* y, const int* guard, cud
 
 template <class TF, class TJ>
 void launch_ras_extract(const RasDev& r, const TJ* vals, TF* fac, cudaStream_t s) {
-  k_ras_extract<TF, TJ><<<grid_for(49 * r.nblocks, 256), 256, 0, s>>>(r.nblocks, r.gblk, vals, fac);
+  k_ras_extract<TF, TJ><<<grid_for(32 * r.nblocks, 256), 256, 0, s>>>(r.nblocks, r.gblk, vals, fac);
 }
 
 template <class TF>

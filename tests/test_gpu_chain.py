@@ -52,7 +52,7 @@ def far(a, b):
 
 
 @pytest.mark.parametrize("ilu,ordering", [(1, 1), (2, 2), (3, 0), (0, 1)])
-@pytest.mark.parametrize("nsub", [2, 256, 257, 384, 385, 900])
+@pytest.mark.parametrize("nsub", [2, 256, 257, 608, 609, 900])
 def test_chain_and_team_match_the_level_scheduled_kernel(case, nsub, ilu, ordering):
     opt = dict(n_subdomains=nsub, ilu_level=ilu, ordering=ordering)
     ref = apply(case, 0, 2, **opt)
@@ -71,7 +71,7 @@ def test_pipelined_factors_are_the_row_kernels_bits(case, precision, nsub, ilu, 
     assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("precision,nsub", [(0, 500), (1, 500), (1, 8)])
+@pytest.mark.parametrize("precision,nsub", [(0, 700), (0, 8), (1, 500), (1, 8)])
 def test_waits_that_run_out_are_reported(case, precision, nsub):
     m, y, r = case
     S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=nsub, fault_test=1))
