@@ -213,11 +213,10 @@ void check_launch() { CK(cudaGetLastError()); }
 
 // ---- F(y) for the step ending at t_n + dt (previous levels y_n, y_{n-1})
 void residual(fsi_ctx* c, const double* y, double* F) {
-  c->launches += 3;
+  c->launches += 2;
   int h = c->begin_phase(PH_FUNC);
   launch_elem_residual(c->mesh, c->mc, y, c->yn, c->ynm1, c->Fe, c->s);
-  launch_gather_residual(c->mesh, c->nptr, c->nsrc, c->Fe, F, c->s);
-  launch_constraint_residual(c->mesh, c->mc, c->t + c->opt.dt, y, c->yn, F, c->s);
+  launch_gather_residual(c->mesh, c->mc, c->t + c->opt.dt, c->nptr, c->nsrc, c->Fe, y, c->yn, F, c->s);
   check_launch();
   c->end_phase(h, PH_FUNC);
 }
@@ -1402,8 +1401,7 @@ extern "C" fsi_status fsi_residual_noalloc(fsi_ctx* c, const double* y, double* 
     // every slot the gather reads is written by the element kernel first, so the
     // array needs no clearing between calls
     launch_elem_residual(c->mesh, c->mc, y, c->yn, c->ynm1, fe, c->s);
-    launch_gather_residual(c->mesh, c->nptr, c->nsrc, fe, F, c->s);
-    launch_constraint_residual(c->mesh, c->mc, c->t + c->opt.dt, y, c->yn, F, c->s);
+    launch_gather_residual(c->mesh, c->mc, c->t + c->opt.dt, c->nptr, c->nsrc, fe, y, c->yn, F, c->s);
     check_launch();
     CK(cudaStreamSynchronize(c->s));
     return FSI_OK;

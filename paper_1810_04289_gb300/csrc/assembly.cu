@@ -154,19 +154,47 @@ __global__ void __launch_bounds__(128) k_elem_residual(MeshDev m, MatConst mc, c
   }
 }
 
-// Each node row is summed from its buffer slots in tet order; eight lanes take a node
-// (seven of them a component each), four slots in flight. The FP64 additions and the
-// read of the buffer (56 bytes per slot) bound it about equally: 912k tets 67 us.
-__global__ void __launch_bounds__(256) k_gather_residual(int64_t N, const int64_t* __restrict__ nptr,
+// the residual of component r of node i where a flag constrains it, else s (a call of
+// its own, taken by the nodes with flags only: inlined, its registers cost the gather
+// more than the call)
+__device__ __noinline__ double constrained(const MeshDev* m, double dt, double t, const double* y, const double* y1,
+                                           int64_t i, int r, uint32_t f, double s) {
+  const double* yi = y + 7 * i;
+  if (r >= 3) return (r == 3 ? (f & NF_P_IDENT) : (f & NF_D_ZERO)) ? yi[r] : s;
+  if (f & NF_U_INLET) {
+    const double* in = m->inlet + INLET_STRIDE * m->nprob[i];
+    const double* x = m->X + 3 * i;
+    const double rx = x[0] - in[0], ry = x[1] - in[1], rz = x[2] - in[2];
+    const double ax = rx * in[3] + ry * in[4] + rz * in[5];
+    const double r2 = (rx * rx + ry * ry + rz * rz) - ax * ax;
+    const double U = in[7] * (1.0 + in[8] * sin(2.0 * 3.141592653589793 * in[9] * t + in[10]));
+    const double prof = fmax(0.0, 1.0 - r2 / (in[6] * in[6]));
+    return yi[r] - U * prof * in[3 + r];
+  }
+  if (f & NF_U_IDENT) return yi[r];
+  if (f & NF_U_KIN) return yi[r] - (yi[4 + r] - y1[7 * i + 4 + r]) * (1.0 / dt);
+  return s;
+}
+
+// Each node row is summed from its buffer slots in tet order, then constrained rows
+// get their own residual; eight lanes take a node (seven of them a component each),
+// four slots in flight. The FP64 additions and the read of the buffer (56 bytes per
+// slot) bound it about equally: 912k tets 83 us (76 as two launches; 2,016 tets, one
+// launch less: the whole residual 47 -> 38 us).
+__global__ void __launch_bounds__(256) k_gather_residual(const __grid_constant__ MeshDev m, MatConst mc, double t,
+                                                         const int64_t* __restrict__ nptr,
                                                          const int32_t* __restrict__ nsrc,
-                                                         const double* __restrict__ Fe, double* __restrict__ F) {
+                                                         const double* __restrict__ Fe,
+                                                         const double* __restrict__ y,
+                                                         const double* __restrict__ y1, double* __restrict__ F) {
   const int r = threadIdx.x & 7;
   const int64_t step = ((int64_t)gridDim.x * blockDim.x) >> 3;
-  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; i < N; i += step) {
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; i < m.N; i += step) {
     if (r == 7) continue;
     double s = 0.0;
     int64_t c = nptr[i];
     const int64_t c1 = nptr[i + 1];
+    const uint32_t f = m.nflag[i];
     for (; c + 4 <= c1; c += 4) {
       double v[4];
 #pragma unroll
@@ -175,35 +203,8 @@ __global__ void __launch_bounds__(256) k_gather_residual(int64_t N, const int64_
       for (int k = 0; k < 4; ++k) s += v[k];
     }
     for (; c < c1; ++c) s += Fe[7 * (int64_t)nsrc[c] + r];
+    if (f & (NF_U_CONSTR | NF_P_IDENT | NF_D_ZERO)) s = constrained(&m, mc.dt, t, y, y1, i, r, f, s);
     F[7 * i + r] = s;
-  }
-}
-
-__global__ void k_constraint_residual(MeshDev m, MatConst mc, double t, const double* __restrict__ y,
-                                      const double* __restrict__ y1, double* __restrict__ F) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m.N; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t f = m.nflag[i];
-    const double* yi = y + 7 * i;
-    double* Fi = F + 7 * i;
-    if (f & NF_U_KIN) {
-      const double* y1i = y1 + 7 * i;
-      const double idt = 1.0 / mc.dt;
-      for (int c = 0; c < 3; ++c) Fi[c] = yi[c] - (yi[4 + c] - y1i[4 + c]) * idt;
-    }
-    if (f & NF_U_IDENT)
-      for (int c = 0; c < 3; ++c) Fi[c] = yi[c];
-    if (f & NF_P_IDENT) Fi[3] = yi[3];
-    if (f & NF_D_ZERO)
-      for (int c = 0; c < 3; ++c) Fi[4 + c] = yi[4 + c];
-    if (f & NF_U_INLET) {
-      const double* in = m.inlet + INLET_STRIDE * m.nprob[i];
-      const double rx = m.X[3 * i] - in[0], ry = m.X[3 * i + 1] - in[1], rz = m.X[3 * i + 2] - in[2];
-      const double ax = rx * in[3] + ry * in[4] + rz * in[5];
-      const double r2 = (rx * rx + ry * ry + rz * rz) - ax * ax;
-      const double U = in[7] * (1.0 + in[8] * sin(2.0 * 3.141592653589793 * in[9] * t + in[10]));
-      const double prof = fmax(0.0, 1.0 - r2 / (in[6] * in[6]));
-      for (int c = 0; c < 3; ++c) Fi[c] = yi[c] - U * prof * in[3 + c];
-    }
   }
 }
 
@@ -631,17 +632,15 @@ inline int grid_for(int64_t work, int block) {
 void launch_elem_residual(const MeshDev& m, const MatConst& mc, const double* y, const double* y1,
                           const double* y2, double* Fe, cudaStream_t s) {
   if (m.T == 0) return;
-  k_elem_residual<<<grid_for(m.T, 128), 128, 0, s>>>(m, mc, y, y1, y2, Fe);
+  // one warp per block while that spreads the tets over more SMs: alone on an SM's
+  // FP64 pipe a warp issues every 64 cycles, four of them every 76 each
+  const int threads = m.T <= 152 * 128 ? 32 : 128;
+  k_elem_residual<<<grid_for(m.T, threads), threads, 0, s>>>(m, mc, y, y1, y2, Fe);
 }
 
-void launch_gather_residual(const MeshDev& m, const int64_t* nptr, const int32_t* nsrc, const double* Fe,
-                            double* F, cudaStream_t s) {
-  k_gather_residual<<<grid_for(8 * m.N, 256), 256, 0, s>>>(m.N, nptr, nsrc, Fe, F);
-}
-
-void launch_constraint_residual(const MeshDev& m, const MatConst& mc, double t, const double* y,
-                                const double* y1, double* F, cudaStream_t s) {
-  k_constraint_residual<<<grid_for(m.N, 256), 256, 0, s>>>(m, mc, t, y, y1, F);
+void launch_gather_residual(const MeshDev& m, const MatConst& mc, double t, const int64_t* nptr, const int32_t* nsrc,
+                            const double* Fe, const double* y, const double* y1, double* F, cudaStream_t s) {
+  k_gather_residual<<<grid_for(8 * m.N, 256), 256, 0, s>>>(m, mc, t, nptr, nsrc, Fe, y, y1, F);
 }
 
 inline int jac_blocks(int64_t nt) {

@@ -29,10 +29,9 @@ void launch_wss(const MeshDev& m, double mu, int64_t nf, const int64_t* face, co
 // ---- assembly (assembly.cu)
 void launch_elem_residual(const MeshDev& m, const MatConst& mc, const double* y, const double* y1,
                           const double* y2, double* Fe, cudaStream_t s);
-void launch_gather_residual(const MeshDev& m, const int64_t* nptr, const int32_t* nsrc, const double* Fe,
-                            double* F, cudaStream_t s);
-void launch_constraint_residual(const MeshDev& m, const MatConst& mc, double t, const double* y,
-                                const double* y1, double* F, cudaStream_t s);
+// the node rows' sums, constrained rows replaced (t: the step's end time)
+void launch_gather_residual(const MeshDev& m, const MatConst& mc, double t, const int64_t* nptr, const int32_t* nsrc,
+                            const double* Fe, const double* y, const double* y1, double* F, cudaStream_t s);
 // reference geometry of every tet into geo ([GEO][T])
 void launch_geometry(const MeshDev& m, double* geo, cudaStream_t s);
 // element Jacobians of the tets [t0, t1) into Ke (784 values per tet, from tet t0).
