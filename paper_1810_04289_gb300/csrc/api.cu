@@ -926,11 +926,11 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     }
     cp->ras = rd;
     // the Jacobian is assembled in chunks of tets so that Ke needs no more than
-    // the factors' size (or 1 GB): the shared buffer is as large as the factors
+    // the factors' size (or 2 GB): the shared buffer is as large as the factors
     {
       const int64_t fac_bytes = (int64_t)(49 * vs) * rd.nblocks;
       const int64_t per_tet = (int64_t)((784 + (cp->mixed ? 0 : JAC_VALUES)) * vs);
-      const int64_t room = std::max<int64_t>(fac_bytes, (int64_t)1 << 30);
+      const int64_t room = std::max<int64_t>(fac_bytes, (int64_t)1 << 31);
       cp->ke_tets = std::max<int64_t>(1, std::min<int64_t>(T0, room / per_tet));
       if (o.jac_chunk > 0) cp->ke_tets = std::min<int64_t>(T0, o.jac_chunk);
       // (+ 16: the pipelined factorisation copies whole 16-byte units)

@@ -304,7 +304,7 @@ k_elem_jacobian(MeshDev m, MatConst mc, const T* __restrict__ Xl, const T* __res
 // (u column: alpha = e_k, eta = 1; p: gamma = 1; d: alpha = -G e_k, gamma = -grad p_k,
 // eta = -1/dt, nu = g_b,k, zeta_a = g_a,k), so a column is a handful of products of
 // per-tet and per-(a, b) values. k_jac_values computes those once per tet (one
-// thread per tet), k_elem_jacobian64 one column per thread from them: 28 x ~170
+// thread per tet), k_elem_jacobian64 one column per thread from them: 28 x ~133
 // FP64 instructions per tet in place of 28 x ~1,900 with dual numbers, each of which
 // redid the value part. Bound by the FP64 pipe all the same.
 // ---------------------------------------------------------------------------
@@ -445,14 +445,81 @@ __global__ void __launch_bounds__(128) k_jac_values(MeshDev m, MatConst mc, cons
   }
 }
 
+// Column kinds have warps of their own (of a block's 8 tets: three warps of u columns,
+// three of d columns, one of p columns): a u column needs 126 FP64 instructions, a d
+// column 170, a p column 45, where a mixed warp would run all three.
+template <int KIND>  // 0: u column, 1: p, 2: d
+__device__ __forceinline__ void fluid_column(const double* s, int b, int kk, double idt, double rho, double mu,
+                                             const uint32_t f[4], double* o) {
+  constexpr bool U = KIND == 0, P = KIND == 1, D = KIND == 2;
+  const double* gb = s + JV_G + 3 * b;
+  const double vol = s[JV_SC], c = s[JV_SC + 1], tv = s[JV_SC + 2], vmu = vol * mu;
+  const double eta = U ? 1.0 : D ? -idt : 0.0;
+  const double theta = P ? 0.0 : eta * s[JV_TH + kk];
+  const double gam = P ? 1.0 : D ? -s[JV_GP + kk] : 0.0;
+  const double nu = D ? gb[kk] : 0.0;
+  double al[3], be[3], dr[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double Gik = P ? 0.0 : s[JV_GU + 3 * i + kk];
+    al[i] = D ? -Gik : 0.0;
+    be[i] = P ? 0.0 : rho * eta * Gik;
+    if (U && i == kk) be[i] += rho * idt;
+    dr[i] = P ? tv * gb[i] : tv * (0.25 * be[i] + (D ? 0.25 * rho * s[JV_S + b] * al[i] + gam * gb[i] : 0.0));
+    if (U && i == kk) dr[i] += tv * (0.25 * rho * s[JV_S + b]);
+  }
+  const double om = U ? gb[kk] : D ? al[0] * gb[0] + al[1] * gb[1] + al[2] * gb[2] : 0.0;
+  const double gac = P ? -0.25 * vol : theta * s[JV_SC + 3] + om * s[JV_SC + 4];
+  const double ceta = c * eta, q4 = 0.25 * vol * om, cg5 = 5.0 * c * gam;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const double* ga = s + JV_G + 3 * a;
+    const double g0 = ga[0], g1 = ga[1], g2 = ga[2];
+    const bool uc = f[a] & NF_U_CONSTR, pc = f[a] & NF_P_IDENT, dz = f[a] & NF_D_ZERO, itf = f[a] & NF_ITF;
+    const double gk = P ? 0.0 : ga[kk];
+    const double e1 = P ? 0.0 : s[JV_E1 + 4 * b + a], e2 = P ? 0.0 : s[JV_E2 + 4 * b + a], hc = ceta * gk;
+    const double gbc = U ? vmu * gk
+                         : D ? vmu * (al[0] * g0 + al[1] * g1 + al[2] * g2) + cg5 * s[JV_S + a] : cg5 * s[JV_S + a];
+    const double K = D ? s[JV_K + 4 * b + a] : 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      double r = gb[i] * gbc + (i == 0 ? g0 : i == 1 ? g1 : g2) * gac;
+      if (!P) {
+        r -= theta * s[JV_Q + 3 * a + i];
+        r += be[i] * e2;
+        r += s[JV_H + 3 * b + i] * hc;
+      }
+      if (U && i == kk) r += e1;
+      if (D) {
+        r += nu * s[JV_RM + 3 * a + i];
+        r += al[i] * e1;
+        r -= gk * s[JV_F + 3 * b + i];
+      }
+      o[196 * a + 7 * i] = uc ? 0.0 : r;
+      o[196 * a + 7 * (4 + i)] = dz ? 0.0 : (itf ? r : (D && i == kk ? K : 0.0));
+    }
+    double rc = q4 + g0 * dr[0] + g1 * dr[1] + g2 * dr[2];
+    if (!P) rc -= theta * s[JV_GR + a];
+    if (D) {
+      rc += nu * s[JV_RC + a];
+      rc -= gk * s[JV_GR + b];
+    }
+    o[196 * a + 7 * 3] = pc ? 0.0 : rc;
+  }
+}
+
 __global__ void __launch_bounds__(28 * JAC_TETS_PER_BLOCK)
 k_elem_jacobian64(MeshDev m, MatConst mc, const double* __restrict__ val, double* __restrict__ Ke, int64_t t0,
                   int64_t t1) {
   __shared__ double sv[JAC_TETS_PER_BLOCK][JV + 1];  // odd row length: the tets of a block on other banks
   const int64_t nt = t1 - t0;
-  const int tl = threadIdx.x / 28;
-  const int colid = threadIdx.x - 28 * tl;
-  const int b = colid / 7, k = colid - 7 * (colid / 7);
+  // kind of column, tet of the block, column (b, k)
+  const int x = threadIdx.x;
+  const int kind = x < 96 ? 0 : x < 192 ? 2 : 1;
+  const int y = kind == 0 ? x : kind == 2 ? x - 96 : x - 192;
+  const int tl = kind == 1 ? y >> 2 : y / 12, cl = kind == 1 ? y & 3 : y - 12 * tl;
+  const int b = kind == 1 ? cl : cl / 3, kk = kind == 1 ? 0 : cl - 3 * b;
+  const int k = kind == 0 ? kk : kind == 1 ? 3 : 4 + kk;
   for (int64_t tb = t0 + blockIdx.x * (int64_t)JAC_TETS_PER_BLOCK; tb < t1;
        tb += (int64_t)gridDim.x * JAC_TETS_PER_BLOCK) {
     __syncthreads();
@@ -469,63 +536,17 @@ k_elem_jacobian64(MeshDev m, MatConst mc, const double* __restrict__ val, double
     load_tet(m, t, n, f);
     double* o = Ke + 784 * (t - t0) + 49 * b + k;
     if (t < m.Tf) {
-      const bool isu = k < 3, isp = k == 3, isd = k > 3;
-      const int kk = isu ? k : (isd ? k - 4 : 0);
-      const double idt = 1.0 / mc.dt, rho = mc.rho_f;
-      const double eta = isu ? 1.0 : (isd ? -idt : 0.0);
-      const double gam = isp ? 1.0 : (isd ? -s[JV_GP + kk] : 0.0);
-      const double* gb = s + JV_G + 3 * b;
-      const double nu = isd ? gb[kk] : 0.0;
-      const double vol = s[JV_SC], c = s[JV_SC + 1], tv = s[JV_SC + 2];
-      const double theta = eta * s[JV_TH + kk];
-      double al[3], be[3], h[3], dr[3];
-      const double rq = 0.25 * rho * s[JV_S + b];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const double Gik = s[JV_GU + 3 * i + kk];
-        al[i] = isu ? (i == kk ? 1.0 : 0.0) : (isd ? -Gik : 0.0);
-        be[i] = rho * eta * Gik + (isu && i == kk ? rho * idt : 0.0);
-        h[i] = s[JV_H + 3 * b + i];
-        dr[i] = tv * (rq * al[i] + 0.25 * be[i] + gam * gb[i]);
-      }
-      const double om = al[0] * gb[0] + al[1] * gb[1] + al[2] * gb[2];
-      const double gac = theta * s[JV_SC + 3] + om * s[JV_SC + 4] - (isp ? 0.25 * vol : 0.0);
-      const double cg5 = 5.0 * c * gam, ceta = c * eta, vmu = vol * mc.mu_f, q4 = 0.25 * vol * om;
-      const double grb = s[JV_GR + b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const double* ga = s + JV_G + 3 * a;
-        const double g0 = ga[0], g1 = ga[1], g2 = ga[2];
-        const double gk = ga[kk];
-        const double zeta = isd ? gk : 0.0, hc = ceta * gk;
-        const double gbc = vmu * (al[0] * g0 + al[1] * g1 + al[2] * g2) + cg5 * s[JV_S + a];
-        const double e1 = s[JV_E1 + 4 * b + a], e2 = s[JV_E2 + 4 * b + a];
-        const bool uc = f[a] & NF_U_CONSTR, pc = f[a] & NF_P_IDENT, dz = f[a] & NF_D_ZERO, itf = f[a] & NF_ITF;
-        const double K = isd ? s[JV_K + 4 * b + a] : 0.0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          double r = nu * s[JV_RM + 3 * a + i] - theta * s[JV_Q + 3 * a + i];
-          r += al[i] * e1;
-          r += be[i] * e2;
-          r += h[i] * hc;
-          r += gb[i] * gbc;
-          r += (i == 0 ? g0 : i == 1 ? g1 : g2) * gac;
-          r -= zeta * s[JV_F + 3 * b + i];
-          o[196 * a + 7 * i] = uc ? 0.0 : r;
-          o[196 * a + 7 * (4 + i)] = dz ? 0.0 : (itf ? r : (i == kk ? K : 0.0));
-        }
-        const double rc = nu * s[JV_RC + a] + q4 - theta * s[JV_GR + a] - zeta * grb + g0 * dr[0] + g1 * dr[1] +
-                          g2 * dr[2];
-        o[196 * a + 7 * 3] = pc ? 0.0 : rc;
-      }
-    } else {
-      // d column k of node b: |K0| (F S)' g0_a and the inertia
-      const int kk = k > 3 ? k - 4 : 0;
+      const double idt = 1.0 / mc.dt;
+      if (kind == 0) fluid_column<0>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
+      else if (kind == 2) fluid_column<2>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
+      else fluid_column<1>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
+    } else if (kind == 2) {
+      // d column: |K0| (F S)' g0_a and the inertia
       const double vmu = mc.mu_s * m.geo[9 * m.T + t], vlam = mc.lam_s * m.geo[9 * m.T + t];
       const double fbk = s[JW_F + 3 * b + kk];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        const bool z = (f[a] & NF_D_ZERO) || k < 4;
+        const bool z = f[a] & NF_D_ZERO;
         const double gg = s[JW_GG + 4 * b + a], fak = vmu * s[JW_F + 3 * a + kk], lb = vlam * fbk;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -536,6 +557,11 @@ k_elem_jacobian64(MeshDev m, MatConst mc, const double* __restrict__ val, double
         }
         o[196 * a + 7 * 3] = 0.0;
       }
+    } else {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int r = 0; r < 7; ++r) o[196 * a + 7 * r] = 0.0;
     }
   }
 }
