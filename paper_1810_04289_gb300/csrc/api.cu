@@ -604,7 +604,9 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     cp->nprob = n_problems;
     const double mu_s = mat->E_s / (2.0 * (1.0 + mat->nu_s));
     const double lam_s = mat->E_s * mat->nu_s / ((1.0 + mat->nu_s) * (1.0 - 2.0 * mat->nu_s));
-    cp->mc = MatConst{mat->rho_f, mat->mu_f, mat->rho_s, mat->eta_s, lam_s, mu_s, o.dt};
+    cp->mc = MatConst{mat->rho_f, mat->mu_f, mat->rho_s, mat->eta_s, lam_s, mu_s, o.dt, 1.0 / o.dt,
+                      mat->rho_f / o.dt, 4.0 * (mat->rho_f / o.dt) * (mat->rho_f / o.dt),
+                      16.0 * mat->mu_f * mat->mu_f, 0.25 * mat->rho_f * mat->rho_f};
 
     const int64_t N = mesh->n_nodes, T0 = mesh->n_tets;
     // validate, then order tets fluid first

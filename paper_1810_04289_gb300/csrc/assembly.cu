@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(128) k_elem_residual(MeshDev m, MatConst mc, c
       load_edges(m, n, Xe);
       FluidValues v;
       fluid_values(Xe, q.de, q.u, q.p, q.d, q.u1, q.d1, m.geo[10 * m.T + t], m.geo[11 * m.T + t], mc, v);
-      double F[4][3], Rm[4][3], gr[4], Rc[4], Rh[4][3];
-      fluid_momentum(v, F, Rm);
+      double Rm[4][3], gr[4], Rc[4], Rh[4][3];
+      fluid_momentum(v, Rm);
       fluid_continuity(v, gr, Rc);
       mesh_motion(q.de, g0, vol0, Rh);
 #pragma unroll
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(128) k_elem_residual(MeshDev m, MatConst mc, c
 // the residual of component r of node i where a flag constrains it, else s (a call of
 // its own, taken by the nodes with flags only: inlined, its registers cost the gather
 // more than the call)
-__device__ __noinline__ double constrained(const MeshDev* m, double dt, double t, const double* y, const double* y1,
+__device__ __noinline__ double constrained(const MeshDev* m, double idt, double t, const double* y, const double* y1,
                                            int64_t i, int r, uint32_t f, double s) {
   const double* yi = y + 7 * i;
   if (r >= 3) return (r == 3 ? (f & NF_P_IDENT) : (f & NF_D_ZERO)) ? yi[r] : s;
@@ -172,7 +172,7 @@ __device__ __noinline__ double constrained(const MeshDev* m, double dt, double t
     return yi[r] - U * prof * in[3 + r];
   }
   if (f & NF_U_IDENT) return yi[r];
-  if (f & NF_U_KIN) return yi[r] - (yi[4 + r] - y1[7 * i + 4 + r]) * (1.0 / dt);
+  if (f & NF_U_KIN) return yi[r] - (yi[4 + r] - y1[7 * i + 4 + r]) * idt;
   return s;
 }
 
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256) k_gather_residual(const __grid_constant__
       for (int k = 0; k < 4; ++k) s += v[k];
     }
     for (; c < c1; ++c) s += Fe[7 * (int64_t)nsrc[c] + r];
-    if (f & (NF_U_CONSTR | NF_P_IDENT | NF_D_ZERO)) s = constrained(&m, mc.dt, t, y, y1, i, r, f, s);
+    if (f & (NF_U_CONSTR | NF_P_IDENT | NF_D_ZERO)) s = constrained(&m, mc.idt, t, y, y1, i, r, f, s);
     F[7 * i + r] = s;
   }
 }
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(128) k_jac_values(MeshDev m, MatConst mc, cons
           for (int j = 0; j < 3; ++j) put(JV_GU + 3 * i + j, v.G[i][j]);
           put(JV_GP + i, v.gp[i]);
           // dD/D per unit of d(a_b,k): (2 rho / h)^2 (A_k/4) / (4 D^2)
-          put(JV_TH + i, 0.25 * rho * rho * m.geo[11 * m.T + t] * v.A[i] * (v.ip * v.ip));
+          put(JV_TH + i, mc.ca * m.geo[11 * m.T + t] * v.A[i] * (v.ip * v.ip));
         }
         put(JV_SC + 0, v.vol);
         put(JV_SC + 1, v.c);
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(128) k_jac_values(MeshDev m, MatConst mc, cons
 #pragma unroll
         for (int i = 0; i < 3; ++i) de[k][i] = y[7 * (int64_t)n[k + 1] + 4 + i] - y[7 * (int64_t)n[0] + 4 + i];
       wall_stress(de, g0, mc, F, S);
-      const double idt = 1.0 / mc.dt, k20 = vol0 * (1.0 / 20.0) * (mc.rho_s * idt * idt + mc.eta_s * idt);
+      const double idt = mc.idt, k20 = vol0 * (1.0 / 20.0) * (mc.rho_s * idt * idt + mc.eta_s * idt);
       double fa[4][3], Sg[4][3];
 #pragma unroll
       for (int a = 0; a < 4; ++a)
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(128) k_jac_values(MeshDev m, MatConst mc, cons
 // three of d columns, one of p columns): a u column needs 126 FP64 instructions, a d
 // column 170, a p column 45, where a mixed warp would run all three.
 template <int KIND>  // 0: u column, 1: p, 2: d
-__device__ __forceinline__ void fluid_column(const double* s, int b, int kk, double idt, double rho, double mu,
+__device__ __forceinline__ void fluid_column(const double* s, int b, int kk, double idt, double ridt, double rho, double mu,
                                              const uint32_t f[4], double* o) {
   constexpr bool U = KIND == 0, P = KIND == 1, D = KIND == 2;
   const double* gb = s + JV_G + 3 * b;
@@ -464,7 +464,7 @@ __device__ __forceinline__ void fluid_column(const double* s, int b, int kk, dou
     const double Gik = P ? 0.0 : s[JV_GU + 3 * i + kk];
     al[i] = D ? -Gik : 0.0;
     be[i] = P ? 0.0 : rho * eta * Gik;
-    if (U && i == kk) be[i] += rho * idt;
+    if (U && i == kk) be[i] += ridt;
     dr[i] = P ? tv * gb[i] : tv * (0.25 * be[i] + (D ? 0.25 * rho * s[JV_S + b] * al[i] + gam * gb[i] : 0.0));
     if (U && i == kk) dr[i] += tv * (0.25 * rho * s[JV_S + b]);
   }
@@ -536,10 +536,10 @@ k_elem_jacobian64(MeshDev m, MatConst mc, const double* __restrict__ val, double
     load_tet(m, t, n, f);
     double* o = Ke + 784 * (t - t0) + 49 * b + k;
     if (t < m.Tf) {
-      const double idt = 1.0 / mc.dt;
-      if (kind == 0) fluid_column<0>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
-      else if (kind == 2) fluid_column<2>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
-      else fluid_column<1>(s, b, kk, idt, mc.rho_f, mc.mu_f, f, o);
+      const double idt = mc.idt;
+      if (kind == 0) fluid_column<0>(s, b, kk, idt, mc.ridt, mc.rho_f, mc.mu_f, f, o);
+      else if (kind == 2) fluid_column<2>(s, b, kk, idt, mc.ridt, mc.rho_f, mc.mu_f, f, o);
+      else fluid_column<1>(s, b, kk, idt, mc.ridt, mc.rho_f, mc.mu_f, f, o);
     } else if (kind == 2) {
       // d column: |K0| (F S)' g0_a and the inertia
       const double vmu = mc.mu_s * m.geo[9 * m.T + t], vlam = mc.lam_s * m.geo[9 * m.T + t];

@@ -28,6 +28,9 @@ namespace fsi {
 
 struct MatConst {
   double rho_f, mu_f, rho_s, eta_s, lam_s, mu_s, dt;
+  // products of the above that the FP64 kernels need in every thread (1/dt, rho/dt,
+  // (2 rho/dt)^2, (4 mu)^2, rho^2/4: an FP64 division alone is a dozen instructions)
+  double idt, ridt, ct2, cv2, ca;
 };
 
 // barycentric weights of the degree-2 4-point rule: alpha at its own vertex,
@@ -263,7 +266,7 @@ struct FluidValues {
   double g[4][3], vol;       // current gradients and volume
   double G[3][3], gp[3], div;
   double a[4][3], A[3];      // advection velocity at the vertices, its sum
-  double n[4][3], W[3];      // inertia at the vertices, N + 5 grad p
+  double n[4][3], N[3], W[3];  // inertia at the vertices, its sum, N + 5 grad p
   double arg, ip;            // D^2, 1/D
   double c, tc;              // tau_M |K|/20, tau_C rho
   double Q[3][3], P[3][3];
@@ -278,7 +281,7 @@ __device__ __forceinline__ void fluid_values(const double Xe[3][3], const double
                                              const double p[4], const double d[4][3], const double u1[4][3],
                                              const double d1[4][3], double h2, double ih2, const MatConst& m,
                                              FluidValues& v) {
-  const double rho = m.rho_f, idt = 1.0 / m.dt;
+  const double rho = m.rho_f, idt = m.idt;
   double e[3][3], x[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k)
@@ -315,22 +318,19 @@ __device__ __forceinline__ void fluid_values(const double Xe[3][3], const double
     v.A[i] = (v.a[0][i] + v.a[1][i]) + (v.a[2][i] + v.a[3][i]);
   }
   // D^2 with the centroid's advection velocity A/4
-  const double ct = 2.0 * rho * idt, cv = 4.0 * m.mu_f * ih2;
-  v.arg = (ct * ct + cv * cv) +
-          (0.25 * rho * rho * ih2) * (v.A[0] * v.A[0] + v.A[1] * v.A[1] + v.A[2] * v.A[2]);
+  v.arg = m.ct2 + (m.cv2 * ih2) * ih2 + (m.ca * ih2) * (v.A[0] * v.A[0] + v.A[1] * v.A[1] + v.A[2] * v.A[2]);
   v.ip = rsqrt(v.arg);
   v.tc = (h2 * (1.0 / 12.0)) * (v.arg * v.ip);
   v.c = rho * v.ip * v.vol * 0.05;
-  const double ridt = rho * idt;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const double r0 = rho * v.G[i][0], r1 = rho * v.G[i][1], r2 = rho * v.G[i][2];
 #pragma unroll
     for (int b = 0; b < 4; ++b)
-      v.n[b][i] = ridt * (u[b][i] - u1[b][i]) + r0 * v.a[b][0] + r1 * v.a[b][1] + r2 * v.a[b][2];
-    const double N = (v.n[0][i] + v.n[1][i]) + (v.n[2][i] + v.n[3][i]);
-    v.W[i] = N + 5.0 * v.gp[i];
-    v.r[i] = 0.25 * N + v.gp[i];
+      v.n[b][i] = m.ridt * (u[b][i] - u1[b][i]) + r0 * v.a[b][0] + r1 * v.a[b][1] + r2 * v.a[b][2];
+    v.N[i] = (v.n[0][i] + v.n[1][i]) + (v.n[2][i] + v.n[3][i]);
+    v.W[i] = v.N[i] + 5.0 * v.gp[i];
+    v.r[i] = 0.25 * v.N[i] + v.gp[i];
   }
   const double pc = 0.25 * ((p[0] + p[1]) + (p[2] + p[3]));
   const double iso = v.vol * (v.tc * v.div - pc), vm = v.vol * m.mu_f;
@@ -355,9 +355,24 @@ __device__ __forceinline__ void fluid_momentum(const FluidValues& v, double F[4]
 #pragma unroll
     for (int a = 1; a < 4; ++a) F[a][i] = v.P[i][0] * v.g[a][0] + v.P[i][1] * v.g[a][1] + v.P[i][2] * v.g[a][2];
     F[0][i] = rest(F[1][i], F[2][i], F[3][i]);
-    const double N = v.W[i] - 5.0 * v.gp[i];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) Rm[a][i] = k20 * (N + v.n[a][i]) + F[a][i];
+    for (int a = 0; a < 4; ++a) Rm[a][i] = k20 * (v.N[i] + v.n[a][i]) + F[a][i];
+  }
+}
+
+// the same Rm alone, |K|/20 N taken into the products' chains
+__device__ __forceinline__ void fluid_momentum(const FluidValues& v, double Rm[4][3]) {
+  const double k20 = 0.05 * v.vol;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double kN = k20 * v.N[i];
+    double f[4];
+#pragma unroll
+    for (int a = 1; a < 4; ++a)
+      f[a] = fma(v.P[i][2], v.g[a][2], fma(v.P[i][1], v.g[a][1], fma(v.P[i][0], v.g[a][0], kN)));
+    f[0] = fma(4.0, kN, rest(f[1], f[2], f[3]));
+#pragma unroll
+    for (int a = 0; a < 4; ++a) Rm[a][i] = fma(k20, v.n[a][i], f[a]);
   }
 }
 
@@ -415,7 +430,7 @@ __device__ __forceinline__ void wall_residual(const double de[3][3], const doubl
                                               const MatConst& m, double Rw[4][3]) {
   double F[3][3], S[3][3];
   wall_stress(de, g0, m, F, S);
-  const double idt = 1.0 / m.dt;
+  const double idt = m.idt;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     double P[3], acc[4];

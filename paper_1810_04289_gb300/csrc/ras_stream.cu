@@ -892,6 +892,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
     }
   } else {
     double A0[8], A1[8], acc = 0.0;
+    bool used = false;  // the warp has had blocks of the row
 #pragma unroll
     for (int e = 0; e < 8; ++e) A0[e] = A1[e] = 0.0;
     auto fetch = [&](double (&A)[8], uint32_t code) {
@@ -912,13 +913,17 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
           for (int e = 0; e < 4; ++e) load16(&x[2 * e], xp + 2 * e);
           const double y = row_fma(A, x, acc);
           if (b < nf) acc = y;
+          used = true;
         }
         if (code & ENTRY_END) {
-          acc += __shfl_xor_sync(0xffffffffu, acc, 16);
-          acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+          if (used) {  // (no additions of zeros: they take the FP64 pipe as long)
+            acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+          }
           par ^= 1;
           if (lane < 7) part[par][v][c] = acc;
           acc = 0.0;
+          used = false;
         }
         if (code & (ENTRY_END | ENTRY_STAGE)) __syncthreads();
         if (code & ENTRY_STAGE) next_stage();
