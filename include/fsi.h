@@ -130,7 +130,8 @@ typedef struct {
                              part; the parts of one level are solved side by side) */
   int32_t factor_mode;    /* ILU factorisation kernel: 0 automatic (4 when the
                              subdomains are dissected, ordering 3, and its rows fit in
-                             shared memory, else 3); rows in order with 1 pivots and
+                             shared memory; else rows in order, pipelined, where its
+                             copies fit; else 3); rows in order with 1 pivots and
                              update sources prefetched into shared memory, 2 sources
                              only, 3 neither (the row alone in shared memory); 4 the
                              parts of each dissection level factored side by side. A
@@ -147,11 +148,13 @@ typedef struct {
                              level-scheduled one); 1 streamed (FSI_ERR_ARG if it does
                              not fit); 2 level-scheduled. Same arithmetic, same result
                              up to the order of the row sums. */
-  int32_t stage_blocks;   /* streamed apply: factor blocks per ring stage, 0 = automatic
-                             (sized from the shared memory left at ceil(n_subdomains / 152),
-                             at most 8, CTAs per SM) */
-  int32_t stages;         /* streamed apply: ring stages in flight per warp, 2..8,
-                             0 = automatic (2) */
+  int32_t stage_blocks;   /* streamed apply: factor blocks per ring stage of dissected
+                             subdomains (ordering 3), and where a row's FP32 sum is cut
+                             into pieces that are added up (every ordering); 0 =
+                             automatic (from the shared memory left at
+                             ceil(n_subdomains / 152), at most 8, CTAs per SM) */
+  int32_t stages;         /* streamed apply: ring stages in flight per warp of dissected
+                             subdomains, 2..8, 0 = automatic (2) */
   int32_t orth;           /* Arnoldi orthogonalisation, FP64 (Sec. 4: classical
                              Gram-Schmidt twice): 0 the new vector's norm taken from the
                              second pass (dots; update; dots with ||w||^2; update and
