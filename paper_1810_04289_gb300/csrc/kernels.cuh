@@ -174,13 +174,18 @@ struct SegDev {
   const int64_t* chunk_beg;  // [n_chunks+1] first dof of each chunk (chunks never straddle problems)
   const int64_t* prob_chunk; // [P+1] chunks of each problem
   const int32_t* node_prob;  // [N] problem of each node
-  int* counter;              // [P * SEG_GROUPS] blocks done per (problem, vector group); zero between launches
+  int* counter;              // [P][SEG_COUNTERS] blocks done per vector group, then groups done; zero between launches
 };
 constexpr int SEG_GROUPS = 9;  // vector groups of 8 in one multi-dot (restart <= 64 -> at most 65 vectors)
-// out[p * ldo + k] = V_k . w for k < nv (and, with_self, out[p * ldo + nv] = w . w);
-// returns the number of kernels launched (1 or 2)
-int launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w, double* partial,
-                    double* out, int32_t ldo, const int* guard, cudaStream_t s, int with_self = 0);
+constexpr int SEG_COUNTERS = SEG_GROUPS + 1;
+// out[p * ldo + k] = V_k . w for k < nv (and, with_self = 1, out[p * ldo + nv] = w . w)
+void launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w, double* partial,
+                     double* out, int32_t ldo, const int* guard, cudaStream_t s, int with_self = 0);
+// the same with w . w, then the norm of w - V out as sqrt(w . w - ||V . w||^2) into hsub where
+// that is safe, its reciprocal into inv, else unsafe[p] = 1 (see krylov.cu)
+void launch_seg_mdot_norm(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w,
+                          double* partial, double* out, int32_t ldo, double* hsub, int64_t ldsub, double* inv,
+                          int* unsafe, int force, const int* guard, cudaStream_t s);
 // selective reorthogonalisation test after one Gram-Schmidt pass (see krylov.cu)
 void launch_seg_reorth_decide(int32_t P, const double* ws, const double* nrm, int32_t ldn, double* hb, int32_t lda,
                               int32_t j, const int* active, int* flag, cudaStream_t s);
@@ -189,23 +194,17 @@ void launch_seg_norm(const SegDev& sg, const double* x, double* partial, double*
 // w -= V h per problem, then w *= scal[p] (scal optional)
 void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, int64_t ldv, const double* h,
                       int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal = nullptr);
-// the new Arnoldi vector's norm as sqrt(||w||^2 - ||h2||^2) where that is safe (see krylov.cu)
-void launch_seg_norm_pythagoras(int32_t P, const double* hb, int32_t lda, int32_t j, double* hsub, int64_t ldsub,
-                                double* inv, int* unsafe, int* flag, int force, const int* guard, cudaStream_t s);
-// where *guard says so: the norms of the problems with unsafe[p] formed from w itself into
-// hsub, and w divided by them
-void launch_seg_norm_fallback(const SegDev& sg, double* w, const int* unsafe, double* hsub,
-                              int64_t ldsub, const int* guard, cudaStream_t s);
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
                           double* y, const int* guard, cudaStream_t s);
 
 void launch_seg_cycle_init(int32_t P, double* g, int32_t ldg, const double* beta, const double* target, int* active,
                            int* kcols, int* any, cudaStream_t s);
 // column j of each active problem's Hessenberg = a + b (the two Gram-Schmidt passes, lda apart per
-// problem), then the Givens update
+// problem), then the Givens update; first, where unsafe[p] (optional), ||w_p|| into H and w_p divided by it
 void launch_seg_givens(int32_t P, const double* a, const double* b, int32_t lda, double* H, int32_t ldh, int32_t m,
                        int32_t j, double* cs, double* sn, double* g, double* res, const double* target, int* active,
-                       int* kcols, int* any, cudaStream_t s);
+                       int* kcols, int* any, const SegDev& sg, double* w, const int* unsafe, const int* guard,
+                       cudaStream_t s);
 void launch_seg_lsq(int32_t P, const double* H, int32_t ldh, int32_t m, const int* kcols, const double* g, double* y,
                     cudaStream_t s);
 void launch_seg_update_x(const SegDev& sg, int64_t n, const double* Z, int64_t ldz, const double* y, int32_t m,

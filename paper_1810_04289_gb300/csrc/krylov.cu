@@ -4,8 +4,7 @@
 // block per chunk, and the last block of a problem to finish (a per-problem
 // counter) sums that problem's chunk partials in fixed order, so results are
 // bitwise reproducible run to run, independent problems never mix, and a
-// reduction is one launch per group width (a multi-dot: one for its full groups
-// of 8 vectors, one for a partial last group).
+// reduction is one launch (a multi-dot's groups of 8 vectors side by side).
 // Per-problem Arnoldi scalars: H (column-major (m+1) x m per problem), g, Givens
 // cs/sn, residual estimates, stop flags.
 //
@@ -52,26 +51,59 @@ __device__ __forceinline__ void warp_sums(double (&v)[W]) {
   for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
 }
 
-// out[p * ldo + k] = sum over the dofs of problem p of V_k . w (V null: w . w,
-// and take_sqrt gives the 2-norm). Block (c, y) forms the partials of chunk c
-// for the vectors of group g = g0 + y, 8g .. 8g + W - 1 (those below nv); the
-// last block of problem p for group g sums the problem's partials (one warp per
-// vector, lanes over the chunks in fixed order) and resets the counter.
-// With nself = 1 there is one more output, index nv_v = nv - 1: w . w itself.
-// Each thread takes U elements per trip (loads in flight); the kernel is bound by
-// the FP64 pipe (one FMA per loaded operand) or, for narrow groups, by latency,
-// so the full groups run with W = 8, U = 2 and a partial last group in its own
-// launch with a narrower W and a deeper U (fewer registers, more loads in flight).
+// The norm of a Gram-Schmidt step's new vector from its second pass (k_seg_mdot):
+// after w1 = w0 - V h1 the second pass's dots h2 = V^T w1 come with ||w1||^2 (the
+// self product), and since V is orthonormal, ||w1 - V h2||^2 = ||w1||^2 - ||h2||^2.
+// The second update then scales in the same sweep (k_seg_maxpy with scal), so the
+// step needs no norm or scaling sweep. Where ||w1||^2 - ||h2||^2 keeps at least 3/4
+// of ||w1||^2 (the subtraction then loses under two bits) hsub[p * ldsub] is its
+// square root and inv[p] the reciprocal (0 for a zero norm); elsewhere (only as a
+// Krylov space is exhausted; for every problem with force = 1, tests of that path)
+// inv[p] = 1 and unsafe[p] = 1: k_seg_givens then forms the norm from the updated vector.
+struct NewNorm {
+  double* hsub;  // null: no norm wanted
+  int64_t ldsub;
+  double* inv;
+  int* unsafe;
+  int force;
+};
+
+// one warp: q = ||h2||^2 and s = ||w1||^2, written by other blocks of this launch
+__device__ void new_norm(const NewNorm& N, int p, const double* h, int nv) {
+  const int lane = threadIdx.x & 31;
+  const double s = __ldcg(h + nv);
+  double q = 0.0;
+  for (int k = lane; k < nv; k += 32) {
+    const double v = __ldcg(h + k);
+    q += v * v;
+  }
+  q = warp_sum(q);
+  if (lane == 0) {
+    const double b2 = s - q;
+    if (!N.force && b2 >= 0.75 * s) {
+      const double b = sqrt(b2);
+      N.hsub[(int64_t)p * N.ldsub] = b;
+      N.inv[p] = b > 0.0 ? 1.0 / b : 0.0;
+      N.unsafe[p] = 0;
+    } else {
+      N.inv[p] = 1.0;
+      N.unsafe[p] = 1;
+    }
+  }
+}
+
+// The partials of chunk c for the vectors of group g, 8g .. 8g + W - 1 (those below nv),
+// and, in the last block of problem p for group g, the sums of the problem's partials
+// (one warp per vector, lanes over the chunks in fixed order). Each thread takes U
+// elements per trip (loads in flight).
 template <int W, int U>
-__global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, int32_t g0, const double* __restrict__ V,
-                                                 int64_t ldv, const double* __restrict__ w,
-                                                 double* __restrict__ partial, double* __restrict__ out,
-                                                 int32_t ldo, int take_sqrt, int nself, const int* guard) {
-  if (off(guard)) return;
+__device__ __forceinline__ void dots(const SegDev& sg, int32_t nv, int g, int n_groups, const double* __restrict__ V,
+                                     int64_t ldv, const double* __restrict__ w, double* __restrict__ partial,
+                                     double* __restrict__ out, int32_t ldo, int take_sqrt, int nself,
+                                     const NewNorm& N) {
   __shared__ double red[W][RB / 32];
   __shared__ int s_last;
   const int c = blockIdx.x;
-  const int g = g0 + blockIdx.y;
   const int k0 = g * MD;
   const int64_t i0 = sg.chunk_beg[c], i1 = sg.chunk_beg[c + 1];
   double acc[W];
@@ -115,8 +147,8 @@ __global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, int32_t 
   __syncthreads();
   const int p = sg.node_prob[i0 / 7];
   const int64_t c0 = sg.prob_chunk[p], c1 = sg.prob_chunk[p + 1];
-  int* cnt = sg.counter + (int64_t)p * SEG_GROUPS + g;
-  if (threadIdx.x == 0) s_last = atomicAdd(cnt, 1) == (int)(c1 - c0) - 1;
+  int* cnt = sg.counter + (int64_t)p * SEG_COUNTERS;
+  if (threadIdx.x == 0) s_last = atomicAdd(cnt + g, 1) == (int)(c1 - c0) - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -127,7 +159,42 @@ __global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, int32_t 
     v = warp_sum(v);
     if (lane == 0) out[(int64_t)p * ldo + k] = take_sqrt ? sqrt(v) : v;
   }
-  if (threadIdx.x == 0) *cnt = 0;
+  if (threadIdx.x == 0) cnt[g] = 0;
+  if (!N.hsub) return;
+  // the last of the problem's groups takes the norm: publish the sums, count the group in
+  __threadfence();
+  __syncthreads();
+  if (warp > 0) return;
+  int last = 0;
+  if (lane == 0) last = n_groups == 1 || atomicAdd(cnt + SEG_GROUPS, 1) == n_groups - 1;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __threadfence();
+  new_norm(N, p, out + (int64_t)p * ldo, nvv);
+  if (lane == 0) cnt[SEG_GROUPS] = 0;
+}
+
+// out[p * ldo + k] = sum over the dofs of problem p of V_k . w (V null: w . w,
+// and take_sqrt gives the 2-norm). With nself = 1 there is one more output, index
+// nv - 1: w . w itself. Block (c, g) takes chunk c and the g-th group of 8 vectors;
+// the last group has W of them at most (W the next power of two).
+// Bound by the FP64 pipe (one FMA per loaded operand) or, for narrow groups, by
+// latency: the full groups take W = 8, U = 2, a partial last group a narrower W and a
+// deeper U (fewer products, more loads in flight). All groups and the new norm in one
+// launch: as two launches and one more for the norm the narrow group ran after the full
+// ones with most of the chip idle, and each launch of the cycle's graph costs 1.4 to 4 us
+// (seven launches per GMRES iteration instead of eleven: a mixed step of the 46,657-node tube
+// 157.7 -> 152.7 ms, an FP64 step of the 12 x 8 x 4 tube 100.6 -> 98.2 ms; the same bits).
+template <int W, int U>
+__global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, const double* __restrict__ V, int64_t ldv,
+                                                 const double* __restrict__ w, double* __restrict__ partial,
+                                                 double* __restrict__ out, int32_t ldo, int take_sqrt, int nself,
+                                                 NewNorm N, const int* guard) {
+  if (off(guard)) return;
+  const int g = blockIdx.y, G = gridDim.y;
+  if (W < MD && g < G - 1)
+    dots<MD, 2>(sg, nv, g, G, V, ldv, w, partial, out, ldo, take_sqrt, nself, N);
+  else
+    dots<W, U>(sg, nv, g, G, V, ldv, w, partial, out, ldo, take_sqrt, nself, N);
 }
 
 // w_i -= sum_k h[p(i)][k] V_k[i], then (scal non-null) w_i *= scal[p(i)]
@@ -161,79 +228,6 @@ __global__ void k_seg_scale_inv(SegDev sg, int64_t n, const double* __restrict__
     }
     y[i] = x[i] * inv;
   }
-}
-
-// Classical Gram-Schmidt twice with the new vector's norm taken from the second
-// pass: after w1 = w0 - V h1 the second pass's dots h2 = V^T w1 come with
-// ||w1||^2 (k_seg_mdot with the self product), and since V is orthonormal,
-// ||w1 - V h2||^2 = ||w1||^2 - ||h2||^2. The second update then scales in the
-// same sweep (k_seg_maxpy with scal), so the step needs no norm or scaling sweep.
-//
-// For every problem p, hb[p][0..j] = h2 and hb[p][j+1] = ||w1||^2: where
-// ||w1||^2 - ||h2||^2 keeps at least 3/4 of ||w1||^2 (the subtraction then loses
-// under two bits) H[p][j+1][j] (hsub + p * ldsub) is its square root and inv[p]
-// the reciprocal (0 for a zero norm); elsewhere (only as a Krylov space is
-// exhausted; for every problem with force = 1, tests of that path) inv[p] = 1,
-// unsafe[p] = 1 and *flag = 1: the norm is then formed from the updated vector
-// by k_seg_norm_fallback.
-__global__ void k_seg_norm_pythagoras(int32_t P, const double* __restrict__ hb, int32_t lda, int32_t j,
-                                      double* __restrict__ hsub, int64_t ldsub, double* __restrict__ inv,
-                                      int* __restrict__ unsafe, int* __restrict__ flag, int force,
-                                      const int* guard) {
-  __shared__ int s_any;
-  if (off(guard)) {
-    if (threadIdx.x == 0) *flag = 0;
-    return;
-  }
-  if (threadIdx.x == 0) s_any = 0;
-  __syncthreads();
-  // one warp per problem
-  for (int p = threadIdx.x >> 5; p < P; p += blockDim.x >> 5) {
-    const int lane = threadIdx.x & 31;
-    const double* h = hb + (int64_t)p * lda;
-    const double s = h[j + 1];
-    double q = 0.0;
-    for (int k = lane; k <= j; k += 32) q += h[k] * h[k];
-    q = warp_sum(q);
-    if (lane == 0) {
-      const double b2 = s - q;
-      if (!force && b2 >= 0.75 * s) {
-        const double b = sqrt(b2);
-        hsub[(int64_t)p * ldsub] = b;
-        inv[p] = b > 0.0 ? 1.0 / b : 0.0;
-        unsafe[p] = 0;
-      } else {
-        inv[p] = 1.0;
-        unsafe[p] = 1;
-        atomicOr(&s_any, 1);
-      }
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *flag = s_any;
-}
-
-// the fallback of k_seg_norm_pythagoras, one block per problem (a rare path: one
-// launch that mostly returns at once in place of three): where unsafe[p],
-// H[p][j+1][j] = ||w_p|| of the updated vector and w_p /= it (0 for a zero norm)
-__global__ void __launch_bounds__(1024) k_seg_norm_fallback(SegDev sg, double* __restrict__ w,
-                                                            const int* __restrict__ unsafe,
-                                                            double* __restrict__ hsub, int64_t ldsub,
-                                                            const int* guard) {
-  if (off(guard)) return;
-  const int p = blockIdx.x;
-  if (!unsafe[p]) return;
-  __shared__ double red[32];
-  const int64_t i0 = sg.chunk_beg[sg.prob_chunk[p]], i1 = sg.chunk_beg[sg.prob_chunk[p + 1]];
-  double s = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += w[i] * w[i];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  s = warp_sum(red[threadIdx.x & 31]);
-  const double nrm = sqrt(s), inv = nrm != 0.0 ? 1.0 / nrm : 0.0;
-  if (threadIdx.x == 0) hsub[(int64_t)p * ldsub] = nrm;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] *= inv;
 }
 
 // start of a cycle for every problem: g = beta e_1, active while beta > target
@@ -284,16 +278,40 @@ __global__ void k_seg_reorth_decide(int32_t P, const double* __restrict__ ws, co
 // One warp per problem (up to 32 at a time): the lanes read the column's sums and the
 // rotations at once and hand them to the chain by shuffles (read one by one inside the
 // chain of rotations they cost an L2 latency each: 7.3 -> 5.9 us for one problem).
+//
+// Where unsafe[p] (non-null; set by new_norm, a rare path), the whole block first forms
+// H[p][j+1][j] = ||w_p|| of the updated vector and scales w_p by its reciprocal (0 for a
+// zero norm); as a launch of its own it cost 2 us a step for nothing.
 __global__ void __launch_bounds__(1024) k_seg_givens(int32_t P, const double* __restrict__ ha,
                                                      const double* __restrict__ hb, int32_t lda,
                                                      double* __restrict__ H, int32_t ldh, int32_t m, int32_t j,
                                                      double* __restrict__ cs, double* __restrict__ sn,
                                                      double* __restrict__ g, double* __restrict__ res,
                                                      const double* __restrict__ target, int* __restrict__ active,
-                                                     int* __restrict__ kcols, int* __restrict__ any) {
+                                                     int* __restrict__ kcols, int* __restrict__ any, SegDev sg,
+                                                     double* __restrict__ w, const int* __restrict__ unsafe,
+                                                     const int* guard) {
   __shared__ int s_any;
   const int lane = threadIdx.x & 31;
+  if (off(guard)) return;  // *any is this flag, 0 already
   if (threadIdx.x == 0) s_any = 0;
+  if (unsafe) {
+    __shared__ double red[32];
+    for (int p = 0; p < P; ++p) {
+      if (!unsafe[p]) continue;
+      const int64_t i0 = sg.chunk_beg[sg.prob_chunk[p]], i1 = sg.chunk_beg[sg.prob_chunk[p + 1]];
+      double s = 0.0;
+      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += w[i] * w[i];
+      s = warp_sum(s);
+      if (lane == 0) red[threadIdx.x >> 5] = s;
+      __syncthreads();
+      s = warp_sum(red[lane]);
+      const double nrm = sqrt(s), inv = nrm != 0.0 ? 1.0 / nrm : 0.0;
+      if (threadIdx.x == 0) H[(int64_t)p * ldh * m + (int64_t)j * ldh + j + 1] = nrm;
+      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] *= inv;
+      __syncthreads();
+    }
+  }
   __syncthreads();
   for (int p = threadIdx.x >> 5; p < P; p += blockDim.x >> 5) {
     if (!active[p]) continue;
@@ -421,40 +439,38 @@ inline int grid_for(int64_t work, int block) {
   return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-// groups of 8 vectors in one launch, then the partial last group (r vectors) in a
-// launch of its own width
-void mdot_groups(const SegDev& sg, int32_t n, const double* V, int64_t ldv, const double* w, double* partial,
-                 double* out, int32_t ldo, int take_sqrt, int nself, const int* guard, cudaStream_t s) {
-  const unsigned nch = (unsigned)sg.n_chunks;
-  const int full = n / MD, r = n % MD;
-  if (full > 0)
-    k_seg_mdot<8, 2><<<dim3(nch, full), RB, 0, s>>>(sg, n, 0, V, ldv, w, partial, out, ldo, take_sqrt, nself, guard);
-  if (r == 0) return;
-  const dim3 g1(nch, 1);
+// one launch; W and U by the size r of the last group
+void mdot(const SegDev& sg, int32_t n, const double* V, int64_t ldv, const double* w, double* partial, double* out,
+          int32_t ldo, int take_sqrt, int nself, const NewNorm& N, const int* guard, cudaStream_t s) {
+  const dim3 grid((unsigned)sg.n_chunks, (unsigned)((n + MD - 1) / MD));
+  const int r = n % MD;
   if (r == 1)
-    k_seg_mdot<1, 8><<<g1, RB, 0, s>>>(sg, n, full, V, ldv, w, partial, out, ldo, take_sqrt, nself, guard);
+    k_seg_mdot<1, 8><<<grid, RB, 0, s>>>(sg, n, V, ldv, w, partial, out, ldo, take_sqrt, nself, N, guard);
   else if (r == 2)
-    k_seg_mdot<2, 4><<<g1, RB, 0, s>>>(sg, n, full, V, ldv, w, partial, out, ldo, take_sqrt, nself, guard);
-  else if (r <= 4)
-    k_seg_mdot<4, 4><<<g1, RB, 0, s>>>(sg, n, full, V, ldv, w, partial, out, ldo, take_sqrt, nself, guard);
+    k_seg_mdot<2, 4><<<grid, RB, 0, s>>>(sg, n, V, ldv, w, partial, out, ldo, take_sqrt, nself, N, guard);
+  else if (r == 3 || r == 4)
+    k_seg_mdot<4, 4><<<grid, RB, 0, s>>>(sg, n, V, ldv, w, partial, out, ldo, take_sqrt, nself, N, guard);
   else
-    k_seg_mdot<8, 2><<<g1, RB, 0, s>>>(sg, n, full, V, ldv, w, partial, out, ldo, take_sqrt, nself, guard);
+    k_seg_mdot<8, 2><<<grid, RB, 0, s>>>(sg, n, V, ldv, w, partial, out, ldo, take_sqrt, nself, N, guard);
 }
 
 }  // namespace
 
-int launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w, double* partial,
-                    double* out, int32_t ldo, const int* guard, cudaStream_t s, int with_self) {
-  const int n = nv + (with_self ? 1 : 0);
-  mdot_groups(sg, n, V, ldv, w, partial, out, ldo, 0, with_self ? 1 : 0, guard, s);
-  return (n / MD > 0 ? 1 : 0) + (n % MD > 0 ? 1 : 0);
+void launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w, double* partial,
+                     double* out, int32_t ldo, const int* guard, cudaStream_t s, int with_self) {
+  mdot(sg, nv + with_self, V, ldv, w, partial, out, ldo, 0, with_self, NewNorm{}, guard, s);
+}
+
+void launch_seg_mdot_norm(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w,
+                          double* partial, double* out, int32_t ldo, double* hsub, int64_t ldsub, double* inv,
+                          int* unsafe, int force, const int* guard, cudaStream_t s) {
+  mdot(sg, nv + 1, V, ldv, w, partial, out, ldo, 0, 1, NewNorm{hsub, ldsub, inv, unsafe, force}, guard, s);
 }
 
 void launch_seg_norm(const SegDev& sg, const double* x, double* partial, double* out, int32_t ldo,
                      const int* guard, cudaStream_t s) {
-  mdot_groups(sg, 1, nullptr, 0, x, partial, out, ldo, 1, 0, guard, s);
+  mdot(sg, 1, nullptr, 0, x, partial, out, ldo, 1, 0, NewNorm{}, guard, s);
 }
-
 
 void launch_seg_reorth_decide(int32_t P, const double* ws, const double* nrm, int32_t ldn, double* hb, int32_t lda,
                               int32_t j, const int* active, int* flag, cudaStream_t s) {
@@ -464,16 +480,6 @@ void launch_seg_reorth_decide(int32_t P, const double* ws, const double* nrm, in
 void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, int64_t ldv, const double* h,
                       int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal) {
   k_seg_maxpy<<<grid_for(n, 256), 256, 0, s>>>(sg, n, nv, V, ldv, h, ldh, w, scal, guard);
-}
-
-void launch_seg_norm_pythagoras(int32_t P, const double* hb, int32_t lda, int32_t j, double* hsub, int64_t ldsub,
-                                double* inv, int* unsafe, int* flag, int force, const int* guard, cudaStream_t s) {
-  k_seg_norm_pythagoras<<<1, 32 * (P < 32 ? P : 32), 0, s>>>(P, hb, lda, j, hsub, ldsub, inv, unsafe, flag, force, guard);
-}
-
-void launch_seg_norm_fallback(const SegDev& sg, double* w, const int* unsafe, double* hsub, int64_t ldsub,
-                              const int* guard, cudaStream_t s) {
-  k_seg_norm_fallback<<<sg.P, 1024, 0, s>>>(sg, w, unsafe, hsub, ldsub, guard);
 }
 
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
@@ -488,8 +494,10 @@ void launch_seg_cycle_init(int32_t P, double* g, int32_t ldg, const double* beta
 
 void launch_seg_givens(int32_t P, const double* a, const double* b, int32_t lda, double* H, int32_t ldh, int32_t m,
                        int32_t j, double* cs, double* sn, double* g, double* res, const double* target, int* active,
-                       int* kcols, int* any, cudaStream_t s) {
-  k_seg_givens<<<1, 32 * (P < 32 ? P : 32), 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res, target, active, kcols, any);
+                       int* kcols, int* any, const SegDev& sg, double* w, const int* unsafe, const int* guard,
+                       cudaStream_t s) {
+  k_seg_givens<<<1, unsafe ? 1024 : 32 * (P < 32 ? P : 32), 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res, target,
+                                                                    active, kcols, any, sg, w, unsafe, guard);
 }
 
 void launch_seg_lsq(int32_t P, const double* H, int32_t ldh, int32_t m, const int* kcols, const double* g, double* y,
