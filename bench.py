@@ -85,7 +85,7 @@ TUNED = {
 # now, keyed by (workload, phase, precision, subdomains, ILU level, ordering);
 # the summary that holds the capture is named beside it
 NCU_TRAFFIC = {
-    ("tree-3gen", "pcapply", "mixed", 16384, 1, 1): (27.41e9, "profiles/k_ras_apply_stream_tree-3gen.md"),
+    ("tree-3gen", "pcapply", "mixed", 16384, 1, 1): (27.36e9, "profiles/k_ras_apply_chain_tree-3gen.md"),
 }
 
 
