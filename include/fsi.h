@@ -142,7 +142,10 @@ typedef struct {
                              issues nothing, so the apply's bounded wait runs out and
                              the call returns FSI_ERR_TIMEOUT; 2 = Gram-Schmidt orth 0
                              forms every new vector's norm from the updated vector (its
-                             fallback path); 0 otherwise */
+                             fallback path); 3 = the pipelined factorisation's copies
+                             are never issued, 4 = every wait in it gives up at once:
+                             its bounded waits run out and the call that builds the
+                             factors returns FSI_ERR_TIMEOUT; 0 otherwise */
   int32_t apply_mode;     /* preconditioner apply kernel: 0 automatic (the streamed
                              apply when its shared-memory footprint fits, else the
                              level-scheduled one); 1 streamed (FSI_ERR_ARG if it does

@@ -354,10 +354,10 @@ __device__ __forceinline__ void pipe_bar_init(uint64_t* b, uint32_t n) {
 __device__ __forceinline__ void pipe_bar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
 }
-// bounded wait: false if the phase did not complete in time
-__device__ __forceinline__ bool pipe_bar_wait(uint64_t* b, uint32_t parity) {
+// bounded wait: false if the phase did not complete within `tries` looks
+__device__ __forceinline__ bool pipe_bar_wait(uint64_t* b, uint32_t parity, uint32_t tries) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(b);
-  for (uint32_t it = 0; it < (1u << 20); ++it) {
+  for (uint32_t it = 0; it < tries; ++it) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -392,6 +392,12 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 // 30,870 -> 12,340 (FP64 pipe). The slots must leave two CTAs per SM (one up to 304
 // subdomains: 46,657-node tube, FP64, 512 subdomains, one CTA 25,000, the kernel
 // above 20,300).
+//
+// Every wait between the roles (the producer warp, the inverting warp, the threads that
+// eliminate) is a bounded wait on an mbarrier or on the row counter. A thread that gives
+// one up waits for nothing more and goes on to the end of the rows, so that the barrier
+// of the eliminating threads stays matched; the other roles leave; nothing is read through
+// an index that was not waited for. The call then reports FSI_ERR_TIMEOUT.
 // threads that eliminate (then one producer warp and one warp that inverts the
 // pivots). FP32: a thread updates a whole column of a target block; FP64: an element
 constexpr int PIPE_HEAD = 160;         // barriers and the row counter
@@ -406,7 +412,8 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
   uint64_t* full = reinterpret_cast<uint64_t*>(fsm);        // [MAXSLOT]
   uint64_t* empty = full + MAXSLOT;                         // [MAXSLOT]
   uint64_t* inv = empty + MAXSLOT;                          // a row's pivot is inverted
-  volatile int* done = reinterpret_cast<volatile int*>(inv + 1);  // rows finished and stored
+  uint64_t* upd = inv + 1;                                  // a row's updates are done
+  volatile int* done = reinterpret_cast<volatile int*>(upd + 1);  // rows finished and stored
   TF* sScl = reinterpret_cast<TF*>(fsm + PIPE_HEAD);              // FP32 [4][56], rows of 8; FP64 [49]
   const int NS = R.pipe_slots;
   const uint32_t slot_bytes = R.pipe_meta + R.pipe_data;
@@ -421,11 +428,13 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
       pipe_bar_init(&empty[i], 1);
     }
     pipe_bar_init(inv, 1);
+    pipe_bar_init(upd, NT / 32);
     *done = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   bool ok = true;
+  const uint32_t tries = R.pipe_tries;
   int slot = 0, phase = 0;
   auto next_slot = [&]() {
     if (++slot == NS) {
@@ -437,7 +446,7 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
   if (w == NT / 32) {
     // producer warp: for every L block in elimination order, its word list and row k's
     // blocks into the next free slot, once row k is finished
-    const int64_t e0 = R.lent_ptr[qb], e1 = R.lent_ptr[qe];
+    const int64_t e0 = R.lent_ptr[qb], e1 = R.pipe_stall ? e0 : R.lent_ptr[qe];
     int fin = 0, issued = 0;
     for (int64_t eb = e0; eb < e1 && ok; eb += 32) {
       const int64_t em = eb + lane < e1 ? eb + lane : e1 - 1;
@@ -449,9 +458,9 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
         const int k = __shfl_sync(0xffffffffu, mk, i), len = __shfl_sync(0xffffffffu, ml, i);
         const int n16 = __shfl_sync(0xffffffffu, mn, i);
         const int64_t kd = __shfl_sync(0xffffffffu, mkd, i), off = __shfl_sync(0xffffffffu, mo, i);
-        if (issued >= NS) ok = pipe_bar_wait(&empty[slot], (uint32_t)(phase ^ 1));
+        if (issued >= NS) ok = pipe_bar_wait(&empty[slot], (uint32_t)(phase ^ 1), tries);
         if (len > 0 && fin <= k) {
-          for (uint32_t it = 0; it < (1u << 24) && (fin = *done) <= k; ++it) __nanosleep(20);
+          for (uint32_t it = 0; it < 16 * tries && (fin = *done) <= k; ++it) __nanosleep(20);
           ok = ok && fin > k;
           __threadfence_block();
         }
@@ -479,10 +488,10 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
   }
 
   if (w == NT / 32 + 1) {
-    // inverts each row's pivot when its updates are done (named barrier 2), beside the
-    // next row's elimination
+    // inverts each row's pivot when its updates are done, beside the next row's elimination
     for (int64_t q = qb; q < qe; ++q) {
-      asm volatile("bar.sync 2, %0;" ::"n"(NT + 32) : "memory");
+      ok = __all_sync(0xffffffffu, pipe_bar_wait(upd, (uint32_t)((q - qb) & 1), tries));
+      if (!ok) break;
       TF* B = sRow + (q & 1) * 49 * R.max_row_blocks + 49 * (int)(R.diag[q] - R.row_ptr[q]);
       warp_invert7_regs<TF>(B, err);
       __syncwarp();
@@ -491,10 +500,11 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
       __threadfence_block();
       __syncwarp();
       if (lane == 0) {
-        *done = (int)(q - qb) + 1;  // (the row's other blocks were stored before barrier 2)
+        *done = (int)(q - qb) + 1;  // (the row's other blocks were stored before upd)
         pipe_bar_arrive(inv);
       }
     }
+    if (!ok && lane == 0) atomicExch(err, 2);
     return;
   }
 
@@ -528,13 +538,14 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
     bar();
     bool inverted = q == qb;  // the previous row's pivot
     auto wait_inverse = [&]() {
-      if (!inverted && ok) ok = pipe_bar_wait(inv, (uint32_t)((q - qb - 1) & 1));
+      if (!inverted && ok) ok = pipe_bar_wait(inv, (uint32_t)((q - qb - 1) & 1), tries);
       inverted = true;
     };
     for (int e = 0; e < nl; ++e) {
-      if (ok) ok = pipe_bar_wait(&full[slot], (uint32_t)phase);
+      if (ok) ok = pipe_bar_wait(&full[slot], (uint32_t)phase, tries);
       const uint32_t* meta = reinterpret_cast<const uint32_t*>(slots + slot * slot_bytes);
-      const uint32_t head = ok ? meta[0] : 0;
+      // (a thread that gave up takes the list's head, and with it the block's branches, from global memory)
+      const uint32_t head = ok ? meta[0] : R.meta[4 * R.meta_off[lp + e]];
       const int ne = (int)(head & 0xffff);
       const uint32_t kind = head >> 28;
       if (kind == PIPE_PREV) wait_inverse();
@@ -610,7 +621,8 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
                                : reinterpret_cast<const TF*>(slots + slot * slot_bytes + R.pipe_meta) +
                                      ((head >> 16) & 15));
       bar();
-      if (tid == 0) pipe_bar_arrive(&empty[slot]);
+      // (a slot that was not waited for is not given back: a copy may still be on its way into it)
+      if (tid == 0 && ok) pipe_bar_arrive(&empty[slot]);
       next_slot();
     }
     // the pivot goes to the inverting warp, the blocks after it to global memory; the other
@@ -618,7 +630,8 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
     for (int x = 49 * (nl + 1) + tid; x < nv; x += NT) fac[49 * rp + x] = row[x];
     wait_inverse();
     __threadfence_block();
-    asm volatile("bar.arrive 2, %0;" ::"n"(NT + 32) : "memory");
+    __syncwarp();
+    if (lane == 0) pipe_bar_arrive(upd);
     nl_prev = nl;
     rp = rp1;
     rp1 = rp2;
@@ -626,7 +639,7 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
     lp = lp1;
     lp1 = lp2;
   }
-  if (!ok && lane == 0) atomicExch(err, 2);
+  if (!ok) atomicExch(err, 2);
 }
 
 // Block ILU on nested-dissection ordered subdomains: the CTA's 256 threads

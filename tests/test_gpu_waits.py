@@ -1,0 +1,43 @@
+"""Bounded waits of the pipelined factorisation that run out (a test switch of the
+options: its copies are never issued, or every wait gives up at once): the call ends
+and reports FSI_ERR_TIMEOUT, and the device and the library stay usable.
+"""
+import numpy as np
+import pytest
+
+import vesselmesh as vm
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("CUDA device required", allow_module_level=True)
+
+from paper_1810_04289_gb300 import fsi  # noqa: E402
+
+MAT = dict(rho_f=1.05, mu_f=0.035, rho_s=1.2, E_s=3.0e6, nu_s=0.45, eta_s=0.0)
+TIMEOUT = 9
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("fault_test,nsub", [(3, 2), (3, 400), (4, 2), (4, 400)])
+def test_factorisation_waits_that_run_out_are_reported(precision, fault_test, nsub):
+    m = vm.tube_mesh(24, 16, 5, 2, seed=3)
+    y = vm.poiseuille_state(m)
+    r = np.random.default_rng(8).normal(size=(m.n_nodes, 7))
+    out = []
+    for ft, mode in ((fault_test, 0), (0, 0), (0, 3)):
+        S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=nsub, fault_test=ft,
+                                                       factor_mode=mode))
+        S.set_state(y, t=0.25)
+        S.jacobian(y)
+        z = S.vec()
+        if ft:
+            with pytest.raises(fsi.FsiError) as e:
+                fsi.fsi_pc_apply(S.ctx, S.vec(r), z)
+            assert e.value.status == TIMEOUT
+        else:
+            fsi.fsi_pc_apply(S.ctx, S.vec(r), z)
+            out.append(z.cpu().numpy())
+        S.close()
+    assert np.array_equal(out[0], out[1])      # the next context's factors: the row kernel's bits
