@@ -323,7 +323,7 @@ __device__ __forceinline__ void warp_invert7_regs(TF* B, int32_t* err) {
         piv = r;
       }
     }
-    if (lane == k && !(best > tiny_pivot<TF>())) atomicExch(err, 1);
+    if (lane == k && !(best > tiny_pivot<TF>())) atomicMax(err, 1);  // (a wait that gave up, 2, stays reported)
     piv = __shfl_sync(0xffffffffu, piv, k);
     const TF ak = a[k];
 #pragma unroll

@@ -41,3 +41,24 @@ def test_factorisation_waits_that_run_out_are_reported(precision, fault_test, ns
             out.append(z.cpu().numpy())
         S.close()
     assert np.array_equal(out[0], out[1])      # the next context's factors: the row kernel's bits
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_wait_that_gave_up_is_reported_before_a_singular_pivot(precision):
+    """Two problems, one subdomain each: a tube, the waits of which run out soon, and
+    20,000 nodes without a tet (empty rows, singular pivots), found singular row by row
+    long after. The status is the wait's, whichever was found last."""
+    m = vm.tube_config("tube-12x8x4")
+    k = 20000
+    m.X = np.concatenate([m.X, np.c_[np.zeros((k, 2)), 100.0 + np.arange(k)]])
+    m.node_tag = np.concatenate([m.node_tag, np.full(k, vm.WALL, dtype=m.node_tag.dtype)])
+    m.node_problem = np.concatenate([m.node_problem, np.ones(k, dtype=m.node_problem.dtype)])
+    m.inlets = [m.inlets[0], m.inlets[0]]
+    S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=2, fault_test=3))
+    y = np.zeros((m.n_nodes, 7))
+    S.set_state(y, t=0.0)
+    S.jacobian(y)
+    with pytest.raises(fsi.FsiError) as e:
+        fsi.fsi_pc_apply(S.ctx, S.vec(np.ones((m.n_nodes, 7))), S.vec())
+    assert e.value.status == TIMEOUT
+    S.close()
