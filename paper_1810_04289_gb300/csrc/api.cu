@@ -892,8 +892,8 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
         FP = build_factor_pipe(R, cap, (int64_t)vs);
         rd.pipe_meta = (int32_t)(16 * FP.max_meta);
         rd.pipe_data = (int32_t)(16 * ((49 * vs * FP.max_len + 31 + 15) / 16));
-        rd.pipe_tries = o.fault_test == 3 ? 1u << 6 : o.fault_test == 4 ? 0 : 1u << 20;
-        rd.pipe_stall = o.fault_test == 3 ? 1 : 0;
+        rd.pipe_stall = o.fault_test == 3 ? 1 : o.fault_test == 4 ? 2 : 0;
+        rd.pipe_tries = rd.pipe_stall ? 64 : 1u << 20;
         for (int per_sm = 2; per_sm >= (R.np > 304 ? 2 : 1) && want == 2; --per_sm)
           for (int ns : {8, 6, 4}) {
             rd.pipe_slots = ns;

@@ -100,7 +100,8 @@ struct RasDev {
   int32_t pipe_meta;       // bytes of a slot's word list
   int32_t pipe_data;       // bytes of a slot's blocks
   uint32_t pipe_tries;     // looks after which a wait gives up
-  int32_t pipe_stall;      // tests only: the producer issues nothing (the waits run out)
+  int32_t pipe_stall;      // tests only: 1 the producer issues nothing, 2 the eliminating threads give up at
+                           // once (the other roles' waits run out)
   const int32_t* sd_depth; // [np] nested-dissection depth of each subdomain (0: one item)
   const int64_t* sd_item;  // [np+1] first item of each subdomain
   const int64_t* item_row; // [items] end row of each item (subdomain-relative)

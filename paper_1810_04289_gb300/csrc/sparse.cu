@@ -357,7 +357,8 @@ __device__ __forceinline__ void pipe_bar_arrive(uint64_t* b) {
 // bounded wait: false if the phase did not complete within `tries` looks
 __device__ __forceinline__ bool pipe_bar_wait(uint64_t* b, uint32_t parity, uint32_t tries) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(b);
-  for (uint32_t it = 0; it < tries; ++it) {
+  uint32_t it = 0;
+  do {  // (tries is looked at after the first miss only)
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -365,7 +366,7 @@ __device__ __forceinline__ bool pipe_bar_wait(uint64_t* b, uint32_t parity, uint
         : "r"(a), "r"(parity)
         : "memory");
     if (ok) return true;
-  }
+  } while (++it < tries);
   return false;
 }
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  bool ok = true;
+  bool ok = R.pipe_stall != 2 || w >= NT / 32;
   const uint32_t tries = R.pipe_tries;
   int slot = 0, phase = 0;
   auto next_slot = [&]() {
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
   if (w == NT / 32) {
     // producer warp: for every L block in elimination order, its word list and row k's
     // blocks into the next free slot, once row k is finished
-    const int64_t e0 = R.lent_ptr[qb], e1 = R.pipe_stall ? e0 : R.lent_ptr[qe];
+    const int64_t e0 = R.lent_ptr[qb], e1 = R.pipe_stall == 1 ? e0 : R.lent_ptr[qe];
     int fin = 0, issued = 0;
     for (int64_t eb = e0; eb < e1 && ok; eb += 32) {
       const int64_t em = eb + lane < e1 ? eb + lane : e1 - 1;
