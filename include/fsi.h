@@ -143,9 +143,11 @@ typedef struct {
                              the call returns FSI_ERR_TIMEOUT; 2 = Gram-Schmidt orth 0
                              forms every new vector's norm from the updated vector (its
                              fallback path); 3 = the pipelined factorisation's copies
-                             are never issued, 4 = every wait in it gives up at once:
-                             its bounded waits run out and the call that builds the
-                             factors returns FSI_ERR_TIMEOUT; 0 otherwise */
+                             are never issued, 4 = its eliminating threads wait for
+                             none: its bounded waits run out and the call that builds
+                             the factors returns FSI_ERR_TIMEOUT; 5 = the streamed
+                             apply's first wait gives up at once, with its copies on
+                             their way (FSI_ERR_TIMEOUT, too); 0 otherwise */
   int32_t apply_mode;     /* preconditioner apply kernel: 0 automatic (the streamed
                              apply when its shared-memory footprint fits, else the
                              level-scheduled one); 1 streamed (FSI_ERR_ARG if it does

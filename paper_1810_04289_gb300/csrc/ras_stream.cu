@@ -242,12 +242,12 @@ __global__ void __launch_bounds__(256) k_ras_apply_stream(RasStreamDev R, const 
 
   WarpFeed f{D, wi, -1, 0, 0, 0, 0, 0, 0, 0};
   const bool active = wi < (1 << D);
-  if (active && lane == 0 && !R.stall)
+  if (active && lane == 0 && R.stall != 1)
     for (int k = 0; k < NST; ++k) feed_issue<TF, STR>(f, ib, Lpack, Upack, ring, full, NST, SB);
   f.issued = __shfl_sync(0xffffffffu, f.issued, 0);
 
   const int j = lane / 7, c = lane - 7 * (lane / 7);  // block slot 0..3 (4 = idle), component
-  bool ok = true;
+  bool ok = R.stall != 2;
   // wait for the next stage of this warp's sequence; false on timeout
   auto next_stage = [&]() -> const TF* {
     const int st = f.uslot;
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256) k_ras_apply_stream(RasStreamDev R, const 
       f.uslot = 0;
       f.uphase ^= 1;
     }
-    if (lane == 0 && !R.stall) feed_issue<TF, STR>(f, ib, Lpack, Upack, ring, full, NST, SB);
+    if (lane == 0 && R.stall != 1) feed_issue<TF, STR>(f, ib, Lpack, Upack, ring, full, NST, SB);
     f.issued = __shfl_sync(0xffffffffu, f.issued, 0);
   };
 
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
   const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
   const TF* src = reinterpret_cast<const TF*>(R.pack) + (size_t)R.L_off[s] * STR;
   const uint8_t* sz = R.stage + R.stage_off[s];
-  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);  // stages not yet asked for
+  int left = R.stall == 1 ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);  // stages not yet asked for
   int nsz = left > 0 ? sz[0] : 0;                                       // blocks of the next one
   uint64_t win = cw[0] | (uint64_t)cw[1] << 32;  // entry codes ahead
   uint32_t ahead = cw[2];
@@ -484,6 +484,18 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
   int slot = 0, phase = 0;  // stage being worked off and its barrier's phase
   const unsigned char* at = ring + 16 * c + (lane >> 3) * BLK;  // this lane's row of the next entry's first group
   bool ok = true;
+  int fslot = 0, fphase = 0;  // the stage given up on
+  // once a wait gives up no stage is asked for any more: a barrier is not armed again
+  // while a copy may still be on its way to its slot
+  auto give_up = [&]() {
+    ok = false;
+    left = 0;
+    fslot = slot;
+    fphase = phase;
+  };
+  auto wait = [&]() {
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
+  };
   // rows of an entry's blocks into registers; what lies behind its blocks is read too and not used
   auto fetch = [&](TF (&A)[G][8], uint32_t code) {
     auto rows = [&](int g) {
@@ -537,7 +549,7 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
         phase ^= slot;
         slot ^= 1;
         at = ring + slot * cap + 16 * c + (lane >> 3) * BLK;
-        ok = ok && mbar_wait(&full[slot], (uint32_t)phase);
+        wait();
       }
       if (ncode < ENTRY_NONE) fetch(N, ncode);
       if (code & ENTRY_PIECE) {
@@ -563,9 +575,11 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
       if (ncode < ENTRY_NONE) fetch(N, ncode);
     }
   };
-  ok = mbar_wait(&full[0], 0u);
+  if (R.stall == 2) give_up();
+  wait();
   if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
-  for (int it = 0; it < 2 * nw && ok; ++it) {
+  // a lane whose wait gave up goes on to the end with the others (the data do not decide any address)
+  for (int it = 0; it < 2 * nw; ++it) {
     const uint32_t w3 = (uint32_t)win;
     step(A0, A1, w3 & 255, (w3 >> 8) & 255);
     step(A1, A0, (w3 >> 8) & 255, (w3 >> 16) & 255);
@@ -576,9 +590,10 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
     }
   }
   if (!ok) {
-    // a wait gave up: record it and let the copy still in flight in the other slot land (bounded)
-    if (lane == 0) atomicExch(err, 2);
-    mbar_wait(&full[slot ^ 1], (uint32_t)(phase ^ slot));
+    // record it and let the copies that may still be in flight land (bounded)
+    atomicExch(err, 2);
+    mbar_wait(&full[fslot], (uint32_t)fphase);
+    mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
   }
 
   // restricted prolongation (R_i^0)^T: owned rows only
@@ -627,7 +642,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
   const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
   const float* src = reinterpret_cast<const float*>(R.pack) + (size_t)R.L_off[s] * STR;
   const uint8_t* sz = R.stage + R.stage_off[s];
-  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
+  int left = R.stall == 1 ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
   int nsz = left > 0 ? sz[0] : 0;
   uint64_t win = cw[0] | (uint64_t)cw[1] << 32;
   uint32_t ahead = cw[2];
@@ -676,13 +691,14 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
   for (int e = 0; e < 8; ++e) A0[e] = A1[e] = float(0);
   const int cc = c < 7 ? c : 6;
   int fslot = 0, fphase = 0;
+  auto give_up = [&]() {
+    ok = false;
+    left = 0;
+    fslot = slot;
+    fphase = phase;
+  };
   auto wait = [&]() {
-    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
-      ok = false;
-      left = 0;
-      fslot = slot;
-      fphase = phase;
-    }
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
   };
   auto step = [&](float (&A)[8], float (&N)[8], uint32_t code, uint32_t ncode) {
     if (code < ENTRY_NONE) {
@@ -734,6 +750,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       if (ncode < ENTRY_NONE) fetch(N, ncode);
     }
   };
+  if (R.stall == 2) give_up();
   wait();
   if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
   // a warp whose wait gave up goes on to the end (the data do not decide any address or barrier)
@@ -798,7 +815,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
   const int nw = (int)(R.code_off[s + 1] - R.code_off[s]) - 2;
   const double* src = reinterpret_cast<const double*>(R.pack) + (size_t)R.L_off[s] * STR;
   const uint8_t* sz = R.stage + R.stage_off[s];
-  int left = R.stall ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
+  int left = R.stall == 1 ? 0 : (int)(R.stage_off[s + 1] - R.stage_off[s]);
   int nsz = left > 0 ? sz[0] : 0;
   uint64_t win = cw[0] | (uint64_t)cw[1] << 32;
   uint32_t ahead = cw[2];
@@ -831,13 +848,14 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
   int slot = 0, phase = 0, par = 0, t = 0, fslot = 0, fphase = 0;
   bool ok = true;
   const unsigned char* at = ring;  // blocks of the next entry to fetch (warp 0: of the current one)
+  auto give_up = [&]() {
+    ok = false;
+    left = 0;
+    fslot = slot;
+    fphase = phase;
+  };
   auto wait = [&]() {
-    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
-      ok = false;
-      left = 0;
-      fslot = slot;
-      fphase = phase;
-    }
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
   };
   auto next_stage = [&]() {
     feed(slot);
@@ -847,6 +865,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
     wait();
   };
   auto size = [](uint32_t code) { return ((code & 15) + ((code & ENTRY_NEAR) ? 1 : 0)) * BLK; };
+  if (R.stall == 2) give_up();
   wait();
 
   if (v == 0) {

@@ -1,6 +1,6 @@
-"""Bounded waits of the pipelined factorisation that run out (a test switch of the
-options: its copies are never issued, or every wait gives up at once): the call ends
-and reports FSI_ERR_TIMEOUT, and the device and the library stay usable.
+"""Bounded waits of the pipelined factorisation and of the streamed apply that run out
+(a test switch of the options: copies are never issued, or a wait gives up at once): the
+call ends and reports FSI_ERR_TIMEOUT, and the device and the library stay usable.
 """
 import numpy as np
 import pytest
@@ -62,3 +62,32 @@ def test_a_wait_that_gave_up_is_reported_before_a_singular_pivot(precision):
         fsi.fsi_pc_apply(S.ctx, S.vec(np.ones((m.n_nodes, 7))), S.vec())
     assert e.value.status == TIMEOUT
     S.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nsub,ordering", [(8, 1), (900, 1), (900, 2), (8, 3)])
+def test_apply_waits_that_give_up_with_copies_on_their_way(precision, nsub, ordering):
+    """Team, chain and ring kernels: no barrier is armed twice, the copies land before
+    the block ends, and the next context's apply is the level-scheduled kernel's."""
+    m = vm.tube_mesh(24, 16, 5, 2, seed=3)
+    y = vm.poiseuille_state(m)
+    r = np.random.default_rng(8).normal(size=(m.n_nodes, 7))
+    out = []
+    for ft, mode in ((5, 1), (0, 1), (0, 2)):
+        S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=nsub, ordering=ordering,
+                                                       fault_test=ft, apply_mode=mode))
+        S.set_state(y, t=0.25)
+        S.jacobian(y)
+        z = S.vec()
+        if ft:
+            with pytest.raises(fsi.FsiError) as e:
+                fsi.fsi_pc_apply(S.ctx, S.vec(r), z)
+            assert e.value.status == TIMEOUT
+        else:
+            fsi.fsi_pc_apply(S.ctx, S.vec(r), z)
+            out.append(z.cpu().numpy())
+        S.close()
+    # FP64: the row sums' order; mixed: FP32 solves of the same factors in another order
+    for c in ([0, 1, 2], [3], [4, 5, 6]):
+        far = np.abs(out[0][:, c] - out[1][:, c]).max() / np.abs(out[1][:, c]).max()
+        assert far <= (1e-2 if precision else 1e-10), far
