@@ -147,7 +147,9 @@ typedef struct {
                              none: its bounded waits run out and the call that builds
                              the factors returns FSI_ERR_TIMEOUT; 5 = the streamed
                              apply's first wait gives up at once, with its copies on
-                             their way (FSI_ERR_TIMEOUT, too); 0 otherwise */
+                             their way, 6 = it does so on one lane of each warp
+                             (where a team of warps takes a subdomain; both
+                             FSI_ERR_TIMEOUT, too); 0 otherwise */
   int32_t apply_mode;     /* preconditioner apply kernel: 0 automatic (the streamed
                              apply when its shared-memory footprint fits, else the
                              level-scheduled one); 1 streamed (FSI_ERR_ARG if it does

@@ -1017,7 +1017,7 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       rs.stage = cp->upload(S.stage);
       rs.stage_off = cp->upload(S.stage_off);
       rs.nst = nst;
-      rs.stall = o.fault_test == 1 ? 1 : o.fault_test == 5 ? 2 : 0;
+      rs.stall = o.fault_test == 1 ? 1 : o.fault_test == 5 ? 2 : o.fault_test == 6 ? 3 : 0;
       rs.stage_blocks = (int32_t)SB;
       rs.chain_blocks = (int32_t)CB;
       rs.max_rows = R.max_rows;

@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       if (ncode < ENTRY_NONE) fetch(N, ncode);
     }
   };
-  if (R.stall == 2) give_up();
+  if (R.stall == 2 || (R.stall == 3 && lane == 1)) give_up();
   wait();
   if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
   // a warp whose wait gave up goes on to the end (the data do not decide any address or barrier)
@@ -765,10 +765,13 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
     }
   }
   if (!ok) {
-    // record it and let the copies that may still be in flight land (bounded)
-    if (lane == 0) atomicExch(err, 2);
-    mbar_wait(&full[fslot], (uint32_t)fphase);
-    mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+    // record it; the thread that asked for the copies lets those that may still be in
+    // flight land (bounded; it has waited for all of them if it has not given up itself)
+    atomicExch(err, 2);
+    if (threadIdx.x == 0) {
+      mbar_wait(&full[fslot], (uint32_t)fphase);
+      mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+    }
   }
   __syncthreads();
   for (int q = threadIdx.x; q < m; q += 128) {
@@ -865,7 +868,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
     wait();
   };
   auto size = [](uint32_t code) { return ((code & 15) + ((code & ENTRY_NEAR) ? 1 : 0)) * BLK; };
-  if (R.stall == 2) give_up();
+  if (R.stall == 2 || (R.stall == 3 && lane == 1)) give_up();
   wait();
 
   if (v == 0) {
@@ -958,9 +961,11 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
     }
   }
   if (!ok) {
-    if (lane == 0) atomicExch(err, 2);
-    mbar_wait(&full[fslot], (uint32_t)fphase);
-    mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+    atomicExch(err, 2);
+    if (threadIdx.x == 0) {
+      mbar_wait(&full[fslot], (uint32_t)fphase);
+      mbar_wait(&full[fslot ^ 1], (uint32_t)(fphase ^ fslot));
+    }
   }
   __syncthreads();
   for (int q = threadIdx.x; q < m; q += 128) {

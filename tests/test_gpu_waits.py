@@ -91,3 +91,16 @@ def test_apply_waits_that_give_up_with_copies_on_their_way(precision, nsub, orde
     for c in ([0, 1, 2], [3], [4, 5, 6]):
         far = np.abs(out[0][:, c] - out[1][:, c]).max() / np.abs(out[1][:, c]).max()
         assert far <= (1e-2 if precision else 1e-10), far
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_wait_that_gives_up_on_one_lane_is_reported(precision):
+    m = vm.tube_mesh(24, 16, 5, 2, seed=3)
+    S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=8, fault_test=6))
+    y = vm.poiseuille_state(m)
+    S.set_state(y, t=0.25)
+    S.jacobian(y)
+    with pytest.raises(fsi.FsiError) as e:
+        fsi.fsi_pc_apply(S.ctx, S.vec(np.ones((m.n_nodes, 7))), S.vec())
+    assert e.value.status == TIMEOUT
+    S.close()
