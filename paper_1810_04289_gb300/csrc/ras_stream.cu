@@ -248,10 +248,12 @@ __global__ void __launch_bounds__(256) k_ras_apply_stream(RasStreamDev R, const 
 
   const int j = lane / 7, c = lane - 7 * (lane / 7);  // block slot 0..3 (4 = idle), component
   bool ok = R.stall != 2;
-  // wait for the next stage of this warp's sequence; false on timeout
+  // wait for the next stage of this warp's sequence; null on timeout, for the whole warp if
+  // for one lane: the loops below end on it, and the lanes shuffle in them
   auto next_stage = [&]() -> const TF* {
     const int st = f.uslot;
-    if (!mbar_wait(&full[st], (uint32_t)f.uphase)) return nullptr;
+    const bool lost = R.stall == 3 && lane == 1;
+    if (!__all_sync(0xffffffffu, !lost && mbar_wait(&full[st], (uint32_t)f.uphase))) return nullptr;
     return ring + (size_t)st * SB * STR;
   };
   // the stage is consumed: lane 0 refills its slot with the next stage in line

@@ -94,9 +94,11 @@ def test_apply_waits_that_give_up_with_copies_on_their_way(precision, nsub, orde
 
 
 @pytest.mark.parametrize("precision", [0, 1])
-def test_a_wait_that_gives_up_on_one_lane_is_reported(precision):
+@pytest.mark.parametrize("ordering", [1, 3])
+def test_a_wait_that_gives_up_on_one_lane_is_reported(precision, ordering):
     m = vm.tube_mesh(24, 16, 5, 2, seed=3)
-    S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=8, fault_test=6))
+    S = fsi.Solver(m, MAT, fsi.fsi_default_options(precision=precision, n_subdomains=8, ordering=ordering,
+                                                   fault_test=6))
     y = vm.poiseuille_state(m)
     S.set_state(y, t=0.25)
     S.jacobian(y)
