@@ -6,8 +6,6 @@
 // prolongation used when the TMA-fed apply (ras_stream.cu) does not fit.
 #include <cuda_runtime.h>
 
-#include <type_traits>
-
 #include "kernels.cuh"
 #include "setup.h"
 
@@ -29,38 +27,23 @@ inline int grid_for(int64_t work, int block) {
 // FP64 instruction per 19 cycles; a tree sum per block took 10 instructions where the
 // chain takes 7: 103k-node tree 240 -> 159 us). Mixed: FP32 values and an FP32 copy
 // of the vector; each block's 7-term product is formed in FP32 and the block products
-// are summed in pairs of floats (two_sum: the rounding error of every addition is kept,
-// about 48 bits): a conversion and an FP64 addition per block product bounded the
-// kernel as much as memory did (174k-node tree 104 -> 98 us).
+// are accumulated in FP64: a conversion and an FP64 addition per block product, which
+// bound the kernel about as much as memory does (174k-node tree 104 us; sums in pairs of
+// floats took 98, but carry 48 bits and FP32's range).
 // ---------------------------------------------------------------------------
-struct SumFloat {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float t) {
-    const float s = __fadd_rn(hi, t), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(t, b)));
-    hi = s;
-  }
-  // (an infinite or NaN sum has no error term)
-  __device__ __forceinline__ double value() const {
-    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
-  }
-};
-struct SumDouble {
-  double s = 0.0;
-  __device__ __forceinline__ double value() const { return s; }
-};
-__device__ __forceinline__ void add_product(SumFloat& acc, const float* A, const float* x) {
+__device__ __forceinline__ double add_product(double acc, const float* A, const float* x) {
   const float s0 = A[0] * x[0] + A[1] * x[1];
   const float s1 = A[2] * x[2] + A[3] * x[3];
   const float s2 = A[4] * x[4] + A[5] * x[5];
-  acc.add((s0 + s1) + (s2 + A[6] * x[6]));
+  return acc + (double)((s0 + s1) + (s2 + A[6] * x[6]));
 }
-__device__ __forceinline__ void add_product(SumDouble& acc, const double* A, const double* x) {
+__device__ __forceinline__ double add_product(double acc, const double* A, const double* x) {
 #pragma unroll
-  for (int k = 0; k < 7; ++k) acc.s = fma(A[k], x[k], acc.s);
+  for (int k = 0; k < 7; ++k) acc = fma(A[k], x[k], acc);
+  return acc;
 }
 
-template <class TV, class SUM, int S>
+template <class TV, int S>
 __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __restrict__ row_ptr,
                                                   const int32_t* __restrict__ col, const TV* __restrict__ vals,
                                                   const TV* __restrict__ x, double* __restrict__ y,
@@ -74,7 +57,7 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __re
   const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / G;
   for (int64_t base = grp0 - (lane / G); base < n; base += ngrp) {
     const int64_t row = base + (lane / G);
-    SUM sum;
+    double acc = 0.0;
     if (r < 7 && row < n) {
       const int64_t b0 = row_ptr[row], b1 = row_ptr[row + 1];
       // four of this lane's blocks per pass: their column indices first, then
@@ -85,10 +68,9 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int64_t n, const int64_t* __re
         for (int u = 0; u < 4; ++u) cl[u] = b + u * S < b1 ? col[b + u * S] : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (cl[u] >= 0) add_product(sum, vals + 49 * (b + u * S) + 7 * r, x + 7 * (int64_t)cl[u]);
+          if (cl[u] >= 0) acc = add_product(acc, vals + 49 * (b + u * S) + 7 * r, x + 7 * (int64_t)cl[u]);
       }
     }
-    double acc = sum.value();
 #pragma unroll
     for (int o = 1; o < S; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (r < 7 && q == 0 && row < n) y[7 * row + r] = acc;
@@ -813,11 +795,10 @@ __global__ void __launch_bounds__(256) k_ras_apply(RasDev R, const TF* __restric
 template <class TV>
 void launch_bsr_spmv(int64_t n, const int64_t* row_ptr, const int32_t* col, const TV* vals, const TV* x,
                      double* y, int threads_per_row, const int* guard, cudaStream_t s) {
-  using SUM = std::conditional_t<sizeof(TV) == 4, SumFloat, SumDouble>;
   if (threads_per_row == 16)
-    k_bsr_spmv<TV, SUM, 2><<<grid_for(16 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
+    k_bsr_spmv<TV, 2><<<grid_for(16 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
   else
-    k_bsr_spmv<TV, SUM, 4><<<grid_for(32 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
+    k_bsr_spmv<TV, 4><<<grid_for(32 * n, 256), 256, 0, s>>>(n, row_ptr, col, vals, x, y, guard);
 }
 
 void launch_to_float(int64_t n, const double* x, float* y, const int* guard, cudaStream_t s) {
