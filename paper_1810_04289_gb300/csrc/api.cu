@@ -97,10 +97,11 @@ struct fsi_ctx {
   int* active = nullptr;         // [P] problem still iterating in the cycle
   int* kcols = nullptr;          // [P] Krylov columns built in the cycle
   int* anyact = nullptr;         // [1] some problem active (guard of the captured kernels)
-  int* reorth = nullptr;         // [1] some problem needs a second Gram-Schmidt pass (orth = 1), or
-                                 // its new norm from the updated vector (orth = 0 fallback)
+  int* reorth = nullptr;         // [1] some problem needs a second Gram-Schmidt pass (orth = 1), or its
+                                 // new norm from the updated vector (orth = 0, NewNorm::flag)
   double* gs_inv = nullptr;      // [P] reciprocal of H[j+1][j] (orth 0)
   int* gs_unsafe = nullptr;      // [P] the norm is taken from the updated vector
+  double* gs_nrm = nullptr;      // [P] that norm
   int* pmask = nullptr;          // [P] problem already converged (Newton)
   double* palpha = nullptr;      // [P] line-search step per problem
   float* zf = nullptr;           // FP32 copy of the SpMV input (mixed precision)
@@ -361,23 +362,23 @@ void arnoldi_step(fsi_ctx* c, int32_t j, const int* guard, cudaStream_t st) {
     launch_seg_norm(c->seg, w, c->partial, hj, ldh * m, c->reorth, st);
     launch_seg_scale_inv(c->seg, n, w, hj, ldh * m, w, guard, st);
     launch_seg_givens(P, c->hA, c->hB, ldh, c->H, ldh, m, j, c->cs, c->sn, c->g, c->gres, c->gtarget, c->active,
-                      c->kcols, c->anyact, c->seg, w, nullptr, guard, st);
+                      c->kcols, c->anyact, c->seg, n, w, NewNorm{}, guard, st);
     c->launches += 9;
     return;
   }
   if (c->opt.orth == 0) {
     // classical Gram-Schmidt twice, the new norm from the second pass: dots;
     // update; dots with ||w||^2; norm = sqrt(||w||^2 - ||h2||^2); update and scale
-    // in one sweep. Where that norm is unsafe the Givens kernel forms it from the
-    // updated vector.
-    double* hj = c->H + (int64_t)j * ldh + j + 1;
+    // in one sweep. Where that norm is unsafe the second update forms it from the
+    // updated vector, and the Givens kernel scales.
+    const NewNorm N{c->H + (int64_t)j * ldh + j + 1, (int64_t)ldh * m, c->gs_inv, c->gs_unsafe, c->reorth, c->gs_nrm,
+                    c->active, c->opt.fault_test == 2 ? 1 : 0};
     launch_seg_mdot(c->seg, j + 1, c->V, n, w, c->partial, c->hA, ldh, guard, st);
-    launch_seg_maxpy(c->seg, n, j + 1, c->V, n, c->hA, ldh, w, guard, st);
-    launch_seg_mdot_norm(c->seg, j + 1, c->V, n, w, c->partial, c->hB, ldh, hj, (int64_t)ldh * m, c->gs_inv,
-                         c->gs_unsafe, c->opt.fault_test == 2 ? 1 : 0, guard, st);
-    launch_seg_maxpy(c->seg, n, j + 1, c->V, n, c->hB, ldh, w, guard, st, c->gs_inv);
+    launch_seg_maxpy(c->seg, n, j + 1, c->V, n, c->hA, ldh, w, guard, st, nullptr, N);
+    launch_seg_mdot_norm(c->seg, j + 1, c->V, n, w, c->partial, c->hB, ldh, N, guard, st);
+    launch_seg_maxpy(c->seg, n, j + 1, c->V, n, c->hB, ldh, w, guard, st, c->gs_inv, N, c->partial);
     launch_seg_givens(P, c->hA, c->hB, ldh, c->H, ldh, m, j, c->cs, c->sn, c->g, c->gres, c->gtarget, c->active,
-                      c->kcols, c->anyact, c->seg, w, c->gs_unsafe, guard, st);
+                      c->kcols, c->anyact, c->seg, n, w, N, guard, st);
     c->launches += 5;
     return;
   }
@@ -390,7 +391,7 @@ void arnoldi_step(fsi_ctx* c, int32_t j, const int* guard, cudaStream_t st) {
   launch_seg_norm(c->seg, w, c->partial, c->H + (int64_t)j * ldh + j + 1, ldh * m, guard, st);
   launch_seg_scale_inv(c->seg, n, w, c->H + (int64_t)j * ldh + j + 1, ldh * m, w, guard, st);
   launch_seg_givens(P, c->hA, c->hB, ldh, c->H, ldh, m, j, c->cs, c->sn, c->g, c->gres, c->gtarget, c->active,
-                    c->kcols, c->anyact, c->seg, w, nullptr, guard, st);
+                    c->kcols, c->anyact, c->seg, n, w, NewNorm{}, guard, st);
   c->launches += 7;
 }
 
@@ -834,6 +835,7 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
     cp->reorth = cp->dalloc<int>(1);
     cp->gs_inv = cp->dalloc<double>(n_problems);
     cp->gs_unsafe = cp->dalloc<int>(n_problems);
+    cp->gs_nrm = cp->dalloc<double>(n_problems);
     cp->pmask = cp->dalloc<int>(n_problems);
     cp->palpha = cp->dalloc<double>(n_problems);
     cp->r = cp->dalloc<double>(n);

@@ -186,30 +186,44 @@ constexpr int SEG_COUNTERS = SEG_GROUPS + 1;
 // out[p * ldo + k] = V_k . w for k < nv (and, with_self = 1, out[p * ldo + nv] = w . w)
 void launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w, double* partial,
                      double* out, int32_t ldo, const int* guard, cudaStream_t s, int with_self = 0);
+// The norm of a Gram-Schmidt step's new vector from its second pass (krylov.cu, new_norm)
+struct NewNorm {
+  double* hsub;       // H[p][j+1][j], ldsub apart per problem; null: no norm wanted
+  int64_t ldsub;
+  double* inv;        // [P] its reciprocal
+  int* unsafe;        // [P] the norm is taken from the updated vector
+  int* flag;          // [1] for some problem (null: no such problem)
+  double* norms;      // [P] those norms
+  const int* active;  // [P] the problem iterates
+  int force;          // tests only: every norm from the updated vector
+};
 // the same with w . w, then the norm of w - V out as sqrt(w . w - ||V . w||^2) into hsub where
-// that is safe, its reciprocal into inv, else unsafe[p] = 1 (see krylov.cu)
+// that is safe, its reciprocal into inv, else unsafe[p] = 1
 void launch_seg_mdot_norm(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w,
-                          double* partial, double* out, int32_t ldo, double* hsub, int64_t ldsub, double* inv,
-                          int* unsafe, int force, const int* guard, cudaStream_t s);
+                          double* partial, double* out, int32_t ldo, const NewNorm& N, const int* guard,
+                          cudaStream_t s);
 // selective reorthogonalisation test after one Gram-Schmidt pass (see krylov.cu)
 void launch_seg_reorth_decide(int32_t P, const double* ws, const double* nrm, int32_t ldn, double* hb, int32_t lda,
                               int32_t j, const int* active, int* flag, cudaStream_t s);
 void launch_seg_norm(const SegDev& sg, const double* x, double* partial, double* out, int32_t ldo,
                      const int* guard, cudaStream_t s);
-// w -= V h per problem, then w *= scal[p] (scal optional)
+// w -= V h per problem, then w *= scal[p] (scal optional). With N.flag: cleared (no scal), or the
+// unsafe problems' norms formed where it is set (partial: n_chunks values)
 void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, int64_t ldv, const double* h,
-                      int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal = nullptr);
+                      int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal = nullptr,
+                      const NewNorm& N = NewNorm{}, double* partial = nullptr);
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
                           double* y, const int* guard, cudaStream_t s);
 
 void launch_seg_cycle_init(int32_t P, double* g, int32_t ldg, const double* beta, const double* target, int* active,
                            int* kcols, int* any, cudaStream_t s);
 // column j of each active problem's Hessenberg = a + b (the two Gram-Schmidt passes, lda apart per
-// problem), then the Givens update; first, where unsafe[p] (optional), ||w_p|| into H and w_p divided by it
+// problem), then the Givens update; beside it, where N.flag (optional) is set, the unsafe problems' w_p
+// divided by their norms (w: n values)
 void launch_seg_givens(int32_t P, const double* a, const double* b, int32_t lda, double* H, int32_t ldh, int32_t m,
                        int32_t j, double* cs, double* sn, double* g, double* res, const double* target, int* active,
-                       int* kcols, int* any, const SegDev& sg, double* w, const int* unsafe, const int* guard,
-                       cudaStream_t s);
+                       int* kcols, int* any, const SegDev& sg, int64_t n, double* w, const NewNorm& N,
+                       const int* guard, cudaStream_t s);
 void launch_seg_lsq(int32_t P, const double* H, int32_t ldh, int32_t m, const int* kcols, const double* g, double* y,
                     cudaStream_t s);
 void launch_seg_update_x(const SegDev& sg, int64_t n, const double* Z, int64_t ldz, const double* y, int32_t m,

@@ -59,14 +59,9 @@ __device__ __forceinline__ void warp_sums(double (&v)[W]) {
 // of ||w1||^2 (the subtraction then loses under two bits) hsub[p * ldsub] is its
 // square root and inv[p] the reciprocal (0 for a zero norm); elsewhere (only as a
 // Krylov space is exhausted; for every problem with force = 1, tests of that path)
-// inv[p] = 1 and unsafe[p] = 1: k_seg_givens then forms the norm from the updated vector.
-struct NewNorm {
-  double* hsub;  // null: no norm wanted
-  int64_t ldsub;
-  double* inv;
-  int* unsafe;
-  int force;
-};
+// inv[p] = 1, unsafe[p] = 1 and *flag = 1: the second update (k_seg_maxpy) then forms the
+// norm of the updated vector and k_seg_givens scales by it. A problem that has already
+// stopped needs no norm: its vector is zeroed (inv[p] = 0).
 
 // one warp: q = ||h2||^2 and s = ||w1||^2, written by other blocks of this launch
 __device__ void new_norm(const NewNorm& N, int p, const double* h, int nv) {
@@ -86,8 +81,10 @@ __device__ void new_norm(const NewNorm& N, int p, const double* h, int nv) {
       N.inv[p] = b > 0.0 ? 1.0 / b : 0.0;
       N.unsafe[p] = 0;
     } else {
-      N.inv[p] = 1.0;
-      N.unsafe[p] = 1;
+      const int a = N.active[p];
+      N.inv[p] = a ? 1.0 : 0.0;
+      N.unsafe[p] = a;
+      if (a) *N.flag = 1;
     }
   }
 }
@@ -197,11 +194,67 @@ __global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, const do
     dots<W, U>(sg, nv, g, G, V, ldv, w, partial, out, ldo, take_sqrt, nself, N);
 }
 
-// w_i -= sum_k h[p(i)][k] V_k[i], then (scal non-null) w_i *= scal[p(i)]
-__global__ void k_seg_maxpy(SegDev sg, int64_t n, int32_t nv, const double* __restrict__ V, int64_t ldv,
-                            const double* __restrict__ h, int32_t ldh, double* __restrict__ w,
-                            const double* __restrict__ scal, const int* guard) {
+// The second update where some problem's norm is unsafe, chunk by chunk: as k_seg_maxpy,
+// and for the unsafe problems hsub[p * ldsub] = norms[p] = ||w_p|| of the updated vector
+// (chunk partials, summed by the last block of the problem in fixed order).
+__device__ __noinline__ void maxpy_norm(const SegDev* sgp, int32_t nv, const double* V, int64_t ldv, const double* h,
+                                        int32_t ldh, double* w, const double* scal, const NewNorm* Np,
+                                        double* partial) {
+  __shared__ double red[RB / 32];
+  __shared__ int s_last;
+  const SegDev& sg = *sgp;
+  const NewNorm& N = *Np;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int64_t c = blockIdx.x; c < sg.n_chunks; c += gridDim.x) {
+    const int64_t i0 = sg.chunk_beg[c], i1 = sg.chunk_beg[c + 1];
+    const int p = sg.node_prob[i0 / 7];
+    const double* hp = h + (int64_t)p * ldh;
+    const double a = scal[p];
+    double q = 0.0;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      double s = w[i];
+      for (int k = 0; k < nv; ++k) s -= hp[k] * V[(int64_t)k * ldv + i];
+      w[i] = s * a;
+      q += s * s;
+    }
+    if (!N.unsafe[p]) continue;
+    q = warp_sum(q);
+    if (lane == 0) red[warp] = q;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 1; k < RB / 32; ++k) q += red[k];
+      partial[c] = q;
+      __threadfence();
+      s_last = atomicAdd(sg.counter + (int64_t)p * SEG_COUNTERS, 1) == (int)(sg.prob_chunk[p + 1] - sg.prob_chunk[p]) - 1;
+    }
+    __syncthreads();
+    if (s_last && warp == 0) {
+      __threadfence();
+      double v = 0.0;
+      for (int64_t cc = sg.prob_chunk[p] + lane; cc < sg.prob_chunk[p + 1]; cc += 32) v += __ldcg(partial + cc);
+      v = warp_sum(v);
+      if (lane == 0) {
+        N.hsub[(int64_t)p * N.ldsub] = N.norms[p] = sqrt(v);
+        sg.counter[(int64_t)p * SEG_COUNTERS] = 0;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// w_i -= sum_k h[p(i)][k] V_k[i], then (scal non-null) w_i *= scal[p(i)]. N.flag (optional): the
+// first update (no scal) clears it, the second takes the form above where it is set.
+__global__ void __launch_bounds__(RB, 8) k_seg_maxpy(const __grid_constant__ SegDev sg, int64_t n, int32_t nv,
+                                                  const double* __restrict__ V, int64_t ldv,
+                                                  const double* __restrict__ h, int32_t ldh, double* __restrict__ w,
+                                                  const double* __restrict__ scal, const int* guard,
+                                                  const __grid_constant__ NewNorm N, double* partial) {
+  if (N.flag && !scal && blockIdx.x == 0 && threadIdx.x == 0) *N.flag = 0;
   if (off(guard)) return;
+  if (N.flag && scal && *N.flag) {
+    maxpy_norm(&sg, nv, V, ldv, h, ldh, w, scal, &N, partial);
+    return;
+  }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int p = sg.node_prob[i / 7];
     const double* hp = h + (int64_t)p * ldh;
@@ -279,9 +332,11 @@ __global__ void k_seg_reorth_decide(int32_t P, const double* __restrict__ ws, co
 // rotations at once and hand them to the chain by shuffles (read one by one inside the
 // chain of rotations they cost an L2 latency each: 7.3 -> 5.9 us for one problem).
 //
-// Where unsafe[p] (non-null; set by new_norm, a rare path), the whole block first forms
-// H[p][j+1][j] = ||w_p|| of the updated vector and scales w_p by its reciprocal (0 for a
-// zero norm); as a launch of its own it cost 2 us a step for nothing.
+// Where *flag (non-null; set by new_norm, a rare path), every block scales its part of the
+// unsafe problems' w_p by 1 / norms[p], the norm of the updated vector (0 for a zero
+// norm); block 0 alone does the rest. As launches of their own the norm and the scaling
+// cost 2 us each a step for nothing; both in this kernel's one block took 829 us a step at
+// 1.2 M unknowns where every norm is unsafe, this form 41 (the normal step is not slower).
 __global__ void __launch_bounds__(1024) k_seg_givens(int32_t P, const double* __restrict__ ha,
                                                      const double* __restrict__ hb, int32_t lda,
                                                      double* __restrict__ H, int32_t ldh, int32_t m, int32_t j,
@@ -289,29 +344,25 @@ __global__ void __launch_bounds__(1024) k_seg_givens(int32_t P, const double* __
                                                      double* __restrict__ g, double* __restrict__ res,
                                                      const double* __restrict__ target, int* __restrict__ active,
                                                      int* __restrict__ kcols, int* __restrict__ any, SegDev sg,
-                                                     double* __restrict__ w, const int* __restrict__ unsafe,
-                                                     const int* guard) {
+                                                     int64_t n, double* __restrict__ w,
+                                                     const __grid_constant__ NewNorm N, const int* guard) {
   __shared__ int s_any;
   const int lane = threadIdx.x & 31;
-  if (off(guard)) return;  // *any is this flag, 0 already
-  if (threadIdx.x == 0) s_any = 0;
-  if (unsafe) {
-    __shared__ double red[32];
-    for (int p = 0; p < P; ++p) {
-      if (!unsafe[p]) continue;
-      const int64_t i0 = sg.chunk_beg[sg.prob_chunk[p]], i1 = sg.chunk_beg[sg.prob_chunk[p + 1]];
-      double s = 0.0;
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += w[i] * w[i];
-      s = warp_sum(s);
-      if (lane == 0) red[threadIdx.x >> 5] = s;
-      __syncthreads();
-      s = warp_sum(red[lane]);
-      const double nrm = sqrt(s), inv = nrm != 0.0 ? 1.0 / nrm : 0.0;
-      if (threadIdx.x == 0) H[(int64_t)p * ldh * m + (int64_t)j * ldh + j + 1] = nrm;
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] *= inv;
-      __syncthreads();
+  if (N.flag && *N.flag) {  // (not under the guard, *any, which block 0 may have stored already)
+    int pc = -1;
+    double inv = 1.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+      const int p = sg.node_prob[i / 7];
+      if (p != pc) {
+        const double a = N.norms[p];
+        inv = !N.unsafe[p] ? 1.0 : a != 0.0 ? 1.0 / a : 0.0;
+        pc = p;
+      }
+      if (inv != 1.0) w[i] *= inv;
     }
   }
+  if (blockIdx.x > 0 || off(guard)) return;  // *any is the guard, 0 already
+  if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
   for (int p = threadIdx.x >> 5; p < P; p += blockDim.x >> 5) {
     if (!active[p]) continue;
@@ -462,9 +513,9 @@ void launch_seg_mdot(const SegDev& sg, int32_t nv, const double* V, int64_t ldv,
 }
 
 void launch_seg_mdot_norm(const SegDev& sg, int32_t nv, const double* V, int64_t ldv, const double* w,
-                          double* partial, double* out, int32_t ldo, double* hsub, int64_t ldsub, double* inv,
-                          int* unsafe, int force, const int* guard, cudaStream_t s) {
-  mdot(sg, nv + 1, V, ldv, w, partial, out, ldo, 0, 1, NewNorm{hsub, ldsub, inv, unsafe, force}, guard, s);
+                          double* partial, double* out, int32_t ldo, const NewNorm& N, const int* guard,
+                          cudaStream_t s) {
+  mdot(sg, nv + 1, V, ldv, w, partial, out, ldo, 0, 1, N, guard, s);
 }
 
 void launch_seg_norm(const SegDev& sg, const double* x, double* partial, double* out, int32_t ldo,
@@ -478,8 +529,9 @@ void launch_seg_reorth_decide(int32_t P, const double* ws, const double* nrm, in
 }
 
 void launch_seg_maxpy(const SegDev& sg, int64_t n, int32_t nv, const double* V, int64_t ldv, const double* h,
-                      int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal) {
-  k_seg_maxpy<<<grid_for(n, 256), 256, 0, s>>>(sg, n, nv, V, ldv, h, ldh, w, scal, guard);
+                      int32_t ldh, double* w, const int* guard, cudaStream_t s, const double* scal, const NewNorm& N,
+                      double* partial) {
+  k_seg_maxpy<<<grid_for(n, RB), RB, 0, s>>>(sg, n, nv, V, ldv, h, ldh, w, scal, guard, N, partial);
 }
 
 void launch_seg_scale_inv(const SegDev& sg, int64_t n, const double* x, const double* scal, int32_t lds,
@@ -494,10 +546,14 @@ void launch_seg_cycle_init(int32_t P, double* g, int32_t ldg, const double* beta
 
 void launch_seg_givens(int32_t P, const double* a, const double* b, int32_t lda, double* H, int32_t ldh, int32_t m,
                        int32_t j, double* cs, double* sn, double* g, double* res, const double* target, int* active,
-                       int* kcols, int* any, const SegDev& sg, double* w, const int* unsafe, const int* guard,
-                       cudaStream_t s) {
-  k_seg_givens<<<1, unsafe ? 1024 : 32 * (P < 32 ? P : 32), 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res, target,
-                                                                    active, kcols, any, sg, w, unsafe, guard);
+                       int* kcols, int* any, const SegDev& sg, int64_t n, double* w, const NewNorm& N,
+                       const int* guard, cudaStream_t s) {
+  // block 0 with a warp per problem; the blocks that scale (rarely) add up to at most two per SM
+  const int warps = P < 32 ? P : 32;
+  const int threads = 32 * (N.flag && warps < 8 ? 8 : warps);
+  const int64_t blocks = N.flag ? (n + 8 * threads - 1) / (8 * threads) : 1;
+  k_seg_givens<<<(int)(blocks < 304 ? blocks : 304), threads, 0, s>>>(P, a, b, lda, H, ldh, m, j, cs, sn, g, res,
+                                                                      target, active, kcols, any, sg, n, w, N, guard);
 }
 
 void launch_seg_lsq(int32_t P, const double* H, int32_t ldh, int32_t m, const int* kcols, const double* g, double* y,
