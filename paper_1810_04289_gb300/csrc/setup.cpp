@@ -534,6 +534,7 @@ namespace {
 template <class Emit>
 StreamPlan make_stream(const RasPlan& R, int64_t stage, Emit&& emit) {
   StreamPlan S;
+  stage = std::min(stage, STAGE_MOST);
   const int32_t np = R.np;
   const int64_t rows = (int64_t)R.gnode.size();
   S.L_cnt.resize(rows);
