@@ -106,9 +106,10 @@ def parse():
     p.add_argument("--threads-per-row", type=int, default=None, choices=[16, 32],
                    help="BSR SpMV threads per block row (fsi_options.threads_per_row)")
     p.add_argument("--stages", type=int, default=None,
-                   help="streamed apply: ring stages (fsi_options.stages); default the library's choice")
+                   help="ring apply of dissected subdomains: stages (fsi_options.stages); default the library's choice")
     p.add_argument("--stage-blocks", type=int, default=None,
-                   help="streamed apply: blocks per ring stage (fsi_options.stage_blocks)")
+                   help="ring apply of dissected subdomains: blocks per stage; elsewhere, mixed: where a row's "
+                        "sum is cut (fsi_options.stage_blocks)")
     p.add_argument("--newton-rtol", type=float, default=1e-6)
     p.add_argument("--gmres-rtol", type=float, default=1e-3)
     p.add_argument("--precisions", default="mixed,fp64")

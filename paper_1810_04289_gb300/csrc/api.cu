@@ -883,7 +883,7 @@ fsi_status fsi_create(const fsi_mesh* mesh, const fsi_material* mat, const fsi_b
       rd.max_depth = R.max_depth;
       auto fits = [&](int mode) { return cp->mixed ? ras_factor_fits<float>(rd, mode) : ras_factor_fits<double>(rd, mode); };
       // automatic: nested-dissection groups when the subdomains are dissected and
-      // the groups' rows fit, else the row-only sequential kernel
+      // the groups' rows fit, else rows in order (pipelined if its slots fit, see below)
       int want = o.factor_mode > 0 ? o.factor_mode - 1 : (R.max_depth > 0 && fits(3) ? 3 : 2);
       FactorPipe FP;
       if (o.factor_mode == 0 && want == 2) {

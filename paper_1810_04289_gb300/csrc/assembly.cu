@@ -8,8 +8,9 @@
 // Element rows are routed to node rows by the node flags (strong interface
 // coupling, Sec. 2.2): continuity -> p row; fluid momentum -> u rows of
 // fluid-only nodes and d rows of interface nodes; mesh motion -> d rows of
-// fluid-only nodes; wall momentum -> d rows. Constrained rows receive zeros
-// and are written afterwards by the constraint kernels.
+// fluid-only nodes; wall momentum -> d rows. Constrained rows receive zeros; the
+// residual's gather puts their own residual in place, a kernel after the Jacobian's
+// gather their diagonal blocks.
 #include <cuda_runtime.h>
 
 #include "kernels.cuh"

@@ -36,16 +36,8 @@ template <class T> __host__ __device__ inline Dual<T> operator/(T a, Dual<T> b) 
 template <class T> __host__ __device__ inline Dual<T>& operator+=(Dual<T>& a, Dual<T> b) { a.v += b.v; a.d += b.d; return a; }
 template <class T> __host__ __device__ inline Dual<T>& operator-=(Dual<T>& a, Dual<T> b) { a.v -= b.v; a.d -= b.d; return a; }
 
-__device__ inline double dsqrt(double a) { return sqrt(a); }
 __device__ inline float dsqrt(float a) { return sqrtf(a); }
 template <class T> __device__ inline Dual<T> dsqrt(Dual<T> a) {
   T s = dsqrt(a.v);
   return Dual<T>(s, a.d / (T(2) * s));
 }
-
-// value part of a scalar
-__device__ inline double val(double a) { return a; }
-__device__ inline float val(float a) { return a; }
-template <class T> __device__ inline T val(Dual<T> a) { return a.v; }
-// tangent part
-template <class T> __device__ inline T tan_of(Dual<T> a) { return a.d; }

@@ -1,8 +1,8 @@
 // Element residuals of the monolithic ALE FSI system on P1 tetrahedra.
 //
 // One routine per element kind, templated on the scalar S of the unknowns
-// (T = double / float for the residual, Dual<T> for one Jacobian column) and the
-// base type T of constant data (reference coordinates, previous time levels).
+// (Dual<T>: one Jacobian column) and the base type T of constant data (reference
+// coordinates, previous time levels), and the same residuals in closed form in FP64.
 //
 //   fluid tets : ALE Navier-Stokes momentum and continuity on the current tet
 //                x = X + d (Sec. 2.1, Eq. 3; backward Euler, Eq. 9), stabilised

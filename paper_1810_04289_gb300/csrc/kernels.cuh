@@ -164,7 +164,8 @@ void launch_pack_factors(const RasStreamDev& r, const TF* fac, cudaStream_t s);
 template <class TF>
 cudaError_t ras_stream_init(const RasStreamDev& r);
 // z = B^{-1} r; z32 (optional) receives an FP32 copy; guard as for the SpMV. Takes
-// the chain kernel, or the ring kernel for dissected subdomains
+// the chain kernel, a team kernel where subdomains are few (r.team), or the ring
+// kernel for dissected subdomains
 template <class TF>
 cudaError_t launch_ras_apply_stream(const RasStreamDev& r, const double* rin, double* z, float* z32, int32_t* err,
                                     const int* guard, cudaStream_t s);

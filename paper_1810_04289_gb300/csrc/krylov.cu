@@ -179,8 +179,9 @@ __device__ __forceinline__ void dots(const SegDev& sg, int32_t nv, int g, int n_
 // deeper U (fewer products, more loads in flight). All groups and the new norm in one
 // launch: as two launches and one more for the norm the narrow group ran after the full
 // ones with most of the chip idle, and each launch of the cycle's graph costs 1.4 to 4 us
-// (seven launches per GMRES iteration instead of eleven: a mixed step of the 46,657-node tube
-// 157.7 -> 152.7 ms, an FP64 step of the 12 x 8 x 4 tube 100.6 -> 98.2 ms; the same bits).
+// (seven launches per GMRES iteration instead of eleven, the same bits: a mixed step of the
+// 46,657-node tube 157.7 -> 152.7 ms, an FP64 step of the 12 x 8 x 4 tube 100.6 -> 98.2 ms; a
+// step's time depends on its random state, both sides are of the same one).
 template <int W, int U>
 __global__ void __launch_bounds__(RB) k_seg_mdot(SegDev sg, int32_t nv, const double* __restrict__ V, int64_t ldv,
                                                  const double* __restrict__ w, double* __restrict__ partial,

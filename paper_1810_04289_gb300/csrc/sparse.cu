@@ -187,8 +187,8 @@ __device__ void warp_invert7(TF* B, TF* aug, int32_t* err) {
 //   1: as 0 but D_k read from global memory (L2) when used;
 //   2: only the row: D_k and the sources read from global memory when used.
 // All three do the same arithmetic in the same order (bitwise identical
-// factors); MODE 2 (factor_mode 3, the row only) is the default (see
-// ras_factor_fits).
+// factors). MODE 2 (factor_mode 3, the row only) runs where the pipelined kernel
+// below does not fit (see ras_factor_fits), 0 and 1 where they are asked for.
 template <class TF>
 __device__ __forceinline__ void cp_async_elem(TF* dst, const TF* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
@@ -823,10 +823,11 @@ size_t ras_factor_smem(const RasDev& r, int mode) {
   return (blocks * 49 + 98) * sizeof(TF);  // + the 7 x 14 inversion scratch
 }
 
-// Fit check of a factorisation mode. The automatic choice is the leanest mode
-// (2): measured on GB300 it is the fastest, because the smaller footprint lets
-// more subdomain CTAs share an SM, which hides the latency of the pivot and
-// source reads better than prefetching them does.
+// Fit check of a factorisation mode. The automatic choice on one-piece subdomains is
+// the pipelined kernel (4) where its slots fit as fsi_create asks, else the leanest
+// mode (2): of modes 0 to 2 it is the fastest, because the smaller footprint lets more
+// subdomain CTAs share an SM, which hides the latency of the pivot and source reads
+// better than prefetching them does.
 template <class TF>
 bool ras_factor_fits(const RasDev& r, int mode) {
   return ras_factor_smem<TF>(r, mode) <= FACTOR_SMEM_MAX;
