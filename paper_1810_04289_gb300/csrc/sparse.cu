@@ -833,11 +833,13 @@ bool ras_factor_fits(const RasDev& r, int mode) {
   return ras_factor_smem<TF>(r, mode) <= FACTOR_SMEM_MAX;
 }
 
+// (the shared-memory limit is the kernel's, not the launch's: set to what one context needs,
+// another thread's launch with more could be refused)
 template <class TF, int MODE>
 void launch_factor_mode(const RasDev& r, TF* fac, int32_t* err, size_t smem, cudaStream_t s) {
   cudaFuncSetAttribute(k_ras_factor_cta<TF, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        (int)cudaSharedmemCarveoutMaxShared);
-  cudaFuncSetAttribute(k_ras_factor_cta<TF, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_ras_factor_cta<TF, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FACTOR_SMEM_MAX);
   k_ras_factor_cta<TF, MODE><<<r.np, 256, smem, s>>>(r, fac, err);
 }
 
@@ -851,13 +853,13 @@ void launch_ras_factor(const RasDev& r, TF* fac, int32_t* err, cudaStream_t s) {
     case 3:
       cudaFuncSetAttribute(k_ras_factor_nd<TF>, cudaFuncAttributePreferredSharedMemoryCarveout,
                            (int)cudaSharedmemCarveoutMaxShared);
-      cudaFuncSetAttribute(k_ras_factor_nd<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_ras_factor_nd<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FACTOR_SMEM_MAX);
       k_ras_factor_nd<TF><<<r.np, 256, smem, s>>>(r, fac, err);
       break;
     case 4:
       cudaFuncSetAttribute(k_ras_factor_pipe<TF>, cudaFuncAttributePreferredSharedMemoryCarveout,
                            (int)cudaSharedmemCarveoutMaxShared);
-      cudaFuncSetAttribute(k_ras_factor_pipe<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_ras_factor_pipe<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FACTOR_SMEM_MAX);
       k_ras_factor_pipe<TF><<<r.np, PIPE_THREADS<TF> + 64, smem, s>>>(r, fac, err);
       break;
     default: break;  // fsi_create rejects such plans
