@@ -525,34 +525,47 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
       inverted = true;
     };
     for (int e = 0; e < nl; ++e) {
-      if (ok) ok = pipe_bar_wait(&full[slot], (uint32_t)phase, tries);
+      // lanes of a warp may give up apart: they must not meet a barrier on different branches of
+      // the block's kind. FP32: the warp votes, so that it takes one; FP64: the barrier is
+      // outside the branches. (The kind from global memory for lanes that gave up, instead: 6-tube
+      // batch refresh 4,394 us where this takes 4,249.)
+      if constexpr (F32) ok = __all_sync(0xffffffffu, ok && pipe_bar_wait(&full[slot], (uint32_t)phase, tries));
+      else if (ok) ok = pipe_bar_wait(&full[slot], (uint32_t)phase, tries);
       const uint32_t* meta = reinterpret_cast<const uint32_t*>(slots + slot * slot_bytes);
-      // (a thread that gave up takes the list's head, and with it the block's branches, from global memory)
-      const uint32_t head = ok ? meta[0] : R.meta[4 * R.meta_off[lp + e]];
+      const uint32_t head = ok ? meta[0] : 0;
       const int ne = (int)(head & 0xffff);
       const uint32_t kind = head >> 28;
       if (kind == PIPE_PREV) wait_inverse();
       // A_ik D_k^{-1}: FP32 in every warp for itself (one barrier per L block), FP64 once
-      auto both = [&](const TF* D) {
+      auto scale = [&](const TF* D) {
         const TF* A = row + 49 * e;
         if constexpr (F32) {
           TF* scl = sScl + 56 * w;
-          if (ok) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int x = lane + 32 * h;
-              if (x < 49) {
-                const int r = h ? r1 : r0, c = h ? c1 : c0;
-                TF v = TF(0);
+          for (int h = 0; h < 2; ++h) {
+            const int x = lane + 32 * h;
+            if (x < 49) {
+              const int r = h ? r1 : r0, c = h ? c1 : c0;
+              TF v = TF(0);
 #pragma unroll
-                for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
-                scl[8 * r + c] = v;
-                if (w == 0) fac[49 * (rp + e) + x] = v;
-              }
+              for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
+              scl[8 * r + c] = v;
+              if (w == 0) fac[49 * (rp + e) + x] = v;
             }
           }
-          __syncwarp();
-          if (ok && tid < 7 * ne) {
+        } else if (tid < 49) {
+          const int r = tid / 7, c = tid - 7 * r;
+          TF v = TF(0);
+#pragma unroll
+          for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
+          sScl[tid] = v;
+          fac[49 * (rp + e) + tid] = v;
+        }
+      };
+      auto update = [&](const TF* D) {
+        if constexpr (F32) {
+          if (tid < 7 * ne) {
+            const TF* scl = sScl + 56 * w;
             float4 sv[14];  // the scaled block, rows of 8
 #pragma unroll
             for (int i = 0; i < 14; ++i) sv[i] = *reinterpret_cast<const float4*>(scl + 4 * i);
@@ -574,35 +587,45 @@ __global__ void __launch_bounds__(PIPE_THREADS<TF> + 64, sizeof(TF) == 4 ? 1 : 2
             }
           }
         } else {
-          if (ok && tid < 49) {
-            const int r = tid / 7, c = tid - 7 * r;
-            TF v = TF(0);
+          for (int x = tid; x < 49 * ne; x += NT) {
+            const int u = x / 49, el = x - 49 * u;
+            const int r = el / 7, c = el - 7 * r;
+            const uint32_t ts = meta[2 + u];
+            TF* T = row + 49 * (ts >> 16) + el;
+            const TF* S = D + 49 * (ts & 0xffff) + c;
+            TF acc = *T;
 #pragma unroll
-            for (int mm = 0; mm < 7; ++mm) v += A[7 * r + mm] * D[7 * mm + c];
-            sScl[tid] = v;
-            fac[49 * (rp + e) + tid] = v;
+            for (int mm = 0; mm < 7; ++mm) acc -= sScl[7 * r + mm] * S[7 * mm];
+            *T = acc;
           }
-          bar();
-          if (ok)
-            for (int x = tid; x < 49 * ne; x += NT) {
-              const int u = x / 49, el = x - 49 * u;
-              const int r = el / 7, c = el - 7 * r;
-              const uint32_t ts = meta[2 + u];
-              TF* T = row + 49 * (ts >> 16) + el;
-              const TF* S = D + 49 * (ts & 0xffff) + c;
-              TF acc = *T;
-#pragma unroll
-              for (int mm = 0; mm < 7; ++mm) acc -= sScl[7 * r + mm] * S[7 * mm];
-              *T = acc;
-            }
         }
       };
-      if (kind == PIPE_DIRECT)
-        both(fac + 49 * R.lent_kdiag[lp + e]);
-      else
-        both(kind == PIPE_PREV ? prow
-                               : reinterpret_cast<const TF*>(slots + slot * slot_bytes + R.pipe_meta) +
-                                     ((head >> 16) & 15));
+      const TF* Ds = kind == PIPE_PREV ? prow
+                                       : reinterpret_cast<const TF*>(slots + slot * slot_bytes + R.pipe_meta) +
+                                             ((head >> 16) & 15);
+      if constexpr (F32) {
+        auto both = [&](const TF* D) {
+          if (ok) scale(D);
+          __syncwarp();
+          if (ok) update(D);
+        };
+        if (kind == PIPE_DIRECT) both(fac + 49 * R.lent_kdiag[lp + e]);
+        else both(Ds);
+      } else {
+        const TF* Dg = fac;
+        if (kind == PIPE_DIRECT) {
+          Dg = fac + 49 * R.lent_kdiag[lp + e];
+          if (ok) scale(Dg);
+        } else if (ok) {
+          scale(Ds);
+        }
+        bar();
+        if (kind == PIPE_DIRECT) {
+          if (ok) update(Dg);
+        } else if (ok) {
+          update(Ds);
+        }
+      }
       bar();
       // (a slot that was not waited for is not given back: a copy may still be on its way into it)
       if (tid == 0 && ok) pipe_bar_arrive(&empty[slot]);
