@@ -147,7 +147,7 @@ typedef struct {
                              none: its bounded waits run out and the call that builds
                              the factors returns FSI_ERR_TIMEOUT; 5 = the streamed
                              apply's first wait gives up at once, with its copies on
-                             their way, 6 = it does so on one lane of each warp
+                             their way, 6 = a wait does so on one lane of each warp
                              (where several warps take a subdomain; both
                              FSI_ERR_TIMEOUT, too); 0 otherwise */
   int32_t apply_mode;     /* preconditioner apply kernel: 0 automatic (the streamed

@@ -147,8 +147,8 @@ struct RasStreamDev {
   int64_t max_rows;       // rows of the largest subdomain
   int32_t nst;            // ring stages in flight per warp (2..8)
   int32_t stall;          // tests only: 1 the producer issues nothing (bounded waits run out), 2 the
-                          // first wait gives up at once, 3 it does on one lane of each warp (team and
-                          // ring kernels)
+                          // first wait gives up at once, 3 a wait gives up on one lane of each warp
+                          // (ring: the first; team kernels: the last)
   // nested-dissection items (one item per subdomain for the other orderings)
   const int32_t* sd_depth;  // [np] depth D: 2^(D+1) - 1 items, solved by 2^D warps
   const int64_t* sd_item;   // [np+1] first item of each subdomain

@@ -485,18 +485,18 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
 
   int slot = 0, phase = 0;  // stage being worked off and its barrier's phase
   const unsigned char* at = ring + 16 * c + (lane >> 3) * BLK;  // this lane's row of the next entry's first group
-  bool ok = true;
+  bool ok = R.stall != 2;
+  if (!ok) left = 0;
   int fslot = 0, fphase = 0;  // the stage given up on
   // once a wait gives up no stage is asked for any more: a barrier is not armed again
   // while a copy may still be on its way to its slot
-  auto give_up = [&]() {
-    ok = false;
-    left = 0;
-    fslot = slot;
-    fphase = phase;
-  };
   auto wait = [&]() {
-    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
+      ok = false;
+      left = 0;
+      fslot = slot;
+      fphase = phase;
+    }
   };
   // rows of an entry's blocks into registers; what lies behind its blocks is read too and not used
   auto fetch = [&](TF (&A)[G][8], uint32_t code) {
@@ -577,7 +577,6 @@ __global__ void __launch_bounds__(32) k_ras_apply_chain(RasStreamDev R, const do
       if (ncode < ENTRY_NONE) fetch(N, ncode);
     }
   };
-  if (R.stall == 2) give_up();
   wait();
   if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
   // a lane whose wait gave up goes on to the end with the others (the data do not decide any address)
@@ -678,7 +677,8 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
 
   int slot = 0, phase = 0, par = 0;
   const unsigned char* at = ring + 16 * c + b * BLK;
-  bool ok = true;
+  bool ok = R.stall != 2;
+  if (!ok) left = 0;
   auto fetch = [&](float (&A)[8], uint32_t code) {
     const int nb = (int)(code & 15) + 1;
     load16(&A[0], reinterpret_cast<const float*>(at));
@@ -693,14 +693,13 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
   for (int e = 0; e < 8; ++e) A0[e] = A1[e] = float(0);
   const int cc = c < 7 ? c : 6;
   int fslot = 0, fphase = 0;
-  auto give_up = [&]() {
-    ok = false;
-    left = 0;
-    fslot = slot;
-    fphase = phase;
-  };
   auto wait = [&]() {
-    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
+      ok = false;
+      left = 0;
+      fslot = slot;
+      fphase = phase;
+    }
   };
   auto step = [&](float (&A)[8], float (&N)[8], uint32_t code, uint32_t ncode) {
     if (code < ENTRY_NONE) {
@@ -752,7 +751,6 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       if (ncode < ENTRY_NONE) fetch(N, ncode);
     }
   };
-  if (R.stall == 2 || (R.stall == 3 && lane == 1)) give_up();
   wait();
   if ((win & 255) < ENTRY_NONE) fetch(A0, (uint32_t)win & 255);
   // a warp whose wait gave up goes on to the end (the data do not decide any address or barrier)
@@ -766,7 +764,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team(RasStreamDev R, const do
       ahead = cw[min((it >> 1) + 3, nw + 1)];
     }
   }
-  if (!ok) {
+  if (!ok || (R.stall == 3 && lane == 1)) {
     // record it; the thread that asked for the copies lets those that may still be in
     // flight land (bounded; it has waited for all of them if it has not given up itself)
     atomicExch(err, 2);
@@ -851,16 +849,16 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
   __syncthreads();
 
   int slot = 0, phase = 0, par = 0, t = 0, fslot = 0, fphase = 0;
-  bool ok = true;
+  bool ok = R.stall != 2;
+  if (!ok) left = 0;
   const unsigned char* at = ring;  // blocks of the next entry to fetch (warp 0: of the current one)
-  auto give_up = [&]() {
-    ok = false;
-    left = 0;
-    fslot = slot;
-    fphase = phase;
-  };
   auto wait = [&]() {
-    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) give_up();
+    if (ok && !mbar_wait(&full[slot], (uint32_t)phase)) {
+      ok = false;
+      left = 0;
+      fslot = slot;
+      fphase = phase;
+    }
   };
   auto next_stage = [&]() {
     feed(slot);
@@ -870,7 +868,6 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
     wait();
   };
   auto size = [](uint32_t code) { return ((code & 15) + ((code & ENTRY_NEAR) ? 1 : 0)) * BLK; };
-  if (R.stall == 2 || (R.stall == 3 && lane == 1)) give_up();
   wait();
 
   if (v == 0) {
@@ -962,7 +959,7 @@ __global__ void __launch_bounds__(128) k_ras_apply_team64(RasStreamDev R, const 
       }
     }
   }
-  if (!ok) {
+  if (!ok || (R.stall == 3 && lane == 1)) {
     atomicExch(err, 2);
     if (threadIdx.x == 0) {
       mbar_wait(&full[fslot], (uint32_t)fphase);
